@@ -818,30 +818,40 @@ __global__ void __launch_bounds__(256) energy_finalize(const double *__restrict_
     if (threadIdx.x == 0) *out = 0.5 * red[0];
 }
 
-// FP16 field storage: natural-extent FP32 array (e0 x e1 x e2, x fastest) in,
-// padded stored values (value / scale, rounded to nearest) out, and back.
-__global__ void put_field_h(const float *__restrict__ src, int e0, int e1, int e2, __half *__restrict__ dst,
-                            long long sy, long long sz, float inv_scale)
+// One component between its dense array (natural extents e0 x e1 x e2, x
+// fastest) and the padded layout (row pitch sy, plane pitch sz), converting
+// between the stored type and the caller's: out = in * scale (FP16 storage;
+// scale is 1 and left out otherwise).  TO_PADDED: dense in, padded out.
+//
+// Bound by memory.  One warp takes a row: the row's place is decoded once
+// (one division per row, not per element), and the lanes walk it in 128-byte
+// segments, four loads in flight each.  Dense rows start at any element, so
+// the accesses stay one element wide; 32 lanes still cover whole sectors.
+// 5.2 TB/s out of a 512^3 FP32 grid (205 us per component; the pitched copy
+// call took 617 us, 1.74 TB/s; the FP16 form with a division per element 815).
+template <bool TO_PADDED, typename In, typename Out>
+__global__ void __launch_bounds__(256) move_field(const In *__restrict__ src, Out *__restrict__ dst, int e0, int e1,
+                                                  long long rows, long long sy, long long sz, float scale)
 {
-    const long long total = (long long)e0 * e1 * e2;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(q % e0);
-        const int j = (int)((q / e0) % e1);
-        const int k = (int)(q / ((long long)e0 * e1));
-        dst[(long long)k * sz + (long long)j * sy + i] = __float2half_rn(src[q] * inv_scale);
-    }
-}
-__global__ void get_field_h(const __half *__restrict__ src, int e0, int e1, int e2, long long sy, long long sz,
-                            float scale, float *__restrict__ dst)
-{
-    const long long total = (long long)e0 * e1 * e2;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(q % e0);
-        const int j = (int)((q / e0) % e1);
-        const int k = (int)(q / ((long long)e0 * e1));
-        dst[q] = __half2float(src[(long long)k * sz + (long long)j * sy + i]) * scale;
+    const int lane = threadIdx.x & 31;
+    for (long long r = blockIdx.x * 8ll + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8ll) {
+        const long long k = r / e1, j = r - k * e1;
+        const long long dense = r * e0, padded = k * sz + j * sy;
+        const In *s = src + (TO_PADDED ? dense : padded);
+        Out *d = dst + (TO_PADDED ? padded : dense);
+        for (int i0 = lane; i0 < e0; i0 += 128) {
+            In v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i0 + 32 * u < e0) v[u] = s[i0 + 32 * u];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i0 + 32 * u < e0) {
+                    if constexpr (std::is_same<In, Out>::value) d[i0 + 32 * u] = v[u];
+                    else if constexpr (TO_PADDED) d[i0 + 32 * u] = __float2half_rn(v[u] * scale);
+                    else d[i0 + 32 * u] = __half2float(v[u]) * scale;
+                }
+        }
     }
 }
 

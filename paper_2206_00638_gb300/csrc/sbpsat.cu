@@ -1363,39 +1363,55 @@ int batch_sample_energy(sbp_batch *b, sbp_batch::Member &m)
 
 }  // namespace
 
-namespace sbp {
+namespace {
 
-// A dense (e0, e1, e2) field into the padded layout (row pitch sy, plane pitch
-// sz) and back: host copies go through a contiguous staging array, so the DMA
-// moves one block instead of e1 * e2 short rows.
-template <typename T>
-__global__ void put_field(const T *__restrict__ src, int e0, int e1, int e2, T *__restrict__ dst, long long sy,
-                          long long sz)
+// One component between a dense device array and the padded array of the
+// current set, on the simulation's stream.
+template <bool TO_PADDED, typename In, typename Out>
+int launch_move(const sbp_sim *s, const int e[3], const void *src, void *dst, double scale)
 {
-    const long long total = (long long)e0 * e1 * e2;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(q % e0);
-        const int j = (int)((q / e0) % e1);
-        const int k = (int)(q / ((long long)e0 * e1));
-        dst[(long long)k * sz + (long long)j * sy + i] = src[q];
-    }
-}
-template <typename T>
-__global__ void get_field(const T *__restrict__ src, int e0, int e1, int e2, long long sy, long long sz,
-                          T *__restrict__ dst)
-{
-    const long long total = (long long)e0 * e1 * e2;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(q % e0);
-        const int j = (int)((q / e0) % e1);
-        const int k = (int)(q / ((long long)e0 * e1));
-        dst[q] = src[(long long)k * sz + (long long)j * sy + i];
-    }
+    const long long rows = (long long)e[1] * e[2];
+    const unsigned ctas = (unsigned)std::min<long long>((rows + 7) / 8, 1 << 20);
+    sbp::move_field<TO_PADDED, In, Out><<<ctas, 256, 0, s->stream>>>(
+        static_cast<const In *>(src), static_cast<Out *>(dst), e[0], e[1], rows, s->sy, s->sz, (float)scale);
+    SBP_CUDA(cudaGetLastError());
+    return SBP_OK;
 }
 
-}  // namespace sbp
+int put_dense(const sbp_sim *s, int comp, const int e[3], const void *dense)
+{
+    void *f = s->set[s->cur][comp];
+    if (s->prec == SBP_FP32_FP16STORE)
+        return launch_move<true, float, __half>(s, e, dense, f, 1.0 / s->fscale[comp >= 3]);
+    if (s->prec == SBP_FP64) return launch_move<true, double, double>(s, e, dense, f, 1.0);
+    return launch_move<true, float, float>(s, e, dense, f, 1.0);
+}
+
+int get_dense(const sbp_sim *s, int comp, const int e[3], void *dense)
+{
+    const void *f = s->set[s->cur][comp];
+    if (s->prec == SBP_FP32_FP16STORE)
+        return launch_move<false, __half, float>(s, e, f, dense, s->fscale[comp >= 3]);
+    if (s->prec == SBP_FP64) return launch_move<false, double, double>(s, e, f, dense, 1.0);
+    return launch_move<false, float, float>(s, e, f, dense, 1.0);
+}
+
+// True when a kernel on the simulation's device can address the caller's
+// array: device or managed memory there, aligned to its elements.  Anything
+// else a copy call takes (another device's memory, pinned host memory) keeps
+// going through the copy engine.
+bool kernel_reachable(const sbp_sim *s, const void *ptr)
+{
+    if (reinterpret_cast<uintptr_t>(ptr) % s->psize) return false;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == s->device;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -1475,9 +1491,8 @@ int sbp_set_field(sbp_sim *s, int comp, const void *src, int is_device)
             SBP_CUDA(cudaMemcpyAsync(tmp, src, bytes, cudaMemcpyHostToDevice, s->stream));
             d_src = tmp;
         }
-        sbp::put_field_h<<<1024, 256, 0, s->stream>>>(d_src, e[0], e[1], e[2], static_cast<__half *>(s->set[s->cur][comp]),
-                                                       s->sy, s->sz, (float)(1.0 / s->fscale[comp >= 3]));
-        SBP_CUDA(cudaGetLastError());
+        const int rc = put_dense(s, comp, e, d_src);
+        if (rc) return rc;
         if (tmp) SBP_CUDA(cudaFreeAsync(tmp, s->stream));
         if (!is_device) SBP_CUDA(cudaStreamSynchronize(s->stream));
         return SBP_OK;
@@ -1489,16 +1504,12 @@ int sbp_set_field(sbp_sim *s, int comp, const void *src, int is_device)
         const size_t bytes = (size_t)e[0] * e[1] * e[2] * s->esize;
         void *stage = s->set[s->cur ^ 1][comp];
         SBP_CUDA(cudaMemcpyAsync(stage, src, bytes, cudaMemcpyHostToDevice, s->stream));
-        if (s->esize == 8)
-            sbp::put_field<double><<<1024, 256, 0, s->stream>>>(static_cast<const double *>(stage), e[0], e[1], e[2],
-                                                               static_cast<double *>(s->set[s->cur][comp]), s->sy, s->sz);
-        else
-            sbp::put_field<float><<<1024, 256, 0, s->stream>>>(static_cast<const float *>(stage), e[0], e[1], e[2],
-                                                              static_cast<float *>(s->set[s->cur][comp]), s->sy, s->sz);
-        SBP_CUDA(cudaGetLastError());
+        const int rc = put_dense(s, comp, e, stage);
+        if (rc) return rc;
         SBP_CUDA(cudaStreamSynchronize(s->stream));
         return SBP_OK;
     }
+    if (is_device && kernel_reachable(s, src)) return put_dense(s, comp, e, src);
     cudaMemcpy3DParms m = {};
     m.srcPtr = make_cudaPitchedPtr(const_cast<void *>(src), e[0] * s->esize, e[0] * s->esize, e[1]);
     m.dstPtr = make_cudaPitchedPtr(s->set[s->cur][comp], s->sy * s->esize, e[0] * s->esize, s->n[1] + 2);
@@ -1519,9 +1530,8 @@ int sbp_get_field(sbp_sim *s, int comp, void *dst, int to_device)
         const size_t bytes = (size_t)e[0] * e[1] * e[2] * sizeof(float);
         float *d_dst = static_cast<float *>(dst);
         if (!to_device) SBP_CUDA(cudaMallocAsync(reinterpret_cast<void **>(&d_dst), bytes, s->stream));
-        sbp::get_field_h<<<1024, 256, 0, s->stream>>>(static_cast<const __half *>(s->set[s->cur][comp]), e[0], e[1], e[2],
-                                                       s->sy, s->sz, (float)s->fscale[comp >= 3], d_dst);
-        SBP_CUDA(cudaGetLastError());
+        const int rc = get_dense(s, comp, e, d_dst);
+        if (rc) return rc;
         if (!to_device) {
             SBP_CUDA(cudaMemcpyAsync(dst, d_dst, bytes, cudaMemcpyDeviceToHost, s->stream));
             SBP_CUDA(cudaFreeAsync(d_dst, s->stream));
@@ -1535,17 +1545,13 @@ int sbp_get_field(sbp_sim *s, int comp, void *dst, int to_device)
         // contiguous copy to the host
         const size_t bytes = (size_t)e[0] * e[1] * e[2] * s->esize;
         void *stage = s->set[s->cur ^ 1][comp];
-        if (s->esize == 8)
-            sbp::get_field<double><<<1024, 256, 0, s->stream>>>(static_cast<const double *>(s->set[s->cur][comp]), e[0],
-                                                               e[1], e[2], s->sy, s->sz, static_cast<double *>(stage));
-        else
-            sbp::get_field<float><<<1024, 256, 0, s->stream>>>(static_cast<const float *>(s->set[s->cur][comp]), e[0],
-                                                              e[1], e[2], s->sy, s->sz, static_cast<float *>(stage));
-        SBP_CUDA(cudaGetLastError());
+        const int rc = get_dense(s, comp, e, stage);
+        if (rc) return rc;
         SBP_CUDA(cudaMemcpyAsync(dst, stage, bytes, cudaMemcpyDeviceToHost, s->stream));
         SBP_CUDA(cudaStreamSynchronize(s->stream));
         return check_error_flag(s);
     }
+    if (to_device && kernel_reachable(s, dst)) return get_dense(s, comp, e, dst);
     cudaMemcpy3DParms m = {};
     m.srcPtr = make_cudaPitchedPtr(s->set[s->cur][comp], s->sy * s->esize, e[0] * s->esize, s->n[1] + 2);
     m.dstPtr = make_cudaPitchedPtr(dst, e[0] * s->esize, e[0] * s->esize, e[1]);

@@ -458,49 +458,57 @@ struct Band {
     unsigned ctas;            // CTAs of 256 threads over all warps
 };
 
-// Node of `lane` in band warp w, the warp's index box [il,ih] x [jl,jh] x {k}
-// and its closure axes G (bit a).  False when the lane has no node.
-__device__ __forceinline__ bool band_lane(const Band &b, const int n[3], unsigned w, int lane, int &i, int &j, int &k,
-                                          int &il, int &ih, int &jl, int &jh, int &G)
+// A warp's share of a band: the node of this lane (valid: there is one), the
+// warp's index box [il,ih] x [jl,jh] x {k} and its closure axes G (bit a).
+struct BandNode {
+    int i, j, k, il, ih, jl, jh, G;
+    bool valid;
+};
+
+// Node of `lane` in band warp w.
+__device__ __forceinline__ BandNode band_lane(const Band &b, const int n[3], unsigned w, int lane)
 {
+    BandNode r;
     const int lo = b.lo;
     if (w < b.wz + b.wy) {
         const bool zs = w < b.wz;
         if (!zs) w -= b.wz;
-        const unsigned r = w / b.segs;
-        const unsigned seg = w - r * b.segs;
+        const unsigned row = w / b.segs;
+        const unsigned seg = w - row * b.segs;
         if (zs) {
-            const unsigned pl = r / b.jin;
-            j = lo + (int)(r - pl * b.jin);
-            k = (int)pl < lo ? (int)pl : b.hi[2] + 1 + ((int)pl - lo);
-            G = 4;
+            const unsigned pl = row / b.jin;
+            r.j = lo + (int)(row - pl * b.jin);
+            r.k = (int)pl < lo ? (int)pl : b.hi[2] + 1 + ((int)pl - lo);
+            r.G = 4;
         } else {
-            const unsigned kk = r / b.yrows;
-            const int jr = (int)(r - kk * b.yrows);
-            k = (int)kk;
-            j = jr < lo ? jr : b.hi[1] + 1 + (jr - lo);
-            G = (k < lo || k > b.hi[2]) ? 6 : 2;
+            const unsigned kk = row / b.yrows;
+            const int jr = (int)(row - kk * b.yrows);
+            r.k = (int)kk;
+            r.j = jr < lo ? jr : b.hi[1] + 1 + (jr - lo);
+            r.G = (r.k < lo || r.k > b.hi[2]) ? 6 : 2;
         }
-        jl = jh = j;
-        il = (int)seg * 32;
-        ih = il + 31;
-        i = il + lane;
-        return i >= lo && i <= b.hi[0];
+        r.jl = r.jh = r.j;
+        r.il = (int)seg * 32;
+        r.ih = r.il + 31;
+        r.i = r.il + lane;
+        r.valid = r.i >= lo && r.i <= b.hi[0];
+        return r;
     }
     w -= b.wz + b.wy;
-    const unsigned side = w & 1u, r = w >> 1;
-    const unsigned kk = r / b.xgroups;
-    const int g = (int)(r - kk * b.xgroups);
-    k = (int)kk;
-    jl = 8 * g;
-    jh = min(jl + 7, n[1] + 1);
-    j = jl + (lane >> 2);
+    const unsigned side = w & 1u, row = w >> 1;
+    const unsigned kk = row / b.xgroups;
+    const int g = (int)(row - kk * b.xgroups);
+    r.k = (int)kk;
+    r.jl = 8 * g;
+    r.jh = min(r.jl + 7, n[1] + 1);
+    r.j = r.jl + (lane >> 2);
     const int c = lane & 3;
-    il = side ? b.hi[0] + 1 : 0;
-    ih = il + 3;
-    i = il + c;
-    G = 1 | ((jl < lo || jh > b.hi[1]) ? 2 : 0) | ((k < lo || k > b.hi[2]) ? 4 : 0);
-    return j <= jh && (side ? i <= n[0] + 1 : c < lo);
+    r.il = side ? b.hi[0] + 1 : 0;
+    r.ih = r.il + 3;
+    r.i = r.il + c;
+    r.G = 1 | ((r.jl < lo || r.jh > b.hi[1]) ? 2 : 0) | ((r.k < lo || r.k > b.hi[2]) ? 4 : 0);
+    r.valid = r.j <= r.jh && (side ? r.i <= n[0] + 1 : c < lo);
+    return r;
 }
 
 // Probes of components [c0, c0+2] inside the warp's box (one bit per probe).
@@ -591,7 +599,7 @@ __device__ __forceinline__ void yee_h(const Params<T, S> &p, const int idx[3], l
 
 template <typename T, bool MUVAR, int C, typename S>
 __device__ __forceinline__ void yee_e(const Params<T, S> &p, const int idx[3], long long o, bool have, unsigned sm,
-                                      double t_half, S *out, T &en)
+                                      const double *J, S *out, T &en)
 {
     if (!have) return;
     const T eold = ld_s(p.F[C] + o);
@@ -599,36 +607,37 @@ __device__ __forceinline__ void yee_e(const Params<T, S> &p, const int idx[3], l
         Tri<T> v[2];
         e_gather<T, C, false, 0>(p, idx, o, v);
         const T se = cell_sum<C, T>(p.eps, o, p.sy, p.sz);
-        en = quant<S>(e_apply<T, C, MUVAR, false, 0>(p, idx, o, eold, se, v, sm, t_half));
+        en = quant<S>(e_apply<T, C, MUVAR, false, 0>(p, idx, o, eold, se, v, sm, J));
     } else {
         en = eold;
     }
     st_s(out + o, en);
 }
 
-// H^{n+1/2} at the nodes of band warp w: p.F = {E^n (old), H^{n-1/2} (old)}, outs = new H.
+// H^{n+1/2} at a warp's band nodes: p.F = {E^n (old), H^{n-1/2} (old)}, outs = new H.
 // CG: field reads through L2 only (the persistent batched kernel, whose other
-// CTAs wrote them earlier in the same launch).
-template <typename T, bool MUVAR, bool CG = false, typename S>
-__device__ __forceinline__ void band_h_warp(const Params<T, S> &p, const Band &b, unsigned w, int lane, long long pslot,
+// CTAs wrote them earlier in the same launch).  YEE: the simulation may be the
+// Yee comparator.
+template <typename T, bool MUVAR, bool CG, bool YEE, typename S>
+__device__ __forceinline__ void band_h_node(const Params<T, S> &p, const BandNode &b, int lane, long long pslot,
                                             S *const outs[3])
 {
-    int i, j, k, il, ih, jl, jh, G;
-    const bool valid = band_lane(b, p.n, w, lane, i, j, k, il, ih, jl, jh, G);
-    const unsigned long long pm = p.nprb ? warp_probe_mask(p.prb, p.nprb, 3, k, il, ih, jl, jh, lane) : 0ull;
-    if (!valid) return;
+    const int i = b.i, j = b.j, k = b.k;
+    const unsigned long long pm =
+        p.nprb ? warp_probe_mask(p.prb, p.nprb, 3, k, b.il, b.ih, b.jl, b.jh, lane) : 0ull;
+    if (!b.valid) return;
     const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
     const int idx[3] = {i, j, k};
     const long long o = (long long)k * p.sz + (long long)j * p.sy + i;
     T hn[3];
     const bool have[3] = {i <= nx && j <= ny + 1 && k <= nz + 1, i <= nx + 1 && j <= ny && k <= nz + 1,
                           i <= nx + 1 && j <= ny + 1 && k <= nz};
-    if (p.fdtd) {
+    if (YEE && p.fdtd) {
         yee_h<T, MUVAR, 3>(p, idx, o, have[0], outs[0], hn[0]);
         yee_h<T, MUVAR, 4>(p, idx, o, have[1], outs[1], hn[1]);
         yee_h<T, MUVAR, 5>(p, idx, o, have[2], outs[2], hn[2]);
     } else {
-        switch (G) {   // uniform per warp
+        switch (b.G) {   // uniform per warp
         case 4: band_h_at<T, MUVAR, 4, CG>(p, idx, o, have, outs, hn); break;
         case 2: band_h_at<T, MUVAR, 2, CG>(p, idx, o, have, outs, hn); break;
         case 6: band_h_at<T, MUVAR, 6, CG>(p, idx, o, have, outs, hn); break;
@@ -637,6 +646,12 @@ __device__ __forceinline__ void band_h_warp(const Params<T, S> &p, const Band &b
         }
     }
     if (pm) band_probes(p, pm, 3, i, j, pslot, hn, have);
+}
+template <typename T, bool MUVAR, bool CG = false, typename S>
+__device__ __forceinline__ void band_h_warp(const Params<T, S> &p, const Band &b, unsigned w, int lane, long long pslot,
+                                            S *const outs[3])
+{
+    band_h_node<T, MUVAR, CG, true>(p, band_lane(b, p.n, w, lane), lane, pslot, outs);
 }
 
 // At most 56 registers: two 256-thread CTAs then fit on an SM beside a 512-thread
@@ -653,7 +668,7 @@ __global__ void __maxnreg__(56) band_h(const Params<T, S> p, const Band b, S *hx
 // E^{n+1} at one band node, closure axes G (see band_h_at).
 template <typename T, bool MUVAR, int G, bool CG, typename S>
 __device__ __forceinline__ void band_e_at(const Params<T, S> &p, const int idx[3], long long o, const bool have[3],
-                                          unsigned sm, double t_half, S *const outs[3], T en[3])
+                                          unsigned sm, const double *J, S *const outs[3], T en[3])
 {
     Tri<T> vx[2], vy[2], vz[2];
     e_gather<T, 0, CG, G>(p, idx, o, vx);
@@ -663,57 +678,53 @@ __device__ __forceinline__ void band_e_at(const Params<T, S> &p, const int idx[3
     const T sx = cell_sum<0, T>(p.eps, o, p.sy, p.sz);
     const T sy = cell_sum<1, T>(p.eps, o, p.sy, p.sz);
     const T sz = cell_sum<2, T>(p.eps, o, p.sy, p.sz);
-    if (have[0]) st_s(outs[0] + o, en[0] = quant<S>(e_apply<T, 0, MUVAR, false, G>(p, idx, o, ex, sx, vx, sm, t_half)));
-    if (have[1]) st_s(outs[1] + o, en[1] = quant<S>(e_apply<T, 1, MUVAR, false, G>(p, idx, o, ey, sy, vy, sm, t_half)));
-    if (have[2]) st_s(outs[2] + o, en[2] = quant<S>(e_apply<T, 2, MUVAR, false, G>(p, idx, o, ez, sz, vz, sm, t_half)));
+    if (have[0]) st_s(outs[0] + o, en[0] = quant<S>(e_apply<T, 0, MUVAR, false, G>(p, idx, o, ex, sx, vx, sm, J)));
+    if (have[1]) st_s(outs[1] + o, en[1] = quant<S>(e_apply<T, 1, MUVAR, false, G>(p, idx, o, ey, sy, vy, sm, J)));
+    if (have[2]) st_s(outs[2] + o, en[2] = quant<S>(e_apply<T, 2, MUVAR, false, G>(p, idx, o, ez, sz, vz, sm, J)));
 }
 
-// E^{n+1} at the nodes of band warp w: p.F = {E^n (old), H^{n+1/2} (new)}, outs = new E.
+// E^{n+1} at a warp's band nodes: p.F = {E^n (old), H^{n+1/2} (new)}, outs = new E.
+template <typename T, bool MUVAR, bool CG, bool YEE, typename S>
+__device__ __forceinline__ void band_e_node(const Params<T, S> &p, const BandNode &b, int lane, long long step,
+                                            long long pslot, S *const outs[3])
+{
+    const int i = b.i, j = b.j, k = b.k;
+    const unsigned long long pm =
+        p.nprb ? warp_probe_mask(p.prb, p.nprb, 0, k, b.il, b.ih, b.jl, b.jh, lane) : 0ull;
+    const double *const J = source_values(p, step, lane, k, k, b.jl, b.jh, b.il, b.ih);
+    if (!b.valid) return;
+    unsigned sm = 0u;
+    if (J)
+        for (int q = 0; q < p.nsrc; ++q)
+            if ((p.src[q].i < 0 || p.src[q].i == i) && (p.src[q].j < 0 || p.src[q].j == j) &&
+                (p.src[q].k < 0 || p.src[q].k == k))
+                sm |= 1u << q;
+    const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
+    const int idx[3] = {i, j, k};
+    const long long o = (long long)k * p.sz + (long long)j * p.sy + i;
+    T en[3];
+    const bool have[3] = {i <= nx + 1 && j <= ny && k <= nz, i <= nx && j <= ny + 1 && k <= nz,
+                          i <= nx && j <= ny && k <= nz + 1};
+    if (YEE && p.fdtd) {
+        yee_e<T, MUVAR, 0>(p, idx, o, have[0], sm, J, outs[0], en[0]);
+        yee_e<T, MUVAR, 1>(p, idx, o, have[1], sm, J, outs[1], en[1]);
+        yee_e<T, MUVAR, 2>(p, idx, o, have[2], sm, J, outs[2], en[2]);
+    } else {
+        switch (b.G) {   // uniform per warp
+        case 4: band_e_at<T, MUVAR, 4, CG>(p, idx, o, have, sm, J, outs, en); break;
+        case 2: band_e_at<T, MUVAR, 2, CG>(p, idx, o, have, sm, J, outs, en); break;
+        case 6: band_e_at<T, MUVAR, 6, CG>(p, idx, o, have, sm, J, outs, en); break;
+        case 1: band_e_at<T, MUVAR, 1, CG>(p, idx, o, have, sm, J, outs, en); break;
+        default: band_e_at<T, MUVAR, 7, CG>(p, idx, o, have, sm, J, outs, en); break;
+        }
+    }
+    if (pm) band_probes(p, pm, 0, i, j, pslot, en, have);
+}
 template <typename T, bool MUVAR, bool CG = false, typename S>
 __device__ __forceinline__ void band_e_warp(const Params<T, S> &p, const Band &b, unsigned w, int lane, long long step,
                                             long long pslot, S *const outs[3])
 {
-    int i, j, k, il, ih, jl, jh, G;
-    const bool valid = band_lane(b, p.n, w, lane, i, j, k, il, ih, jl, jh, G);
-    const unsigned long long pm = p.nprb ? warp_probe_mask(p.prb, p.nprb, 0, k, il, ih, jl, jh, lane) : 0ull;
-    // sources that can reach the warp's box (point, line or sheet), then this node's
-    unsigned wm = 0u;
-    if (p.nsrc) {
-        bool hit = false;
-        if (lane < p.nsrc) {
-            const Src &Sr = p.src[lane];
-            hit = (Sr.i < 0 || (Sr.i >= il && Sr.i <= ih)) && (Sr.j < 0 || (Sr.j >= jl && Sr.j <= jh)) &&
-                  (Sr.k < 0 || Sr.k == k);
-        }
-        wm = __ballot_sync(0xffffffffu, hit);
-    }
-    if (!valid) return;
-    unsigned sm = 0u;
-    for (unsigned m = wm; m; m &= m - 1) {
-        const int q = __ffs(m) - 1;
-        if ((p.src[q].i < 0 || p.src[q].i == i) && (p.src[q].j < 0 || p.src[q].j == j)) sm |= 1u << q;
-    }
-    const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
-    const int idx[3] = {i, j, k};
-    const long long o = (long long)k * p.sz + (long long)j * p.sy + i;
-    const double t_half = ((double)step + 0.5) * p.dt;
-    T en[3];
-    const bool have[3] = {i <= nx + 1 && j <= ny && k <= nz, i <= nx && j <= ny + 1 && k <= nz,
-                          i <= nx && j <= ny && k <= nz + 1};
-    if (p.fdtd) {
-        yee_e<T, MUVAR, 0>(p, idx, o, have[0], sm, t_half, outs[0], en[0]);
-        yee_e<T, MUVAR, 1>(p, idx, o, have[1], sm, t_half, outs[1], en[1]);
-        yee_e<T, MUVAR, 2>(p, idx, o, have[2], sm, t_half, outs[2], en[2]);
-    } else {
-        switch (G) {   // uniform per warp
-        case 4: band_e_at<T, MUVAR, 4, CG>(p, idx, o, have, sm, t_half, outs, en); break;
-        case 2: band_e_at<T, MUVAR, 2, CG>(p, idx, o, have, sm, t_half, outs, en); break;
-        case 6: band_e_at<T, MUVAR, 6, CG>(p, idx, o, have, sm, t_half, outs, en); break;
-        case 1: band_e_at<T, MUVAR, 1, CG>(p, idx, o, have, sm, t_half, outs, en); break;
-        default: band_e_at<T, MUVAR, 7, CG>(p, idx, o, have, sm, t_half, outs, en); break;
-        }
-    }
-    if (pm) band_probes(p, pm, 0, i, j, pslot, en, have);
+    band_e_node<T, MUVAR, CG, true>(p, band_lane(b, p.n, w, lane), lane, step, pslot, outs);
 }
 
 template <typename T, bool MUVAR, typename S>

@@ -1,0 +1,557 @@
+// In-place half-steps (sm_103a): one launch updates every node of H, the next
+// every node of E.
+//
+//   half_h  H^{n+1/2} = H^{n-1/2} + dt/mu (D- E^n) + SAT_H      Eqs. (10)-(15), Alg. 2
+//   half_e  E^{n+1}   = E^n + dt/eps (D+ H^{n+1/2} - J) + SAT_E Eqs. (7)-(9), (19)-(21), Alg. 1
+//
+// The nodes of a block are dealt to two kinds of CTAs of one launch.
+//   - Box CTAs: the nodes whose rows are two-point rows along every axis and
+//     meet no face.  A thread owns V neighbouring x nodes of one row (vector
+//     loads and stores) and marches kz planes, carrying the z-neighbours and the
+//     eps sums of the previous plane in registers.
+//   - Rim CTAs: every node around the box, one per thread, x fastest.  The rows
+//     of all three axes are three entries with coefficients, so one short code
+//     serves faces, edges and corners; it loads everything a node needs before
+//     it computes.  A grid's first wave is over in a few microseconds, and what
+//     counts there is the longest chain of a rim thread: rim code that took
+//     four nodes per thread, or called its penalties one after the other, made
+//     a 61x47x38 half-step 6 us long where the box alone takes 2.
+// Threads are dealt over (row, vector) pairs without gaps, so narrow grids fill
+// their warps.  The rim of a plane is listed next to the box CTAs of the same
+// planes: an end node sits in a DRAM unit that the box part of its row reads as
+// well, and so finds it in L2.
+#pragma once
+#include "fused.cuh"
+
+namespace sbp {
+
+constexpr int kSweepThreads = 128;        // threads of a CTA
+
+// n / d for n < 2^31, with the multiplier of d found on the host.
+struct FastDiv { unsigned mul, shift; };
+__device__ __forceinline__ unsigned operator/(unsigned n, const FastDiv &d) { return (__umulhi(n, d.mul) + n) >> d.shift; }
+
+// Work list of one in-place half-step launch.
+struct Sweep {
+    int lo[3], hi[3];         // the box, inclusive per axis; empty along an axis when hi < lo
+    int kz;                   // planes per z-chunk
+    unsigned nv, vecs;        // vectors per row and per plane of the box
+    unsigned xs, rows;        // nodes per row and rows of a whole plane
+    unsigned ends;            // nodes of a row left and right of the box
+    unsigned zplanes;         // planes below and above the box
+    unsigned ynodes, rim;     // rim nodes of a box plane: y layers, in all
+    unsigned cz;              // CTAs of the planes below and above the box (first in the list)
+    unsigned cbox, cchunk;    // box CTAs and all CTAs of a z-chunk
+    unsigned ctas;
+    FastDiv dnv, dxs, drows, dends, drim, dchunk;
+};
+
+// --- programmatic dependent launch -----------------------------------------
+// Each half-step lets the next one start as soon as all of its own CTAs run,
+// and waits for the previous one before it touches a field: the launch latency
+// (about a third of a small grid's half-step) overlaps the running kernel.
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// --- vector access ----------------------------------------------------------
+template <int V, typename S>
+__device__ __forceinline__ void ldv(const S *p, compute_t<S> (&v)[V])
+{
+    constexpr int bytes = V * (int)sizeof(S);
+    if constexpr (V == 1) {
+        v[0] = ld_s(p);
+    } else {
+        static_assert(bytes == 8 || bytes == 16, "vector width");
+        using W = typename std::conditional<bytes == 16, uint4, uint2>::type;
+        union { W w; S s[V]; } u;
+        u.w = *reinterpret_cast<const W *>(p);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            if constexpr (std::is_same<S, __half>::value) v[q] = __half2float(u.s[q]);
+            else v[q] = u.s[q];
+        }
+    }
+}
+// Store v (already rounded to the storage type), or its first `count` elements.
+template <int V, typename S, typename T>
+__device__ __forceinline__ void stv(S *p, const T (&v)[V], int count)
+{
+    constexpr int bytes = V * (int)sizeof(S);
+    if constexpr (V > 1) {
+        if (count >= V) {
+            using W = typename std::conditional<bytes == 16, uint4, uint2>::type;
+            union { W w; S s[V]; } u;
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                if constexpr (std::is_same<S, __half>::value) u.s[q] = __float2half_rn(v[q]);
+                else u.s[q] = v[q];
+            }
+            *reinterpret_cast<W *>(p) = u.w;
+            return;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < V; ++q)
+        if (q < count) st_s(p + q, v[q]);
+}
+// Cell values (FP32) in the arithmetic type.
+template <int V, typename T>
+__device__ __forceinline__ void ldcells(const float *p, T (&v)[V])
+{
+    float f[V];
+    if constexpr (V == 4) {
+        const float4 w = __ldg(reinterpret_cast<const float4 *>(p));
+        f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w;
+    } else if constexpr (V == 2) {
+        const float2 w = __ldg(reinterpret_cast<const float2 *>(p));
+        f[0] = w.x; f[1] = w.y;
+    } else {
+        f[0] = __ldg(p);
+    }
+#pragma unroll
+    for (int q = 0; q < V; ++q) v[q] = widen<T>(f[q]);
+}
+
+// old + increment of two curl terms, in the rounding order of the general path
+// (FP64 accumulates into the old value: one operation less).
+template <typename S, typename T>
+__device__ __forceinline__ T advance_plain(T old, const Coef<T> &c0, T d0, const Coef<T> &c1, T d1)
+{
+    if constexpr (std::is_same<T, double>::value) {
+        return fma(-c1.hi, d1, fma(c0.hi, d0, old));
+    } else {
+        typename AccOf<T, S>::type a;
+        a.add(c0, d0);
+        a.add(c1, d1, T(-1));
+        return old + plain_increment(a);
+    }
+}
+
+// Probes of components c0..c0+2 near a warp's rows and planes (bit per probe);
+// every lane of the warp calls it.
+__device__ __forceinline__ unsigned long long rows_probe_mask(const Prb *prb, int nprb, int c0, int k0, int k1, int j0,
+                                                              int j1, int lane)
+{
+    unsigned long long m = 0ull;
+    for (int q0 = 0; q0 < nprb; q0 += 32) {
+        const int q = q0 + lane;
+        bool hit = false;
+        if (q < nprb) {
+            const Prb P = prb[q];
+            hit = P.comp >= c0 && P.comp <= c0 + 2 && P.k >= k0 && P.k <= k1 && P.j >= j0 && P.j <= j1;
+        }
+        m |= (unsigned long long)__ballot_sync(0xffffffffu, hit) << q0;
+    }
+    return m;
+}
+
+template <int V, typename T, typename S>
+__device__ __forceinline__ void vec_probes(const Params<T, S> &p, unsigned long long m, int c0, int i0, int j, int k,
+                                           const T (&a)[V], const T (&b)[V], const T (&c)[V])
+{
+    for (; m; m &= m - 1) {
+        const int q = __ffsll((long long)m) - 1;
+        const Prb &P = p.prb[q];
+        if (P.j != j || P.k != k || p.probe_slot >= p.probe_cap) continue;
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+            if (P.i == i0 + e)
+                p.probe_buf[(long long)q * p.probe_cap + p.probe_slot] =
+                    (P.comp == c0 ? a[e] : P.comp == c0 + 1 ? b[e] : c[e]) * p.fscale[c0 >= 3];
+    }
+}
+
+// First x, row and plane range of a box thread, and the rows of its warp.
+struct VecPlace { int i0, j, jmin, jmax, k0, k1; bool valid; };
+
+template <int V>
+__device__ __forceinline__ VecPlace vec_place(const Sweep &w, unsigned cta, int chunk)
+{
+    VecPlace r;
+    const unsigned t = cta * (unsigned)kSweepThreads + threadIdx.x;
+    r.valid = t < w.vecs;
+    const unsigned tc = min(t, w.vecs - 1u), row = tc / w.dnv;
+    r.j = w.lo[1] + (int)row;
+    r.i0 = w.lo[0] + V * (int)(tc - row * w.nv);
+    r.jmin = __shfl_sync(0xffffffffu, r.j, 0);
+    r.jmax = __shfl_sync(0xffffffffu, r.j, 31);
+    r.k0 = max(chunk * w.kz, w.lo[2]);
+    r.k1 = min(chunk * w.kz + w.kz - 1, w.hi[2]);
+    return r;
+}
+
+template <typename T, typename S, bool MUVAR, int V>
+__device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, unsigned cta, int chunk)
+{
+    const VecPlace r = vec_place<V>(w, cta, chunk);
+    if (r.k0 > r.k1) return;
+    const unsigned long long pm =
+        p.nprb ? rows_probe_mask(p.prb, p.nprb, 3, r.k0, r.k1, r.jmin, r.jmax, threadIdx.x & 31) : 0ull;
+    if (!r.valid) return;
+    const long long sy = p.sy, sz = p.sz;
+    long long o = (long long)r.k0 * sz + (long long)r.j * sy + r.i0;
+    const S *const Ex = p.F[0], *const Ey = p.F[1], *const Ez = p.F[2];
+    S *const Hx = p.F[3], *const Hy = p.F[4], *const Hz = p.F[5];
+    const Coef<T> Bx = p.B[0], By = p.B[1], Bz = p.B[2];
+    pdl_wait();
+    T exm[V], eym[V], m0[V];
+    ldv<V>(Ex + o - sz, exm);
+    ldv<V>(Ey + o - sz, eym);
+    if constexpr (MUVAR) ldcells<V>(p.mu + o, m0);
+    for (int k = r.k0; k <= r.k1; ++k, o += sz) {
+        T ex[V], ey[V], ez[V], exj[V], ezj[V], hx[V], hy[V], hz[V];
+        ldv<V>(Ex + o, ex);
+        ldv<V>(Ey + o, ey);
+        ldv<V>(Ez + o, ez);
+        ldv<V>(Ex + o - sy, exj);
+        ldv<V>(Ez + o - sy, ezj);
+        const T eyl = ld_s(Ey + o - 1), ezl = ld_s(Ez + o - 1);
+        ldv<V>(Hx + o, hx);
+        ldv<V>(Hy + o, hy);
+        ldv<V>(Hz + o, hz);
+        T mj[V], mk[V], mr = T(0);
+        if constexpr (MUVAR) {
+            ldcells<V>(p.mu + o + sy, mj);
+            ldcells<V>(p.mu + o + sz, mk);
+            mr = widen<T>(__ldg(p.mu + o + V));
+        }
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const T eyi = q ? ey[q - 1] : eyl, ezi = q ? ez[q - 1] : ezl;
+            const T d0 = ey[q] - eym[q], d1 = ez[q] - ezj[q];       // Hx: Bz dEy/dz - By dEz/dy
+            const T d2 = ez[q] - ezi, d3 = ex[q] - exm[q];          // Hy: Bx dEz/dx - Bz dEx/dz
+            const T d4 = ex[q] - exj[q], d5 = ey[q] - eyi;          // Hz: By dEx/dy - Bx dEy/dx
+            if constexpr (MUVAR) {
+                const T mi = q + 1 < V ? m0[q + 1 < V ? q + 1 : q] : mr;
+                typename AccOf<T, S>::type a, b, c;
+                a.add(Bz, d0); a.add(By, d1, T(-1));
+                b.add(Bx, d2); b.add(Bz, d3, T(-1));
+                c.add(By, d4); c.add(Bx, d5, T(-1));
+                hx[q] = quant<S>(add_scaled(hx[q], a, m0[q] + mi));
+                hy[q] = quant<S>(add_scaled(hy[q], b, m0[q] + mj[q]));
+                hz[q] = quant<S>(add_scaled(hz[q], c, m0[q] + mk[q]));
+            } else {
+                hx[q] = quant<S>(advance_plain<S>(hx[q], Bz, d0, By, d1));
+                hy[q] = quant<S>(advance_plain<S>(hy[q], Bx, d2, Bz, d3));
+                hz[q] = quant<S>(advance_plain<S>(hz[q], By, d4, Bx, d5));
+            }
+        }
+        stv<V>(Hx + o, hx, V);
+        stv<V>(Hy + o, hy, V);
+        stv<V>(Hz + o, hz, V);
+        if (pm) vec_probes<V>(p, pm, 3, r.i0, r.j, k, hx, hy, hz);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            exm[q] = ex[q];
+            eym[q] = ey[q];
+            if constexpr (MUVAR) m0[q] = mk[q];
+        }
+    }
+}
+
+// Pair sums of the eps cells (j, j+1; i, i+1) of one plane, from which the node
+// sums of cell_sum are built in its association.
+template <int V, typename T>
+__device__ __forceinline__ void eps_pairs(const float *eps, long long o, long long sy, T (&a)[V], T (&b)[V], T (&c)[V])
+{
+    T f[V], g[V];
+    ldcells<V>(eps + o, f);
+    ldcells<V>(eps + o + sy, g);
+    const T fr = widen<T>(__ldg(eps + o + V)), gr = widen<T>(__ldg(eps + o + sy + V));
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        const int n = q + 1 < V ? q + 1 : q;
+        a[q] = f[q] + g[q];
+        b[q] = f[q] + (q + 1 < V ? f[n] : fr);
+        c[q] = g[q] + (q + 1 < V ? g[n] : gr);
+    }
+}
+
+template <typename T, typename S, int V>
+__device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, unsigned cta, int chunk)
+{
+    const VecPlace r = vec_place<V>(w, cta, chunk);
+    if (r.k0 > r.k1) return;
+    const int lane = threadIdx.x & 31;
+    const unsigned long long pm =
+        p.nprb ? rows_probe_mask(p.prb, p.nprb, 0, r.k0, r.k1, r.jmin, r.jmax, lane) : 0ull;
+    const double *const J = source_values(p, p.step, lane, r.k0, r.k1, r.jmin, r.jmax, 0, INT32_MAX);
+    if (!r.valid) return;
+    const long long sy = p.sy, sz = p.sz;
+    long long o = (long long)r.k0 * sz + (long long)r.j * sy + r.i0;
+    S *const Ex = p.F[0], *const Ey = p.F[1], *const Ez = p.F[2];
+    const S *const Hx = p.F[3], *const Hy = p.F[4], *const Hz = p.F[5];
+    const Coef<T> Ax = p.A[0], Ay = p.A[1], Az = p.A[2];
+    pdl_wait();
+    T qa[V], qb[V], qc[V];
+    eps_pairs<V>(p.eps, o, sy, qa, qb, qc);
+    T hx[V], hy[V];
+    ldv<V>(Hx + o, hx);
+    ldv<V>(Hy + o, hy);
+    for (int k = r.k0; k <= r.k1; ++k, o += sz) {
+        T hxn[V], hyn[V], hz[V], hzj[V], hxj[V], ex[V], ey[V], ez[V], na[V], nb[V], nc[V];
+        ldv<V>(Hx + o + sz, hxn);
+        ldv<V>(Hy + o + sz, hyn);
+        ldv<V>(Hz + o, hz);
+        ldv<V>(Hz + o + sy, hzj);
+        ldv<V>(Hx + o + sy, hxj);
+        const T hyr = ld_s(Hy + o + V), hzr = ld_s(Hz + o + V);
+        ldv<V>(Ex + o, ex);
+        ldv<V>(Ey + o, ey);
+        ldv<V>(Ez + o, ez);
+        eps_pairs<V>(p.eps, o + sz, sy, na, nb, nc);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            const int n = q + 1 < V ? q + 1 : q;
+            const T hyi = q + 1 < V ? hy[n] : hyr, hzi = q + 1 < V ? hz[n] : hzr;
+            typename AccOf<T, S>::type a, b, c;
+            a.add(Ay, hzj[q] - hz[q]); a.add(Az, hyn[q] - hy[q], T(-1));
+            b.add(Az, hxn[q] - hx[q]); b.add(Ax, hzi - hz[q], T(-1));
+            c.add(Ax, hyi - hy[q]);    c.add(Ay, hxj[q] - hx[q], T(-1));
+            if (J) {
+                for (int s = 0; s < p.nsrc; ++s) {
+                    const Src &P = p.src[s];
+                    if ((P.k >= 0 && P.k != k) || (P.j >= 0 && P.j != r.j) || (P.i >= 0 && P.i != r.i0 + q)) continue;
+                    if (P.comp == 0) a.add(p.AJ, T(J[s]), T(-1));
+                    else if (P.comp == 1) b.add(p.AJ, T(J[s]), T(-1));
+                    else c.add(p.AJ, T(J[s]), T(-1));
+                }
+            }
+            ex[q] = quant<S>(add_scaled(ex[q], a, qa[q] + na[q]));
+            ey[q] = quant<S>(add_scaled(ey[q], b, qb[q] + nb[q]));
+            ez[q] = quant<S>(add_scaled(ez[q], c, qb[q] + qc[q]));
+        }
+        stv<V>(Ex + o, ex, V);
+        stv<V>(Ey + o, ey, V);
+        stv<V>(Ez + o, ez, V);
+        if (pm) vec_probes<V>(p, pm, 0, r.i0, r.j, k, ex, ey, ez);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            hx[q] = hxn[q]; hy[q] = hyn[q];
+            qa[q] = na[q]; qb[q] = nb[q]; qc[q] = nc[q];
+        }
+    }
+}
+
+// --- rim CTAs ----------------------------------------------------------------
+// One axis of a rim node: its D row there (offset of the first entry from the
+// node, coefficients) and the face it lies on (side -1 / +1, 0 for none).
+template <typename T> struct RimAxis {
+    long long off, st;
+    T k[3];
+    int side, type;
+};
+
+template <bool ELECTRIC, typename T, typename S>
+__device__ __forceinline__ RimAxis<T> rim_axis(const Params<T, S> &p, int a, int r)
+{
+    const int n = p.n[a], last = n + (ELECTRIC ? 0 : 1);
+    RimAxis<T> x;
+    x.st = a == 0 ? 1 : a == 1 ? p.sy : p.sz;
+    if constexpr (ELECTRIC) dplus_coefs(r, n, x.k);
+    else dminus_coefs(r, n, x.k);
+    x.off = (long long)((ELECTRIC ? dplus_start(r, n) : dminus_start(r, n)) - r) * x.st;
+    x.side = r == 0 ? -1 : r == last ? 1 : 0;
+    x.type = x.side ? p.face[2 * a + (x.side > 0)] : (ELECTRIC ? kPEC : kPMC);   // the type without a penalty
+    return x;
+}
+
+// The row on its entries.  A two-point row gives the same bits either way; FP64,
+// whose pipe is the narrow one, takes the single subtraction.
+template <typename T>
+__device__ __forceinline__ T rim_row(const RimAxis<T> &x, const Tri<T> &v)
+{
+    if constexpr (std::is_same<T, double>::value)
+        if (x.k[2] == T(0)) return v.b - v.a;
+    return row_chain(x.k, v.a, v.b, v.c);
+}
+
+// The partner's value of field u at the face node that node (i, j, k) faces along a.
+template <typename T, typename S, bool ELECTRIC>
+__device__ __noinline__ T rim_partner(const Params<T, S> &p, int f, int u, int i, int j, int k)
+{
+    const Link &L = p.link[f];
+    const int a = f >> 1, nidx = L.side < 0 ? 0 : ELECTRIC ? L.n_norm + 1 : L.n_norm;
+    const long long on = (long long)(a == 0 ? nidx : i) + (long long)(a == 1 ? nidx : j) * L.sy +
+                         (long long)(a == 2 ? nidx : k) * L.sz;
+    return link_value<false, T, S>(L, u, on);
+}
+
+// Absorbing self term along axis a from the sums of the node's cells.  One copy,
+// called: roots and divisions inlined at the six sites of the rim code made its
+// warps wait for instruction fetch (cavity in FP64 21.3 -> 12.4 us per step,
+// 121 x 101 x 88 with mu_r 20.8 -> 18.8, 512^3 in FP16 storage 1114 -> 1064).
+template <typename T, typename S, bool ELECTRIC, bool MUVAR>
+__device__ __noinline__ T rim_gamma(const Params<T, S> &p, int a, T se, T sm)
+{
+    if constexpr (ELECTRIC) {
+        const T mr = MUVAR ? sm * T(0.25) : T(1);
+        return abs_gamma_e(T(p.A[a].hi) * p.uA, se, node_eta(p.eta0, mr, se * T(0.25)));
+    } else {
+        const T er = se * T(0.5), mr = MUVAR ? sm * T(0.5) : T(1);
+        const T ba = (MUVAR ? T(p.B[a].hi) * T(0.5) / mr : T(p.B[a].hi)) * p.uB;
+        return abs_gamma_h(ba, node_eta(p.eta0, mr, er));
+    }
+}
+// New value of component C at a rim node, in the operation order of h_apply /
+// e_apply.  v[t]: the entries of the two curl terms; se: sum of the node's eps
+// cells (4 for E, 2 for H, there only read on an absorbing face).
+template <typename T, int C, bool MUVAR, typename S>
+__device__ __forceinline__ T rim_apply(const Params<T, S> &p, const RimAxis<T> (&ax)[3], const int (&idx)[3], T old,
+                                       const Tri<T> (&v)[2], T se, T sm, const double *J)
+{
+    constexpr bool electric = C < 3;
+    typename AccOf<T, S>::type acc;
+    T gam = T(0);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int u = curl_comp(C, t), a = curl_axis(C, t), sg = curl_sign(t);
+        const Coef<T> &cf = electric ? p.A[a] : p.B[a];
+        acc.add(cf, rim_row(ax[a], v[t]), T(sg));
+        if (ax[a].type == (electric ? kPEC : kPMC)) continue;
+        const T phi = T(-sg * ax[a].side);
+        T pv = ax[a].side < 0 ? v[t].a : v[t].c;
+        if (ax[a].type == kIFACE)
+            pv = pv - rim_partner<T, S, electric>(p, 2 * a + (ax[a].side > 0), u, idx[0], idx[1], idx[2]);
+        acc.add(cf, pv, ax[a].type == (electric ? kPMC : kPEC) ? T(2) * phi : phi);
+        if (ax[a].type == kABS) gam += rim_gamma<T, S, electric, MUVAR>(p, a, se, sm);
+    }
+    if (electric && J) {
+        for (int s = 0; s < p.nsrc; ++s) {
+            const Src &P = p.src[s];
+            if (P.comp == C && (P.i < 0 || P.i == idx[0]) && (P.j < 0 || P.j == idx[1]) && (P.k < 0 || P.k == idx[2]))
+                acc.add(p.AJ, T(J[s]), T(-1));
+        }
+    }
+    const T inc = electric ? scaled_increment(acc, se) : MUVAR ? scaled_increment(acc, sm) : plain_increment(acc);
+    return quant<S>(sat_finish(old, inc, gam));
+}
+
+// The entries of component C's two curl terms (a third entry only on closure rows).
+template <int C, typename T, typename S>
+__device__ __forceinline__ void rim_gather(const Params<T, S> &p, const RimAxis<T> (&ax)[3], long long o, Tri<T> (&v)[2])
+{
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const RimAxis<T> &x = ax[curl_axis(C, t)];
+        const S *const q = p.F[curl_comp(C, t)] + (o + x.off);
+        v[t].a = ld_s(q);
+        v[t].b = ld_s(q + x.st);
+        v[t].c = x.k[2] != T(0) ? ld_s(q + 2 * x.st) : T(0);
+    }
+}
+
+// One rim node of a half-step (J, pm: the warp's sources and probes).  One code
+// for every rim node: variants for the row ends and for the layers took a
+// quarter fewer instructions and 15 % more time, waiting for instruction fetch.
+template <typename T, typename S, bool ELECTRIC, bool MUVAR>
+__device__ __forceinline__ void rim_node(const Params<T, S> &p, int i, int j, int k, const double *J,
+                                         unsigned long long pm)
+{
+    constexpr int c0 = ELECTRIC ? 0 : 3;
+    const int idx[3] = {i, j, k};
+    const RimAxis<T> ax[3] = {rim_axis<ELECTRIC, T>(p, 0, i), rim_axis<ELECTRIC, T>(p, 1, j),
+                              rim_axis<ELECTRIC, T>(p, 2, k)};
+    const long long o = (long long)k * p.sz + (long long)j * p.sy + i;
+    const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
+    const bool abs = ax[0].type == kABS || ax[1].type == kABS || ax[2].type == kABS;
+    pdl_wait();
+    Tri<T> vx[2], vy[2], vz[2];
+    rim_gather<c0>(p, ax, o, vx);
+    rim_gather<c0 + 1>(p, ax, o, vy);
+    rim_gather<c0 + 2>(p, ax, o, vz);
+    T x = ld_s(p.F[c0] + o), y = ld_s(p.F[c0 + 1] + o), z = ld_s(p.F[c0 + 2] + o);
+    T ex = T(0), ey = T(0), ez = T(0), mx = T(0), my = T(0), mz = T(0);
+    if (ELECTRIC || abs) {
+        ex = cell_sum<c0, T>(p.eps, o, p.sy, p.sz);
+        ey = cell_sum<c0 + 1, T>(p.eps, o, p.sy, p.sz);
+        ez = cell_sum<c0 + 2, T>(p.eps, o, p.sy, p.sz);
+    }
+    if (MUVAR && (!ELECTRIC || abs)) {
+        mx = cell_sum<c0, T>(p.mu, o, p.sy, p.sz);
+        my = cell_sum<c0 + 1, T>(p.mu, o, p.sy, p.sz);
+        mz = cell_sum<c0 + 2, T>(p.mu, o, p.sy, p.sz);
+    }
+    x = rim_apply<T, c0, MUVAR>(p, ax, idx, x, vx, ex, mx, J);
+    y = rim_apply<T, c0 + 1, MUVAR>(p, ax, idx, y, vy, ey, my, J);
+    z = rim_apply<T, c0 + 2, MUVAR>(p, ax, idx, z, vz, ez, mz, J);
+    // nodes of each component (Table I); the others are not stored and hold no probe
+    const int e = ELECTRIC ? 1 : 0;
+    if (i <= nx + e && j <= ny + 1 - e && k <= nz + 1 - e) st_s(p.F[c0] + o, x);
+    if (i <= nx + 1 - e && j <= ny + e && k <= nz + 1 - e) st_s(p.F[c0 + 1] + o, y);
+    if (i <= nx + 1 - e && j <= ny + 1 - e && k <= nz + e) st_s(p.F[c0 + 2] + o, z);
+    if (pm) {
+        const T a[1] = {x}, b[1] = {y}, c[1] = {z};
+        vec_probes<1>(p, pm, c0, i, j, k, a, b, c);
+    }
+}
+
+// Rim CTAs: the planes below and above the box first, then per z-chunk the y
+// layers and the row ends of its box planes.
+template <typename T, typename S, bool ELECTRIC, bool MUVAR>
+__device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w, unsigned cta, unsigned q, int chunk)
+{
+    unsigned t, count;
+    int i, j, k;
+    if (cta < w.cz) {
+        t = cta * (unsigned)kSweepThreads + threadIdx.x;
+        count = w.zplanes * w.rows * w.xs;
+        if ((t & ~31u) >= count) return;
+        const unsigned tc = min(t, count - 1u), row = tc / w.dxs, pl = row / w.drows;
+        i = (int)(tc - row * w.xs);
+        j = (int)(row - pl * w.rows);
+        k = (int)pl < w.lo[2] ? (int)pl : w.hi[2] + 1 + ((int)pl - w.lo[2]);
+    } else {
+        const int kb = max(chunk * w.kz, w.lo[2]), ke = min(chunk * w.kz + w.kz - 1, w.hi[2]);
+        if (kb > ke) return;
+        t = (q - w.cbox) * (unsigned)kSweepThreads + threadIdx.x;
+        count = (unsigned)(ke - kb + 1) * w.rim;
+        if ((t & ~31u) >= count) return;
+        const unsigned tc = min(t, count - 1u), pl = tc / w.drim, u = tc - pl * w.rim;
+        k = kb + (int)pl;
+        if (u < w.ynodes) {
+            const unsigned row = u / w.dxs;
+            i = (int)(u - row * w.xs);
+            j = (int)row < w.lo[1] ? (int)row : w.hi[1] + 1 + ((int)row - w.lo[1]);
+        } else {
+            const unsigned row = (u - w.ynodes) / w.dends, e = u - w.ynodes - row * w.ends;
+            i = (int)e < w.lo[0] ? (int)e : w.hi[0] + 1 + ((int)e - w.lo[0]);
+            j = w.lo[1] + (int)row;
+        }
+    }
+    unsigned long long pm = 0ull;
+    const double *J = nullptr;
+    if (p.nprb || (ELECTRIC && p.nsrc)) {
+        const int lane = threadIdx.x & 31;
+        const int jmin = __reduce_min_sync(0xffffffffu, j), jmax = __reduce_max_sync(0xffffffffu, j);
+        const int kmin = __reduce_min_sync(0xffffffffu, k), kmax = __reduce_max_sync(0xffffffffu, k);
+        if (p.nprb) pm = rows_probe_mask(p.prb, p.nprb, ELECTRIC ? 0 : 3, kmin, kmax, jmin, jmax, lane);
+        if (ELECTRIC) J = source_values(p, p.step, lane, kmin, kmax, jmin, jmax, 0, INT32_MAX);
+    }
+    if (t >= count) return;
+    rim_node<T, S, ELECTRIC, MUVAR>(p, i, j, k, J, pm);
+}
+
+template <typename T, typename S, bool MUVAR, int V>
+__global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 4 : 5)
+    half_h(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
+{
+    pdl_release();
+    const unsigned cta = blockIdx.x, r = cta < w.cz ? 0u : cta - w.cz;
+    const unsigned chunk = r / w.dchunk, q = r - chunk * w.cchunk;
+    if (cta >= w.cz && q < w.cbox) box_h<T, S, MUVAR, V>(p, w, q, (int)chunk);
+    else sweep_rim<T, S, false, MUVAR>(p, w, cta, q, (int)chunk);
+}
+
+template <typename T, typename S, bool MUVAR, int V>
+__global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 4 : 5)
+    half_e(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
+{
+    pdl_release();
+    const unsigned cta = blockIdx.x, r = cta < w.cz ? 0u : cta - w.cz;
+    const unsigned chunk = r / w.dchunk, q = r - chunk * w.cchunk;
+    if (cta >= w.cz && q < w.cbox) box_e<T, S, V>(p, w, q, (int)chunk);
+    else sweep_rim<T, S, true, MUVAR>(p, w, cta, q, (int)chunk);
+}
+
+}  // namespace sbp

@@ -1,17 +1,12 @@
 // Device code of the GB300 SBP-SAT FDTD library (arXiv 2206.00638).
 //
-// Two fused kernels advance one leapfrog step:
-//   h_update  H^{n+1/2} = H^{n-1/2} + dt/mu (D- E^n) + SAT_H     Eqs. (10)-(15), Alg. 2
-//   e_update  E^{n+1}   = E^n + dt/eps (D+ H^{n+1/2} - J) + SAT_E Eqs. (7)-(9), (19)-(21), Alg. 1
-// Each thread owns one (i, j) column of nodes and marches up a chunk of z
-// planes (2.5D blocking): the z-neighbour needed by the staggered difference
-// is carried in a register from the previous plane, x/y neighbours come from
-// L1.  Interior nodes (every index in [3, n-2]) take a branch-free fast path
-// with the two-point stencil; the three boundary layers of each axis take the
-// general path, which evaluates the closure rows of D+ / D- (Appendix), the
-// SAT penalties of the face type (PEC / PMC / absorbing / interface), point
-// and sheet sources and probes.  The fast/general choice is uniform per warp
-// except in the two x-edge warps of a row.
+// This file holds what every kernel shares: the operator rows (Appendix) with
+// their closure rows, the SAT penalties of the face types (PEC / PMC /
+// absorbing / interface), node materials, sources and the arithmetic of one
+// node, and the kernels that do not step: the energy, the copies of a field in
+// and out of the padded layout, the coefficient build.  halfstep.cuh steps in
+// place, one launch per half-step; fused.cuh steps the deep interior in one
+// pass between two field sets.
 //
 // FP32 arithmetic keeps its coefficients exact to ~1e-14: every material
 // coefficient dt/(eps h) is carried as an unevaluated sum hi + lo of two
@@ -102,7 +97,7 @@ struct Params {
     T *probe_buf;
     long long probe_cap, probe_slot;   // sample slot of this step (skip if >= cap)
     long long step;                    // n: the E half-step injects J(t^{n+1/2})
-    double *partials;                  // energy partial sums, one per CTA of h_update
+    double *partials;                  // energy partial sums, one per CTA of energy_sum
     int kchunk;
     int fdtd;                          // 1: plain Yee FDTD comparator (band kernels only)
 };
@@ -137,6 +132,33 @@ __device__ __forceinline__ void recip_pair(float s, float &rh, float &rl)
     rl = r * e;
 }
 
+// A positive normal float as T.  The FP64 form moves the bits with integer
+// operations: the FP64 pipe, which converts too, takes 2 lanes per clock and SM.
+template <typename T> __device__ __forceinline__ T widen(float f);
+template <> __device__ __forceinline__ float widen<float>(float f) { return f; }
+template <> __device__ __forceinline__ double widen<double>(float f)
+{
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+}
+
+// 1/s for a positive s: an FP32 approximation of the reciprocal of s's leading
+// bits (relative error d < 2^-21) corrected in FP64, r (1 + d + d^2), which
+// leaves d^3 < 2^-63 beside the rounding of the last operation.  Three FP64
+// operations; a division takes about ten, at 2 lanes per clock and SM.  Values
+// outside FP32's comfortable range divide.
+__device__ __noinline__ double recip64_any(double s) { return 1.0 / s; }
+__device__ __forceinline__ double recip64(double s)
+{
+    const int hi = __double2hiint(s);
+    if ((unsigned)(hi - (923 << 20)) >= (unsigned)(200 << 20)) return recip64_any(s);    // not in [2^-100, 2^100)
+    const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(s), (unsigned)(hi - (896 << 20)), 3));
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+    const double rd = widen<double>(r), d = fma(-s, rd, 1.0);
+    return fma(rd, fma(d, d, d), rd);
+}
+
 // increment = r * acc with r = 1/s (E nodes, or H nodes with varying mu)
 __device__ __forceinline__ float scaled_increment(const Acc<float> &a, float s)
 {
@@ -146,7 +168,7 @@ __device__ __forceinline__ float scaled_increment(const Acc<float> &a, float s)
 }
 __device__ __forceinline__ double scaled_increment(const Acc<double> &a, double s)
 {
-    return a.hi / s;
+    return a.hi * recip64(s);
 }
 __device__ __forceinline__ float plain_increment(const Acc<float> &a) { return a.hi + a.lo; }
 __device__ __forceinline__ double plain_increment(const Acc<double> &a) { return a.hi; }
@@ -168,6 +190,14 @@ __device__ __forceinline__ float scaled_increment(const AccLite &a, float s)
     return fmaf(rh, a.hi, rl * a.hi);
 }
 __device__ __forceinline__ float plain_increment(const AccLite &a) { return a.hi; }
+
+// old + acc / s (interior nodes).
+template <typename A>
+__device__ __forceinline__ float add_scaled(float old, const A &a, float s) { return old + scaled_increment(a, s); }
+__device__ __forceinline__ double add_scaled(double old, const Acc<double> &a, double s)
+{
+    return fma(a.hi, recip64(s), old);
+}
 
 // The accumulator of arithmetic type T for fields stored as S.
 template <typename T, typename S> struct AccOf { using type = Acc<T>; };
@@ -318,7 +348,10 @@ __device__ __forceinline__ T abs_gamma_e(T a, T se, T eta) { return a / se / (T(
 template <typename T>
 __device__ __forceinline__ T sat_finish(T old, T inc, T gam)
 {
-    if (gam != T(0)) return fma_t(T(1) - gam, old, inc) / (T(1) + gam);
+    if (gam != T(0)) {
+        if constexpr (std::is_same<T, double>::value) return fma_t(T(1) - gam, old, inc) * recip64(T(1) + gam);
+        return fma_t(T(1) - gam, old, inc) / (T(1) + gam);
+    }
     return old + inc;
 }
 
@@ -339,7 +372,8 @@ __device__ __forceinline__ int extent(const int n[3], int c, int a) { return n[a
 template <typename S>
 __device__ __forceinline__ S pair_sum(const float *__restrict__ m, long long o, long long a, long long b)
 {
-    return (S(__ldg(m + o)) + S(__ldg(m + o + a))) + (S(__ldg(m + o + b)) + S(__ldg(m + o + a + b)));
+    return (widen<S>(__ldg(m + o)) + widen<S>(__ldg(m + o + a))) +
+           (widen<S>(__ldg(m + o + b)) + widen<S>(__ldg(m + o + a + b)));
 }
 
 // Sum of the ghost-padded cell values around a node of component c: the
@@ -358,7 +392,7 @@ __device__ __forceinline__ S cell_sum(const float *__restrict__ m, long long o, 
     if (px && pz) return pair_sum<S>(m, o, 1, sz);
     if (py && pz) return pair_sum<S>(m, o, sy, sz);
     const long long d = px ? 1 : py ? sy : sz;
-    return S(__ldg(m + o)) + S(__ldg(m + o + d));
+    return widen<S>(__ldg(m + o)) + widen<S>(__ldg(m + o + d));
 }
 // number of entries summed by cell_sum<C>
 __host__ __device__ constexpr int cell_count(int c)
@@ -366,8 +400,10 @@ __host__ __device__ constexpr int cell_count(int c)
     return (on_plus(c, 0) ? 2 : 1) * (on_plus(c, 1) ? 2 : 1) * (on_plus(c, 2) ? 2 : 1);
 }
 
-// Source waveforms (Sec. VI-B, VI-C): t and t0, tw in seconds.
-__device__ __forceinline__ double waveform(int wf, double t, double tw, double t0, double f)
+// Source waveforms (Sec. VI-B, VI-C): t and t0, tw in seconds.  A call, not
+// inlined: a few lanes of a launch reach it, and its code would sit between the
+// instructions that every warp fetches.
+__device__ __noinline__ double waveform(int wf, double t, double tw, double t0, double f)
 {
     const double x = (t - t0) / tw;
     const double g = exp(-4.0 * 3.14159265358979323846 * x * x);
@@ -378,35 +414,32 @@ __device__ __forceinline__ double waveform(int wf, double t, double tw, double t
     return sin(6.283185307179586 * ph) * g;
 }
 
+// J(t^{n+1/2}) of the sources that reach the index box of a warp, in the
+// warp's slots of shared memory (entry q for source q), or null when none
+// does.  One lane evaluates each source, once for the warp: the FP64 waveform
+// costs about as much as a whole node.  Every lane of the warp calls it.
 template <typename T, typename S>
-__device__ __forceinline__ bool probe_here(const Params<T, S> &p, unsigned long long mask, int k)
+__device__ __forceinline__ const double *source_values(const Params<T, S> &p, long long step, int lane, int k0, int k1,
+                                                       int j0, int j1, int i0, int i1)
 {
-    while (mask) {
-        int q = __ffsll(mask) - 1;
-        mask &= mask - 1;
-        if (p.prb[q].k == k) return true;
+    static_assert(kMaxSources <= 32, "one lane per source");
+    __shared__ double sJ[8][kMaxSources];
+    if (!p.nsrc) return nullptr;
+    bool hit = false;
+    if (lane < p.nsrc) {
+        const Src &Sr = p.src[lane];
+        hit = (Sr.i < 0 || (Sr.i >= i0 && Sr.i <= i1)) && (Sr.j < 0 || (Sr.j >= j0 && Sr.j <= j1)) &&
+              (Sr.k < 0 || (Sr.k >= k0 && Sr.k <= k1));
     }
-    return false;
-}
-template <typename T, typename S>
-__device__ __forceinline__ bool source_here(const Params<T, S> &p, unsigned mask, int k)
-{
-    while (mask) {
-        int q = __ffs(mask) - 1;
-        mask &= mask - 1;
-        if (p.src[q].k == k || p.src[q].k < 0) return true;
+    if (!__any_sync(0xffffffffu, hit)) return nullptr;
+    double *const J = sJ[(threadIdx.x >> 5) & 7];
+    __syncwarp();                                     // reads of an earlier use are done
+    if (hit) {
+        const Src &Sr = p.src[lane];
+        J[lane] = Sr.amp * waveform(Sr.wf, ((double)step + 0.5) * p.dt, Sr.tw, Sr.t0, Sr.f);
     }
-    return false;
-}
-template <typename T, typename S>
-__device__ __forceinline__ void write_probes(const Params<T, S> &p, unsigned long long mask, int c, int k, T v)
-{
-    while (mask) {
-        int q = __ffsll(mask) - 1;
-        mask &= mask - 1;
-        if (p.prb[q].comp == c && p.prb[q].k == k && p.probe_slot < p.probe_cap)
-            p.probe_buf[(long long)q * p.probe_cap + p.probe_slot] = v * p.fscale[c >= 3];
-    }
+    __syncwarp();
+    return J;
 }
 
 // Block-wide deterministic sum of one double per thread (fixed tree).
@@ -531,7 +564,7 @@ __device__ __forceinline__ void e_gather(const Params<T, S> &p, const int idx[3]
 // node and the gathered H.
 template <typename T, int C, bool MUVAR, bool CG = false, int G = 7, typename S = T>
 __device__ __forceinline__ T e_apply(const Params<T, S> &p, const int idx[3], long long o, T eold, T se, const Tri<T> v[2],
-                                     unsigned smask, double t_half)
+                                     unsigned smask, const double *J)
 {
     typename AccOf<T, S>::type acc;
     T gam = T(0);
@@ -573,48 +606,20 @@ __device__ __forceinline__ T e_apply(const Params<T, S> &p, const int idx[3], lo
         const int q = __ffs(m) - 1;
         m &= m - 1;
         const Src &Sr = p.src[q];
-        if (Sr.comp == C && (Sr.k < 0 || Sr.k == idx[2])) {
-            const double J = Sr.amp * waveform(Sr.wf, t_half, Sr.tw, Sr.t0, Sr.f);
-            acc.add(p.AJ, T(J), T(-1));
-        }
+        if (Sr.comp == C && (Sr.k < 0 || Sr.k == idx[2])) acc.add(p.AJ, T(J[q]), T(-1));
     }
     const T inc = scaled_increment(acc, se);
     return sat_finish(eold, inc, gam);
-}
-
-// E half-step, general path, one component at one node (Eqs. (7)-(9), (19)-(21)).
-template <typename T, int C, bool MUVAR, bool CG = false, typename S = T>
-__device__ __forceinline__ T e_node(const Params<T, S> &p, const int idx[3], long long o, T eold,
-                                    unsigned smask, double t_half)
-{
-    const T se = cell_sum<C, T>(p.eps, o, p.sy, p.sz);     // 4 * eps_r(node)
-    Tri<T> v[2];
-    e_gather<T, C, CG, 7>(p, idx, o, v);
-    return e_apply<T, C, MUVAR, CG, 7>(p, idx, o, eold, se, v, smask, t_half);
 }
 
 // ---------------------------------------------------------------------------
 // Kernels
 // ---------------------------------------------------------------------------
 
-// Per-thread masks of the probes / sources whose (i, j) match this column.
-template <typename T, typename S>
-__device__ __forceinline__ void column_masks(const Params<T, S> &p, int i, int j, bool want_h,
-                                             unsigned long long &pm, unsigned &sm)
-{
-    pm = 0ull;
-    sm = 0u;
-    for (int q = 0; q < p.nprb; ++q)
-        if (p.prb[q].i == i && p.prb[q].j == j && ((p.prb[q].comp >= 3) == want_h)) pm |= 1ull << q;
-    if (!want_h)
-        for (int q = 0; q < p.nsrc; ++q)
-            if ((p.src[q].i < 0 || p.src[q].i == i) && (p.src[q].j < 0 || p.src[q].j == j)) sm |= 1u << q;
-}
-
-// H half-step.  ENERGY: also accumulate the leapfrog energy of Eq. (16) into
-// p.partials (FP64); STORE: write H^{n+1/2} (false = energy query only).
-template <typename T, typename S, bool ENERGY, bool STORE, bool MUVAR>
-__global__ void __launch_bounds__(kBlockX *kBlockY) h_update(const Params<T, S> p)
+// Leapfrog energy of Eq. (16) (FP64) over every node, one partial sum per CTA
+// in p.partials: H^{n+1/2} is formed on the fly, no field is changed.
+template <typename T, typename S, bool MUVAR>
+__global__ void __launch_bounds__(kBlockX *kBlockY) energy_sum(const Params<T, S> p)
 {
     const int i = blockIdx.x * kBlockX + threadIdx.x;
     const int j = blockIdx.y * kBlockY + threadIdx.y;
@@ -623,183 +628,61 @@ __global__ void __launch_bounds__(kBlockX *kBlockY) h_update(const Params<T, S> 
     const int k1 = min(k0 + p.kchunk, nz + 2);
     double wacc = 0.0;
     if (i < nx + 2 && j < ny + 2) {
-        S *__restrict__ Hx = p.F[3];
-        S *__restrict__ Hy = p.F[4];
-        S *__restrict__ Hz = p.F[5];
+        const S *__restrict__ Hx = p.F[3];
+        const S *__restrict__ Hy = p.F[4];
+        const S *__restrict__ Hz = p.F[5];
         const S *__restrict__ Ex = p.F[0];
         const S *__restrict__ Ey = p.F[1];
         const S *__restrict__ Ez = p.F[2];
         const double es2 = (double)p.fscale[0] * (double)p.fscale[0];   // energy of stored values
         const double hs2 = (double)p.fscale[1] * (double)p.fscale[1];
-        unsigned long long pm;
-        unsigned sm;
-        column_masks(p, i, j, true, pm, sm);
-        const bool xyin = i >= 3 && i <= nx - 2 && j >= 3 && j <= ny - 2;
-        const Coef<T> Bx = p.B[0], By = p.B[1], Bz = p.B[2];
         long long o = (long long)k0 * p.sz + (long long)j * p.sy + i;
-        T exm = k0 > 0 ? ldg_s(Ex + o - p.sz) : T(0);
-        T eym = k0 > 0 ? ldg_s(Ey + o - p.sz) : T(0);
         for (int k = k0; k < k1; ++k, o += p.sz) {
-            const T exc = ldg_s(Ex + o);
-            const T eyc = ldg_s(Ey + o);
-            const bool fast = !ENERGY && !MUVAR && xyin && k >= 3 && k <= nz - 2 && !(pm && probe_here(p, pm, k));
-            if (fast) {
-                const T ezc = ldg_s(Ez + o);
-                const T ex_jm = ldg_s(Ex + o - p.sy);
-                const T ey_im = ldg_s(Ey + o - 1);
-                const T ez_im = ldg_s(Ez + o - 1);
-                const T ez_jm = ldg_s(Ez + o - p.sy);
-                const T dEy_z = eyc - eym, dEz_y = ezc - ez_jm;
-                const T dEz_x = ezc - ez_im, dEx_z = exc - exm;
-                const T dEx_y = exc - ex_jm, dEy_x = eyc - ey_im;
-                typename AccOf<T, S>::type ax, ay, az;
-                ax.add(Bz, dEy_z); ax.add(By, dEz_y, T(-1));
-                ay.add(Bx, dEz_x); ay.add(Bz, dEx_z, T(-1));
-                az.add(By, dEx_y); az.add(Bx, dEy_x, T(-1));
-                st_s(Hx + o, ld_s(Hx + o) + plain_increment(ax));
-                st_s(Hy + o, ld_s(Hy + o) + plain_increment(ay));
-                st_s(Hz + o, ld_s(Hz + o) + plain_increment(az));
-            } else {
-                const int idx[3] = {i, j, k};
-                // Hx (x+, y-, z-)
-                if (i <= nx && j <= ny + 1 && k <= nz + 1) {
-                    const T ho = ld_s(Hx + o);
-                    const T hn = quant<S>(h_node<T, 3, MUVAR>(p, idx, o, ho));
-                    if (STORE) st_s(Hx + o, hn);
-                    if (STORE && pm) write_probes(p, pm, 3, k, hn);
-                    if (ENERGY) {
-                        const double w = norm_weight(true, i, nx) * norm_weight(false, j, ny) * norm_weight(false, k, nz);
-                        const double mr = MUVAR ? 0.5 * cell_sum<3, double>(p.mu, o, p.sy, p.sz) : 1.0;
-                        wacc += p.mu0 * mr * w * (double)ho * (double)hn * hs2;
-                    }
-                }
-                // Hy (x-, y+, z-)
-                if (i <= nx + 1 && j <= ny && k <= nz + 1) {
-                    const T ho = ld_s(Hy + o);
-                    const T hn = quant<S>(h_node<T, 4, MUVAR>(p, idx, o, ho));
-                    if (STORE) st_s(Hy + o, hn);
-                    if (STORE && pm) write_probes(p, pm, 4, k, hn);
-                    if (ENERGY) {
-                        const double w = norm_weight(false, i, nx) * norm_weight(true, j, ny) * norm_weight(false, k, nz);
-                        const double mr = MUVAR ? 0.5 * cell_sum<4, double>(p.mu, o, p.sy, p.sz) : 1.0;
-                        wacc += p.mu0 * mr * w * (double)ho * (double)hn * hs2;
-                    }
-                }
-                // Hz (x-, y-, z+)
-                if (i <= nx + 1 && j <= ny + 1 && k <= nz) {
-                    const T ho = ld_s(Hz + o);
-                    const T hn = quant<S>(h_node<T, 5, MUVAR>(p, idx, o, ho));
-                    if (STORE) st_s(Hz + o, hn);
-                    if (STORE && pm) write_probes(p, pm, 5, k, hn);
-                    if (ENERGY) {
-                        const double w = norm_weight(false, i, nx) * norm_weight(false, j, ny) * norm_weight(true, k, nz);
-                        const double mr = MUVAR ? 0.5 * cell_sum<5, double>(p.mu, o, p.sy, p.sz) : 1.0;
-                        wacc += p.mu0 * mr * w * (double)ho * (double)hn * hs2;
-                    }
-                }
-                if (ENERGY) {
-                    // E^n part: eps P''' E^2 at this node position for every E component present
-                    if (i <= nx + 1 && j <= ny && k <= nz) {   // Ex (x-, y+, z+)
-                        const double w = norm_weight(false, i, nx) * norm_weight(true, j, ny) * norm_weight(true, k, nz);
-                        wacc += p.eps0 * 0.25 * cell_sum<0, double>(p.eps, o, p.sy, p.sz) * w * (double)exc * (double)exc * es2;
-                    }
-                    if (i <= nx && j <= ny + 1 && k <= nz) {   // Ey (x+, y-, z+)
-                        const double w = norm_weight(true, i, nx) * norm_weight(false, j, ny) * norm_weight(true, k, nz);
-                        wacc += p.eps0 * 0.25 * cell_sum<1, double>(p.eps, o, p.sy, p.sz) * w * (double)eyc * (double)eyc * es2;
-                    }
-                    if (i <= nx && j <= ny && k <= nz + 1) {   // Ez (x+, y+, z-)
-                        const double w = norm_weight(true, i, nx) * norm_weight(true, j, ny) * norm_weight(false, k, nz);
-                        const T ezc = ldg_s(Ez + o);
-                        wacc += p.eps0 * 0.25 * cell_sum<2, double>(p.eps, o, p.sy, p.sz) * w * (double)ezc * (double)ezc * es2;
-                    }
-                }
-            }
-            exm = exc;
-            eym = eyc;
-        }
-    }
-    if (ENERGY) {
-        const double hvol = p.h[0] * p.h[1] * p.h[2];
-        block_sum_to(wacc * hvol, p.partials + ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
-    }
-}
-
-// E half-step with sources (J at t^{n+1/2}) and E probes.
-template <typename T, typename S, bool MUVAR>
-__global__ void __launch_bounds__(kBlockX *kBlockY) e_update(const Params<T, S> p)
-{
-    const int i = blockIdx.x * kBlockX + threadIdx.x;
-    const int j = blockIdx.y * kBlockY + threadIdx.y;
-    const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
-    const int k0 = blockIdx.z * p.kchunk;
-    const int k1 = min(k0 + p.kchunk, nz + 2);
-    if (i >= nx + 2 || j >= ny + 2) return;
-    S *__restrict__ Ex = p.F[0];
-    S *__restrict__ Ey = p.F[1];
-    S *__restrict__ Ez = p.F[2];
-    const S *__restrict__ Hx = p.F[3];
-    const S *__restrict__ Hy = p.F[4];
-    const S *__restrict__ Hz = p.F[5];
-    const float *__restrict__ eps = p.eps;
-    unsigned long long pm;
-    unsigned sm;
-    column_masks(p, i, j, false, pm, sm);
-    const bool xyin = i >= 3 && i <= nx - 2 && j >= 3 && j <= ny - 2;
-    const Coef<T> Ax = p.A[0], Ay = p.A[1], Az = p.A[2];
-    const double t_half = ((double)p.step + 0.5) * p.dt;
-    long long o = (long long)k0 * p.sz + (long long)j * p.sy + i;
-    // plane-k carries: Hx, Hy at (i,j,k) and eps at the four cells (i..i+1, j..j+1, k)
-    T hxc = ldg_s(Hx + o), hyc = ldg_s(Hy + o);
-    float f00 = __ldg(eps + o), f10 = __ldg(eps + o + 1), f01 = __ldg(eps + o + p.sy), f11 = __ldg(eps + o + 1 + p.sy);
-    for (int k = k0; k < k1; ++k, o += p.sz) {
-        const bool fast = xyin && k >= 3 && k <= nz - 2 && !(pm && probe_here(p, pm, k)) && !(sm && source_here(p, sm, k));
-        // next plane (k+1) always exists inside the padded array for k <= nz
-        const bool has_next = k + 1 < nz + 2;
-        const T hxn = has_next ? ldg_s(Hx + o + p.sz) : T(0);
-        const T hyn = has_next ? ldg_s(Hy + o + p.sz) : T(0);
-        const float e00 = has_next ? __ldg(eps + o + p.sz) : 0.f;
-        const float e10 = has_next ? __ldg(eps + o + p.sz + 1) : 0.f;
-        const float e01 = has_next ? __ldg(eps + o + p.sz + p.sy) : 0.f;
-        const float e11 = has_next ? __ldg(eps + o + p.sz + p.sy + 1) : 0.f;
-        if (fast) {
-            const T hzc = ldg_s(Hz + o);
-            const T hz_jp = ldg_s(Hz + o + p.sy);
-            const T hz_ip = ldg_s(Hz + o + 1);
-            const T hx_jp = ldg_s(Hx + o + p.sy);
-            const T hy_ip = ldg_s(Hy + o + 1);
-            typename AccOf<T, S>::type ax, ay, az;
-            ax.add(Ay, hz_jp - hzc); ax.add(Az, hyn - hyc, T(-1));
-            ay.add(Az, hxn - hxc);   ay.add(Ax, hz_ip - hzc, T(-1));
-            az.add(Ax, hy_ip - hyc); az.add(Ay, hx_jp - hxc, T(-1));
-            // node sums in the association of cell_sum: Ex (m, +sy, +sz, +sy+sz),
-            // Ey (m, +1, +sz, +1+sz), Ez (m, +1, +sy, +1+sy)
-            const T sx = (T(f00) + T(f01)) + (T(e00) + T(e01));
-            const T sy = (T(f00) + T(f10)) + (T(e00) + T(e10));
-            const T sz = (T(f00) + T(f10)) + (T(f01) + T(f11));
-            st_s(Ex + o, ld_s(Ex + o) + scaled_increment(ax, sx));
-            st_s(Ey + o, ld_s(Ey + o) + scaled_increment(ay, sy));
-            st_s(Ez + o, ld_s(Ez + o) + scaled_increment(az, sz));
-        } else {
             const int idx[3] = {i, j, k};
-            if (i <= nx + 1 && j <= ny && k <= nz) {          // Ex (x-, y+, z+)
-                const T en = quant<S>(e_node<T, 0, MUVAR>(p, idx, o, ld_s(Ex + o), sm, t_half));
-                st_s(Ex + o, en);
-                if (pm) write_probes(p, pm, 0, k, en);
+            // Hx (x+, y-, z-)
+            if (i <= nx && j <= ny + 1 && k <= nz + 1) {
+                const T ho = ld_s(Hx + o);
+                const T hn = quant<S>(h_node<T, 3, MUVAR>(p, idx, o, ho));
+                const double w = norm_weight(true, i, nx) * norm_weight(false, j, ny) * norm_weight(false, k, nz);
+                const double mr = MUVAR ? 0.5 * cell_sum<3, double>(p.mu, o, p.sy, p.sz) : 1.0;
+                wacc += p.mu0 * mr * w * (double)ho * (double)hn * hs2;
             }
-            if (i <= nx && j <= ny + 1 && k <= nz) {          // Ey (x+, y-, z+)
-                const T en = quant<S>(e_node<T, 1, MUVAR>(p, idx, o, ld_s(Ey + o), sm, t_half));
-                st_s(Ey + o, en);
-                if (pm) write_probes(p, pm, 1, k, en);
+            // Hy (x-, y+, z-)
+            if (i <= nx + 1 && j <= ny && k <= nz + 1) {
+                const T ho = ld_s(Hy + o);
+                const T hn = quant<S>(h_node<T, 4, MUVAR>(p, idx, o, ho));
+                const double w = norm_weight(false, i, nx) * norm_weight(true, j, ny) * norm_weight(false, k, nz);
+                const double mr = MUVAR ? 0.5 * cell_sum<4, double>(p.mu, o, p.sy, p.sz) : 1.0;
+                wacc += p.mu0 * mr * w * (double)ho * (double)hn * hs2;
             }
-            if (i <= nx && j <= ny && k <= nz + 1) {          // Ez (x+, y+, z-)
-                const T en = quant<S>(e_node<T, 2, MUVAR>(p, idx, o, ld_s(Ez + o), sm, t_half));
-                st_s(Ez + o, en);
-                if (pm) write_probes(p, pm, 2, k, en);
+            // Hz (x-, y-, z+)
+            if (i <= nx + 1 && j <= ny + 1 && k <= nz) {
+                const T ho = ld_s(Hz + o);
+                const T hn = quant<S>(h_node<T, 5, MUVAR>(p, idx, o, ho));
+                const double w = norm_weight(false, i, nx) * norm_weight(false, j, ny) * norm_weight(true, k, nz);
+                const double mr = MUVAR ? 0.5 * cell_sum<5, double>(p.mu, o, p.sy, p.sz) : 1.0;
+                wacc += p.mu0 * mr * w * (double)ho * (double)hn * hs2;
+            }
+            // E^n part: eps P E^2 at this node position for every E component present
+            if (i <= nx + 1 && j <= ny && k <= nz) {   // Ex (x-, y+, z+)
+                const double w = norm_weight(false, i, nx) * norm_weight(true, j, ny) * norm_weight(true, k, nz);
+                const T e = ldg_s(Ex + o);
+                wacc += p.eps0 * 0.25 * cell_sum<0, double>(p.eps, o, p.sy, p.sz) * w * (double)e * (double)e * es2;
+            }
+            if (i <= nx && j <= ny + 1 && k <= nz) {   // Ey (x+, y-, z+)
+                const double w = norm_weight(true, i, nx) * norm_weight(false, j, ny) * norm_weight(true, k, nz);
+                const T e = ldg_s(Ey + o);
+                wacc += p.eps0 * 0.25 * cell_sum<1, double>(p.eps, o, p.sy, p.sz) * w * (double)e * (double)e * es2;
+            }
+            if (i <= nx && j <= ny && k <= nz + 1) {   // Ez (x+, y+, z-)
+                const double w = norm_weight(true, i, nx) * norm_weight(true, j, ny) * norm_weight(false, k, nz);
+                const T e = ldg_s(Ez + o);
+                wacc += p.eps0 * 0.25 * cell_sum<2, double>(p.eps, o, p.sy, p.sz) * w * (double)e * (double)e * es2;
             }
         }
-        hxc = hxn; hyc = hyn;
-        f00 = e00; f10 = e10; f01 = e01; f11 = e11;
     }
+    const double hvol = p.h[0] * p.h[1] * p.h[2];
+    block_sum_to(wacc * hvol, p.partials + ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
 
 // Fixed-order sum of the per-CTA energy partials (one CTA, deterministic).

@@ -9,11 +9,11 @@
 // addresses node (i, j, k) of every component; positions outside a
 // component's natural extents (Table I) stay zero.
 //
-// Two step paths.  FP32 blocks with uniform mu and at least 8 cells per axis
-// keep two field sets and advance with three launches per step (band_h,
+// Two step paths, bit-identical where both run.  Large FP32 blocks with uniform
+// mu keep two field sets and advance with three launches per step (band_h,
 // fused_interior, band_e: old set -> new set, then swap).  Everything else
-// (FP64, varying mu, energy-monitor steps, the half-step calls) uses the
-// in-place h_update / e_update pair on the current set.
+// (smaller grids, FP16 storage, FP64, varying mu, the half-step calls) uses the
+// in-place half_h / half_e pair on the current set.
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -36,6 +36,7 @@
 #include "sbpsat.h"
 #include "kernels.cuh"
 #include "fused.cuh"
+#include "halfstep.cuh"
 
 namespace {
 
@@ -93,6 +94,7 @@ struct sbp_sim {
                        {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}};
     int cur = 0;                          // index of the set holding the current fields
     bool fused_ok = false;                // second set allocated, fused path usable
+    bool one_pass = false;                // steps run it (else the in-place half-steps)
     bool fused_step = false;              // this step runs the fused path (set during a step)
     int *error_flag = nullptr;            // device flag raised by a pipeline wait that gave up
     sbp::FusedMaps maps[2];               // TMA tensor maps reading set 0 / set 1
@@ -104,6 +106,8 @@ struct sbp_sim {
     cudaStream_t side = nullptr;          // band_h runs here, concurrently with fused_interior
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     sbp::Band band_hb, band_eb;
+    sbp::Sweep sweep[2];                  // in-place half-steps: work lists (H, E) and vector width
+    int sweep_v = 1;
     float *eps = nullptr;
     float *mu = nullptr;
     double *partials = nullptr;
@@ -397,6 +401,88 @@ int encode_maps(sbp_sim *s)
     return SBP_OK;
 }
 
+// Multiplier and shift of FastDiv's n / d for n < 2^31.
+sbp::FastDiv fast_div(unsigned d)
+{
+    unsigned l = 0;
+    while ((1ull << l) < d) l++;
+    return {(unsigned)(((1ull << 32) * ((1ull << l) - d)) / d + 1), l};
+}
+
+// Work list of an in-place half-step (electric: of E, else of H) of an n-cell
+// grid: vectors of v nodes, z-chunks of kz planes.
+int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w)
+{
+    std::memset(&w, 0, sizeof(w));
+    long long box[3];
+    for (int a = 0; a < 3; a++) {
+        // two-point rows of D+ : 2..n-2, of D- : 3..n-2; along x the box is whole vectors
+        const int lo = electric ? 2 : 3, hi = n[a] - 2;
+        w.lo[a] = a ? lo : (lo + v - 1) / v * v;
+        w.hi[a] = std::max(a ? hi : (hi + 1) / v * v - 1, w.lo[a] - 1);
+        box[a] = w.hi[a] - w.lo[a] + 1;
+    }
+    const long long nv = box[0] / v, planes = n[2] + 2, rows = n[1] + 2, xs = n[0] + 2;
+    const long long vecs = nv * box[1], zplanes = planes - box[2], ynodes = (rows - box[1]) * xs;
+    const long long ends = xs - box[0], rim = ynodes + ends * box[1];
+    auto ctas_of = [&](long long items) { return (items + sbp::kSweepThreads - 1) / sbp::kSweepThreads; };
+    const long long cz = ctas_of(zplanes * rows * xs), cbox = ctas_of(vecs), cchunk = cbox + ctas_of(kz * rim);
+    const long long ctas = cz + cchunk * ((planes + kz - 1) / kz);
+    if (std::max(std::max(zplanes * rows * xs, vecs), kz * rim) >= (1ll << 31) - 1024 || ctas >= (1ll << 31))
+        return SBP_EINVAL;
+    w.kz = kz;
+    w.nv = (unsigned)std::max(nv, 1ll);
+    w.vecs = (unsigned)vecs;
+    w.xs = (unsigned)xs;
+    w.rows = (unsigned)rows;
+    w.ends = (unsigned)std::max(ends, 1ll);
+    w.zplanes = (unsigned)zplanes;
+    w.ynodes = (unsigned)ynodes;
+    w.rim = (unsigned)std::max(rim, 1ll);
+    w.cz = (unsigned)cz;
+    w.cbox = (unsigned)cbox;
+    w.cchunk = (unsigned)cchunk;
+    w.ctas = (unsigned)ctas;
+    w.dnv = fast_div(w.nv);
+    w.dxs = fast_div(w.xs);
+    w.drows = fast_div(w.rows);
+    w.dends = fast_div(w.ends);
+    w.drim = fast_div(w.rim);
+    w.dchunk = fast_div(w.cchunk);
+    return SBP_OK;
+}
+
+// Vector width and planes per z-chunk of the in-place half-steps, by the nodes
+// of the grid.  Measured per step, CTAs of 128 threads (256 are 0-10 % slower
+// everywhere: fewer warps fit beside the register use):
+//   125 k nodes (61 x 47 x 38)    V 1: 7.8 us; V 2: 13, too few threads
+//   1.6 M nodes (117 x 96 x 131)  V 2, 4 planes: 22.7 us; V 1 27.7; V 4 24.3;
+//                                 V 2, 2 planes: 24.7, 1 plane: 28.6 (CTAs start at about one per ns)
+//   17 M nodes (256^3)            V 4, 8 planes: 229 us; V 2: 234; V 4, 4 planes: 230
+//   512^3, FP16 storage           V 4, 16 planes: 1138 us, 8 planes: 1168
+// FP64 is bound by its pipe and runs one node per thread (two: 1 % slower).
+int choose_sweep(sbp_sim *s)
+{
+    const long long nodes = (long long)(s->n[0] + 2) * (s->n[1] + 2) * (s->n[2] + 2);
+    int v = nodes < 200000 || s->prec == SBP_FP64 ? 1 : 4, kz = nodes < 200000 ? 1 : nodes < 600000 ? 2 : 4;
+    if (s->prec == SBP_FP64) kz = std::min(kz, 2);
+    else if (nodes > 64000000) kz = 16;
+    else if (nodes > 4000000) kz = 8;
+    else if (v == 4 && s->prec == SBP_FP32) v = 2;
+    s->sweep_v = v;
+    int rc = make_sweep(s->n, false, v, kz, s->sweep[0]);
+    return rc ? rc : make_sweep(s->n, true, v, kz, s->sweep[1]);
+}
+
+// Whether a step of this simulation runs the one-pass kernel (else the in-place
+// half-steps).  One pass moves 13 words per node instead of 19, but marches
+// planes behind a barrier and leaves the boundary to separate band launches, so
+// it pays where the grid is far larger than L2 (per step, FP32, one pass /
+// in place: 61 x 47 x 38 17.6 / 7.8 us, 117 x 96 x 131 39 / 22.7 us, 256^3 236 /
+// 229 us, 512^3 1483 / 1600 us).  With FP16 storage one pass is issue-bound
+// (512^3: 1337 / 1140 us) and never pays.
+constexpr long long kOnePassNodes = 24000000;
+
 int setup(sbp_sim *s, const sbp_grid_desc *d, const Layout &L, char *ws)
 {
     s->prec = d->precision;
@@ -422,10 +508,15 @@ int setup(sbp_sim *s, const sbp_grid_desc *d, const Layout &L, char *ws)
     s->grid = L.grid;
     s->npartials = L.npartials;
     s->fused_ok = L.fused;
+    s->one_pass = L.fused && ((d->precision == SBP_FP32 && (long long)(d->nx + 2) * (d->ny + 2) * (d->nz + 2) > kOnePassNodes) ||
+                              (d->flags & (SBP_FLAG_FDTD | SBP_FLAG_TEST_WAIT_TIMEOUT)));
+    if (const char *env = std::getenv("SBP_STEP_PATH"))   // tests compare the two paths
+        s->one_pass = L.fused && (s->one_pass || std::strcmp(env, "onepass") == 0);
     s->fused_kchunk = L.fused_kchunk;
     s->fused_rows = L.fused_rows;
     s->fused_width = L.fused_width;
     s->fused_grid = L.fused_grid;
+    if (int rc = choose_sweep(s)) return rc;
     char *p = ws;
     for (int set = 0; set < (L.fused ? 2 : 1); set++)
         for (int c = 0; c < 6; c++) { s->set[set][c] = p; p += L.field_bytes; }
@@ -575,52 +666,47 @@ int make_params(const sbp_sim *s, sbp::Params<T, S> &p, int eset, int hset)
     return SBP_OK;
 }
 
-template <typename T, typename S>
-int launch_h(const sbp_sim *s, bool energy, bool store)
+// A launch that may start while the kernel before it on the stream still runs
+// (it waits for that kernel before it touches a field).
+template <typename K, typename P>
+int launch_dependent(K kernel, cudaStream_t st, const P &p, const sbp::Sweep &w)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(w.ctas);
+    cfg.blockDim = dim3(sbp::kSweepThreads);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    SBP_CUDA(cudaLaunchKernelEx(&cfg, kernel, p, w));
+    return SBP_OK;
+}
+
+// One in-place half-step of the current set (h: H, else E).
+template <typename T, typename S, int V>
+int launch_half_t(const sbp_sim *s, bool h)
 {
     sbp::Params<T, S> p;
     int rc = make_params<T, S>(s, p, s->cur, s->cur);
     if (rc) return rc;
-    const dim3 block(sbp::kBlockX, sbp::kBlockY);
-    const bool muv = s->mu != nullptr;
-    if (!energy) {
-        if (muv) sbp::h_update<T, S, false, true, true><<<s->grid, block, 0, s->stream>>>(p);
-        else sbp::h_update<T, S, false, true, false><<<s->grid, block, 0, s->stream>>>(p);
-    } else if (store) {
-        if (muv) sbp::h_update<T, S, true, true, true><<<s->grid, block, 0, s->stream>>>(p);
-        else sbp::h_update<T, S, true, true, false><<<s->grid, block, 0, s->stream>>>(p);
-    } else {
-        if (muv) sbp::h_update<T, S, true, false, true><<<s->grid, block, 0, s->stream>>>(p);
-        else sbp::h_update<T, S, true, false, false><<<s->grid, block, 0, s->stream>>>(p);
-    }
-    SBP_CUDA(cudaGetLastError());
-    return SBP_OK;
+    const sbp::Sweep &w = s->sweep[h ? 0 : 1];
+    if (s->mu)
+        return h ? launch_dependent(sbp::half_h<T, S, true, V>, s->stream, p, w)
+                 : launch_dependent(sbp::half_e<T, S, true, V>, s->stream, p, w);
+    return h ? launch_dependent(sbp::half_h<T, S, false, V>, s->stream, p, w)
+             : launch_dependent(sbp::half_e<T, S, false, V>, s->stream, p, w);
 }
 
-template <typename T, typename S>
-int launch_e(const sbp_sim *s)
+int launch_half(const sbp_sim *s, bool h)
 {
-    sbp::Params<T, S> p;
-    int rc = make_params<T, S>(s, p, s->cur, s->cur);
-    if (rc) return rc;
-    const dim3 block(sbp::kBlockX, sbp::kBlockY);
-    if (s->mu) sbp::e_update<T, S, true><<<s->grid, block, 0, s->stream>>>(p);
-    else sbp::e_update<T, S, false><<<s->grid, block, 0, s->stream>>>(p);
-    SBP_CUDA(cudaGetLastError());
-    return SBP_OK;
-}
-
-int launch_h_any(const sbp_sim *s, bool energy, bool store)
-{
-    if (s->prec == SBP_FP64) return launch_h<double, double>(s, energy, store);
-    if (s->prec == SBP_FP32_FP16STORE) return launch_h<float, __half>(s, energy, store);
-    return launch_h<float, float>(s, energy, store);
-}
-int launch_e_any(const sbp_sim *s)
-{
-    if (s->prec == SBP_FP64) return launch_e<double, double>(s);
-    if (s->prec == SBP_FP32_FP16STORE) return launch_e<float, __half>(s);
-    return launch_e<float, float>(s);
+    const int v = s->sweep_v;
+    if (s->prec == SBP_FP64) return launch_half_t<double, double, 1>(s, h);
+    if (s->prec == SBP_FP32_FP16STORE)
+        return v > 1 ? launch_half_t<float, __half, 4>(s, h) : launch_half_t<float, __half, 1>(s, h);
+    return v == 4 ? launch_half_t<float, float, 4>(s, h)
+         : v == 2 ? launch_half_t<float, float, 2>(s, h) : launch_half_t<float, float, 1>(s, h);
 }
 
 // Parameters of the one-pass interior step reading set `old`, writing set old^1.
@@ -785,13 +871,6 @@ bool linked_to_other(const sbp_sim *s)
     return false;
 }
 
-int finalize_energy(const sbp_sim *s, double *dst)
-{
-    sbp::energy_finalize<<<1, 256, 0, s->stream>>>(s->partials, s->npartials, dst);
-    SBP_CUDA(cudaGetLastError());
-    return SBP_OK;
-}
-
 // Partial sums of sbp_energy_noalloc: a fixed array in this library, so that
 // call allocates nothing.  In host code the name is only a stand-in for the
 // symbol; its device address comes from cudaGetSymbolAddress, looked up when a
@@ -821,8 +900,8 @@ int energy_into_t(const sbp_sim *s, double *partials, double *dst)
     if (rc) return rc;
     p.partials = partials;
     const dim3 block(sbp::kBlockX, sbp::kBlockY);
-    if (s->mu) sbp::h_update<T, S, true, false, true><<<s->grid, block, 0, s->stream>>>(p);
-    else sbp::h_update<T, S, true, false, false><<<s->grid, block, 0, s->stream>>>(p);
+    if (s->mu) sbp::energy_sum<T, S, true><<<s->grid, block, 0, s->stream>>>(p);
+    else sbp::energy_sum<T, S, false><<<s->grid, block, 0, s->stream>>>(p);
     SBP_CUDA(cudaGetLastError());
     sbp::energy_finalize<<<1, 256, 0, s->stream>>>(partials, s->npartials, dst);
     SBP_CUDA(cudaGetLastError());
@@ -897,22 +976,25 @@ int check_group(sbp_sim **sims, int nsims)
     return SBP_OK;
 }
 
+// The energy monitor: W at the current step into the series when it is due.
+int sample_energy(sbp_sim *s)
+{
+    if (s->energy_every <= 0 || s->step % s->energy_every) return SBP_OK;
+    const long long idx = s->step / s->energy_every;
+    int rc = ensure_series(s, idx + 1);
+    if (rc) return rc;
+    rc = energy_into(s, s->partials, s->eseries + idx);
+    if (rc) return rc;
+    s->eseries_count = idx + 1;
+    return SBP_OK;
+}
+
 int half_h(sbp_sim **sims, int nsims)
 {
     for (int q = 0; q < nsims; q++) {
-        sbp_sim *s = sims[q];
-        const bool mon = s->energy_every > 0 && (s->step % s->energy_every) == 0;
-        if (mon) {
-            int rc = ensure_series(s, s->step / s->energy_every + 1);
-            if (rc) return rc;
-        }
-        int rc = launch_h_any(s, mon, true);
+        int rc = sample_energy(sims[q]);
+        if (!rc) rc = launch_half(sims[q], true);
         if (rc) return rc;
-        if (mon) {
-            rc = finalize_energy(s, s->eseries + s->step / s->energy_every);
-            if (rc) return rc;
-            s->eseries_count = s->step / s->energy_every + 1;
-        }
     }
     return SBP_OK;
 }
@@ -920,7 +1002,7 @@ int half_h(sbp_sim **sims, int nsims)
 int half_e(sbp_sim **sims, int nsims)
 {
     for (int q = 0; q < nsims; q++) {
-        int rc = launch_e_any(sims[q]);
+        int rc = launch_half(sims[q], false);
         if (rc) return rc;
     }
     for (int q = 0; q < nsims; q++) sims[q]->step++;
@@ -945,12 +1027,12 @@ int step_group(sbp_sim **sims, int nsims, int64_t nsteps)
         // decide each block's path first: interface partners read it
         for (int q = 0; q < nsims; q++) {
             sbp_sim *s = sims[q];
-            const bool mon = s->energy_every > 0 && (s->step % s->energy_every) == 0;
-            s->fused_step = s->fused_ok && !mon;
+            if ((rc = sample_energy(s))) return rc;
+            s->fused_step = s->one_pass;
         }
         for (int q = 0; q < nsims; q++) {
             sbp_sim *s = sims[q];
-            rc = s->fused_step ? launch_fused_phase1(s, !linked_to_other(s)) : half_h(&s, 1);
+            rc = s->fused_step ? launch_fused_phase1(s, !linked_to_other(s)) : launch_half(s, true);
             if (rc) return rc;
         }
         for (int q = 0; q < nsims; q++) {
@@ -960,7 +1042,7 @@ int step_group(sbp_sim **sims, int nsims, int64_t nsteps)
                 rc = launch_fused_phase2(s);
                 if (rc) return rc;
             } else {
-                rc = launch_e_any(s);
+                rc = launch_half(s, false);
                 if (rc) return rc;
             }
         }
@@ -974,8 +1056,8 @@ int step_group(sbp_sim **sims, int nsims, int64_t nsteps)
     return SBP_OK;
 }
 
-// sbp_step with CUDA events around every launch (kernel kinds: 0 h_update,
-// 1 e_update, 2 band_h, 3 fused_interior, 4 band_e).
+// sbp_step with CUDA events around every launch (kernel kinds: 0 h_update
+// (half_h), 1 e_update (half_e), 2 band_h, 3 fused_interior, 4 band_e).
 int step_timed(sbp_sim *s, int64_t nsteps, double *avg_ms, int64_t *launches, int n_out)
 {
     constexpr int kKinds = 5;
@@ -993,8 +1075,8 @@ int step_timed(sbp_sim *s, int64_t nsteps, double *avg_ms, int64_t *launches, in
     };
     int rc = SBP_OK;
     for (int64_t t = 0; t < nsteps && !rc; t++) {
-        const bool mon = s->energy_every > 0 && (s->step % s->energy_every) == 0;
-        s->fused_step = s->fused_ok && !mon && s->face[0] != SBP_INTERFACE && s->face[1] != SBP_INTERFACE &&
+        if ((rc = sample_energy(s))) break;
+        s->fused_step = s->one_pass && s->face[0] != SBP_INTERFACE && s->face[1] != SBP_INTERFACE &&
                         s->face[2] != SBP_INTERFACE && s->face[3] != SBP_INTERFACE && s->face[4] != SBP_INTERFACE &&
                         s->face[5] != SBP_INTERFACE;
         if (s->fused_step) {
@@ -1012,10 +1094,10 @@ int step_timed(sbp_sim *s, int64_t nsteps, double *avg_ms, int64_t *launches, in
             s->cur ^= 1;
         } else {
             if ((rc = mark(0))) break;
-            if ((rc = half_h(&s, 1))) break;
+            if ((rc = launch_half(s, true))) break;
             if ((rc = mark(-1))) break;
             if ((rc = mark(1))) break;
-            if ((rc = launch_e_any(s))) break;
+            if ((rc = launch_half(s, false))) break;
             if ((rc = mark(-1))) break;
         }
         s->fused_step = false;
@@ -1708,9 +1790,7 @@ int sbp_energy_group(sbp_sim **sims, int nsims, double *W)
         if (!s) return SBP_EINVAL;
         if (s->fdtd) return SBP_ESTATE;   // the energy of Eq. (16) is not the Yee scheme's
         DeviceGuard dg(s->device);
-        int rc = launch_h_any(s, true, false);
-        if (rc) return rc;
-        rc = finalize_energy(s, s->escalar);
+        int rc = energy_into(s, s->partials, s->escalar);
         if (rc) return rc;
         double v = 0.0;
         SBP_CUDA(cudaMemcpyAsync(&v, s->escalar, sizeof(double), cudaMemcpyDeviceToHost, s->stream));

@@ -179,7 +179,7 @@ def device_digest():
     """Digest of the device code (the two headers every kernel is compiled from)."""
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2206_00638_gb300", "csrc")
-    for f in ("kernels.cuh", "fused.cuh"):
+    for f in ("kernels.cuh", "fused.cuh", "halfstep.cuh"):
         with open(os.path.join(d, f), "rb") as fh:
             h.update(f.encode())
             h.update(fh.read())

@@ -228,11 +228,11 @@ int sbp_step_timed(sbp_sim *s, int64_t nsteps, double *avg_ms, int64_t *launches
  * stream.  A block joined to others by interface faces may be tuned: its
  * trial steps read the partners' current fields and write nothing of theirs.
  * Errors: SBP_EINVAL, SBP_ESTATE (the grid does not run the one-pass step),
- * SBP_ECUDA, SBP_ETIMEOUT.  A batch runs all its members on one tile, 64 columns wide:
- * 16 rows when every member has at least 20 cells along y and the batch steps
- * with three launches per step, else 8 (the environment variable
- * SBP_FUSED_ROWS=8 forces 8); a member's own tile is changed to it when the
- * batch is built. */
+ * SBP_ECUDA, SBP_ETIMEOUT.  Which grids step through the one-pass kernel is the
+ * library's choice (large FP32 grids); for the others, which step in place, the
+ * tile is kept but not used.  A persistent batch runs its members on tiles of 64
+ * columns by 8 rows; a member's own tile is changed to it when the batch is
+ * built. */
 int sbp_autotune(sbp_sim *s, int trial_steps, int *chosen_depth, double *ms_per_step);
 /* Tile of the one-pass step: H rows per CTA (8, 12 or 16), z-block depth
  * and H columns per CTA (64 or 128); each pointer may be NULL.  SBP_ESTATE if
@@ -240,8 +240,10 @@ int sbp_autotune(sbp_sim *s, int trial_steps, int *chosen_depth, double *ms_per_
 int sbp_tile(const sbp_sim *s, int *rows, int *depth, int *width);
 
 /* Batches: continuous batching of many simulations.  A batch advances all
- * its member simulations together, one kernel launch per kernel kind per
- * step covering every member (a tile table over the members), so many small
+ * its member simulations together.  Small members share launches, one per
+ * half-step for as many grids as stay in L2 together (a table of work lists over
+ * the grids); a member that fills the GPU by itself has its own.  A group runs a
+ * whole chunk of steps before the next group, so its fields stay in L2, and small
  * grids fill the GPU as one large launch.  Each member keeps its own fields,
  * sources, probes and step count and gives bit-identical results to
  * stepping it alone with sbp_step.  Members must be single-block FP32
@@ -257,9 +259,8 @@ int sbp_tile(const sbp_sim *s, int *rows, int *depth, int *width);
 typedef struct sbp_batch sbp_batch;
 /* flags: SBP_BATCH_GRAPHS records each chunk (sbp_batch_step call) as a CUDA
  * graph and replays it, updated in place when the membership changes.  By
- * default a chunk advances the members with three launches per step (the
- * one-pass kernel, band H and band E of every member, the band kernels on a
- * second stream).  SBP_BATCH_PERSISTENT runs the whole chunk as one
+ * default a chunk advances each group of members with two launches per step
+ * (the H and the E half-step, in place).  SBP_BATCH_PERSISTENT runs the whole chunk as one
  * persistent launch instead: CTAs that stay resident take (step, work item)
  * tickets in order; an item waits only for its own grid's previous step (and
  * band E for its grid's band H), so grids at different steps overlap.  It is

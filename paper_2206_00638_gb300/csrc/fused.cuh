@@ -29,8 +29,8 @@
 
 namespace sbp {
 
-constexpr int kFTX = 64;                 // H footprint width of the default tile and of batches
-constexpr int kFTY = 8;                  // H footprint rows of the default tile and of batches
+constexpr int kFTX = 64;                 // H footprint width of the default tile and of persistent batches
+constexpr int kFTY = 8;                  // H footprint rows of the default tile and of persistent batches
 #ifndef SBP_FUSED_STAGES
 #define SBP_FUSED_STAGES 4
 #endif
@@ -737,13 +737,9 @@ __global__ void __launch_bounds__(256, 4) band_e(const Params<T, S> p, const Ban
 }
 
 // ---------------------------------------------------------------------------
-// Batched step: one launch per kernel kind advances every grid of a batch
-// (continuous batching of many simulations).  A CTA finds its grid in a
-// prefix table of CTA counts; the grid's parameters and TMA maps live in
-// global memory; the step index comes from a device counter, so a captured
-// chunk of K steps can be replayed (the launches of a chunk carry offsets
-// 0..K-1 and batch_advance adds the steps taken).  Grids that reached their
-// target step skip their work, so a chunk may end a grid early.
+// A member of a batch that steps in one persistent launch: its parameters and
+// TMA maps live in global memory, the step index comes from a device counter.
+// A member that reached its target step skips its work.
 // ---------------------------------------------------------------------------
 struct BatchGrid {
     FusedMaps maps[2];            // TMA maps reading field set 0 / set 1
@@ -752,7 +748,7 @@ struct BatchGrid {
     Params<float> pe[2];          // band E: E of set c, H of set c^1
     float *hout[2][3], *eout[2][3];   // new-set outputs when the current set is c
     Band bh, be;
-    long long *counter;           // steps taken (device)
+    const long long *counter;     // steps taken (device)
     long long target;             // the grid stops when the counter reaches this
     long long cstart;             // counter value at which the current set was cur0
     long long probe_base;
@@ -777,48 +773,6 @@ __device__ __forceinline__ bool batch_state(const BatchGrid &g, int offset, long
     if (step >= g.target) return false;
     par = (g.cur0 + (int)((step - g.cstart) & 1)) & 1;
     return true;
-}
-
-// R: tile rows of every member's one-pass tiles (8, or 16 when every member
-// has a full 16-row tile).
-template <int R>
-__global__ void __launch_bounds__(R * 32, R >= 16 ? 1 : (kStages <= 3 ? 3 : 2))
-    fused_batched(const BatchGrid *G, const int *pre, int n, int offset)
-{
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int g = find_slot(pre, n, blockIdx.x);
-    const BatchGrid &B = G[g];
-    long long step;
-    int par;
-    if (!batch_state(B, offset, step, par)) return;
-    const int local = blockIdx.x - pre[g];
-    const int tx = B.tiles[0], ty = B.tiles[1];
-    fused_body<true, float, R>(B.maps[par], B.fp[par], step, step - B.probe_base, local % tx, (local / tx) % ty,
-                               local / (tx * ty), smem_raw);
-}
-
-__global__ void __launch_bounds__(256) band_h_batched(const BatchGrid *G, const int *pre, int n, int offset)
-{
-    const int g = find_slot(pre, n, blockIdx.x);
-    const BatchGrid &B = G[g];
-    long long step;
-    int par;
-    if (!batch_state(B, offset, step, par)) return;
-    const unsigned w = (unsigned)(blockIdx.x - pre[g]) * 8u + (threadIdx.x >> 5);
-    if (w >= B.bh.wz + B.bh.wy + B.bh.wx) return;
-    band_h_warp<float, false>(B.ph[par], B.bh, w, threadIdx.x & 31, step - B.probe_base, B.hout[par]);
-}
-
-__global__ void __launch_bounds__(256) band_e_batched(const BatchGrid *G, const int *pre, int n, int offset)
-{
-    const int g = find_slot(pre, n, blockIdx.x);
-    const BatchGrid &B = G[g];
-    long long step;
-    int par;
-    if (!batch_state(B, offset, step, par)) return;
-    const unsigned w = (unsigned)(blockIdx.x - pre[g]) * 8u + (threadIdx.x >> 5);
-    if (w >= B.be.wz + B.be.wy + B.be.wx) return;
-    band_e_warp<float, false>(B.pe[par], B.be, w, threadIdx.x & 31, step, step - B.probe_base, B.eout[par]);
 }
 
 // ---------------------------------------------------------------------------
@@ -940,14 +894,6 @@ __global__ void __launch_bounds__(kFTY * 32, kStages <= 3 ? 3 : 2)
             atomicAdd(&P.done[2 * g], 1u);
         }
     }
-}
-
-__global__ void batch_advance(const BatchGrid *G, int n, long long k)
-{
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n) return;
-    const long long c = *G[g].counter, t = G[g].target;
-    *G[g].counter = c + k < t ? c + k : (c < t ? t : c);
 }
 
 }  // namespace sbp

@@ -145,18 +145,21 @@ __device__ __forceinline__ unsigned long long rows_probe_mask(const Prb *prb, in
     return m;
 }
 
+// Step index and probe sample slot of a launch.
+struct When { long long step, slot; };
+
 template <int V, typename T, typename S>
-__device__ __forceinline__ void vec_probes(const Params<T, S> &p, unsigned long long m, int c0, int i0, int j, int k,
+__device__ __forceinline__ void vec_probes(const Params<T, S> &p, When t, unsigned long long m, int c0, int i0, int j, int k,
                                            const T (&a)[V], const T (&b)[V], const T (&c)[V])
 {
     for (; m; m &= m - 1) {
         const int q = __ffsll((long long)m) - 1;
         const Prb &P = p.prb[q];
-        if (P.j != j || P.k != k || p.probe_slot >= p.probe_cap) continue;
+        if (P.j != j || P.k != k || t.slot >= p.probe_cap) continue;
 #pragma unroll
         for (int e = 0; e < V; ++e)
             if (P.i == i0 + e)
-                p.probe_buf[(long long)q * p.probe_cap + p.probe_slot] =
+                p.probe_buf[(long long)q * p.probe_cap + t.slot] =
                     (P.comp == c0 ? a[e] : P.comp == c0 + 1 ? b[e] : c[e]) * p.fscale[c0 >= 3];
     }
 }
@@ -181,7 +184,7 @@ __device__ __forceinline__ VecPlace vec_place(const Sweep &w, unsigned cta, int 
 }
 
 template <typename T, typename S, bool MUVAR, int V>
-__device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, unsigned cta, int chunk)
+__device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, When when, unsigned cta, int chunk)
 {
     const VecPlace r = vec_place<V>(w, cta, chunk);
     if (r.k0 > r.k1) return;
@@ -239,7 +242,7 @@ __device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, uns
         stv<V>(Hx + o, hx, V);
         stv<V>(Hy + o, hy, V);
         stv<V>(Hz + o, hz, V);
-        if (pm) vec_probes<V>(p, pm, 3, r.i0, r.j, k, hx, hy, hz);
+        if (pm) vec_probes<V>(p, when, pm, 3, r.i0, r.j, k, hx, hy, hz);
 #pragma unroll
         for (int q = 0; q < V; ++q) {
             exm[q] = ex[q];
@@ -268,14 +271,14 @@ __device__ __forceinline__ void eps_pairs(const float *eps, long long o, long lo
 }
 
 template <typename T, typename S, int V>
-__device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, unsigned cta, int chunk)
+__device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, When when, unsigned cta, int chunk)
 {
     const VecPlace r = vec_place<V>(w, cta, chunk);
     if (r.k0 > r.k1) return;
     const int lane = threadIdx.x & 31;
     const unsigned long long pm =
         p.nprb ? rows_probe_mask(p.prb, p.nprb, 0, r.k0, r.k1, r.jmin, r.jmax, lane) : 0ull;
-    const double *const J = source_values(p, p.step, lane, r.k0, r.k1, r.jmin, r.jmax, 0, INT32_MAX);
+    const double *const J = source_values(p, when.step, lane, r.k0, r.k1, r.jmin, r.jmax, 0, INT32_MAX);
     if (!r.valid) return;
     const long long sy = p.sy, sz = p.sz;
     long long o = (long long)r.k0 * sz + (long long)r.j * sy + r.i0;
@@ -324,7 +327,7 @@ __device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, uns
         stv<V>(Ex + o, ex, V);
         stv<V>(Ey + o, ey, V);
         stv<V>(Ez + o, ez, V);
-        if (pm) vec_probes<V>(p, pm, 0, r.i0, r.j, k, ex, ey, ez);
+        if (pm) vec_probes<V>(p, when, pm, 0, r.i0, r.j, k, ex, ey, ez);
 #pragma unroll
         for (int q = 0; q < V; ++q) {
             hx[q] = hxn[q]; hy[q] = hyn[q];
@@ -445,7 +448,7 @@ __device__ __forceinline__ void rim_gather(const Params<T, S> &p, const RimAxis<
 // for every rim node: variants for the row ends and for the layers took a
 // quarter fewer instructions and 15 % more time, waiting for instruction fetch.
 template <typename T, typename S, bool ELECTRIC, bool MUVAR>
-__device__ __forceinline__ void rim_node(const Params<T, S> &p, int i, int j, int k, const double *J,
+__device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i, int j, int k, const double *J,
                                          unsigned long long pm)
 {
     constexpr int c0 = ELECTRIC ? 0 : 3;
@@ -482,14 +485,15 @@ __device__ __forceinline__ void rim_node(const Params<T, S> &p, int i, int j, in
     if (i <= nx + 1 - e && j <= ny + 1 - e && k <= nz + e) st_s(p.F[c0 + 2] + o, z);
     if (pm) {
         const T a[1] = {x}, b[1] = {y}, c[1] = {z};
-        vec_probes<1>(p, pm, c0, i, j, k, a, b, c);
+        vec_probes<1>(p, when, pm, c0, i, j, k, a, b, c);
     }
 }
 
 // Rim CTAs: the planes below and above the box first, then per z-chunk the y
 // layers and the row ends of its box planes.
 template <typename T, typename S, bool ELECTRIC, bool MUVAR>
-__device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w, unsigned cta, unsigned q, int chunk)
+__device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w, When when, unsigned cta, unsigned q,
+                                          int chunk)
 {
     unsigned t, count;
     int i, j, k;
@@ -526,10 +530,23 @@ __device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w,
         const int jmin = __reduce_min_sync(0xffffffffu, j), jmax = __reduce_max_sync(0xffffffffu, j);
         const int kmin = __reduce_min_sync(0xffffffffu, k), kmax = __reduce_max_sync(0xffffffffu, k);
         if (p.nprb) pm = rows_probe_mask(p.prb, p.nprb, ELECTRIC ? 0 : 3, kmin, kmax, jmin, jmax, lane);
-        if (ELECTRIC) J = source_values(p, p.step, lane, kmin, kmax, jmin, jmax, 0, INT32_MAX);
+        if (ELECTRIC) J = source_values(p, when.step, lane, kmin, kmax, jmin, jmax, 0, INT32_MAX);
     }
     if (t >= count) return;
-    rim_node<T, S, ELECTRIC, MUVAR>(p, i, j, k, J, pm);
+    rim_node<T, S, ELECTRIC, MUVAR>(p, when, i, j, k, J, pm);
+}
+
+// CTA `cta` of a half-step's work list.
+template <bool ELECTRIC, bool MUVAR, int V, typename T, typename S>
+__device__ __forceinline__ void half_cta(const Params<T, S> &p, const Sweep &w, When when, unsigned cta)
+{
+    const unsigned r = cta < w.cz ? 0u : cta - w.cz, chunk = r / w.dchunk, q = r - chunk * w.cchunk;
+    if (cta >= w.cz && q < w.cbox) {
+        if constexpr (ELECTRIC) box_e<T, S, V>(p, w, when, q, (int)chunk);
+        else box_h<T, S, MUVAR, V>(p, w, when, q, (int)chunk);
+    } else {
+        sweep_rim<T, S, ELECTRIC, MUVAR>(p, w, when, cta, q, (int)chunk);
+    }
 }
 
 template <typename T, typename S, bool MUVAR, int V>
@@ -537,10 +554,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 4 : 5)
     half_h(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
 {
     pdl_release();
-    const unsigned cta = blockIdx.x, r = cta < w.cz ? 0u : cta - w.cz;
-    const unsigned chunk = r / w.dchunk, q = r - chunk * w.cchunk;
-    if (cta >= w.cz && q < w.cbox) box_h<T, S, MUVAR, V>(p, w, q, (int)chunk);
-    else sweep_rim<T, S, false, MUVAR>(p, w, cta, q, (int)chunk);
+    half_cta<false, MUVAR, V>(p, w, {p.step, p.probe_slot}, blockIdx.x);
 }
 
 template <typename T, typename S, bool MUVAR, int V>
@@ -548,10 +562,76 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 4 : 5)
     half_e(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
 {
     pdl_release();
-    const unsigned cta = blockIdx.x, r = cta < w.cz ? 0u : cta - w.cz;
-    const unsigned chunk = r / w.dchunk, q = r - chunk * w.cchunk;
-    if (cta >= w.cz && q < w.cbox) box_e<T, S, V>(p, w, q, (int)chunk);
-    else sweep_rim<T, S, true, MUVAR>(p, w, cta, q, (int)chunk);
+    half_cta<true, MUVAR, V>(p, w, {p.step, p.probe_slot}, blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// Batched half-steps: one launch advances every grid of a group of a batch.  A
+// CTA finds its grid in a prefix table of CTA counts and copies the grid's
+// parameters to shared memory (one round trip, before it waits for the launch
+// before it); the step index comes from a device counter, so a captured chunk
+// of K steps can be replayed (its launches carry offsets 0..K-1, batch_advance
+// adds the steps taken).  Grids that reached their target step skip their work,
+// so a chunk may end a grid early.
+//
+// The grids of a batch are independent, so a chunk need not take every grid
+// through a step before the next: it takes a group of grids, as many as stay in
+// L2 together, through all its steps, then the next group.
+// ---------------------------------------------------------------------------
+struct alignas(16) BatchSweep : Sweep {};
+static_assert(sizeof(BatchSweep) % 16 == 0 && offsetof(Params<float>, link) % 16 == 0, "copied in 16-byte units");
+
+struct alignas(16) BatchHalf {
+    alignas(16) Params<float> p;  // the member's fields, in place (step and probe slot come from the counter)
+    BatchSweep w[2];              // work lists of H and E
+    const long long *counter;     // steps taken (device)
+    long long target;             // the grid stops when the counter reaches this
+    long long probe_base;
+};
+
+template <bool ELECTRIC, int V>
+__global__ void __launch_bounds__(kSweepThreads, V == 4 ? 5 : 7)
+    half_batched(const BatchHalf *grids, const int *pre, int n, int offset)
+{
+    __shared__ __align__(16) Params<float> p;
+    __shared__ BatchSweep w;
+    pdl_release();
+    // the tables and counters were written before the chunk's first launch, which
+    // waited for them whole: they can be read while the launch before runs
+    const int first = pre[0], g = find_slot(pre, n, (int)blockIdx.x + first);
+    const BatchHalf &B = grids[g];
+    auto copy = [](void *dst, const void *src, int bytes) {
+        for (int q = threadIdx.x; q < bytes / 16; q += kSweepThreads)
+            static_cast<uint4 *>(dst)[q] = __ldg(static_cast<const uint4 *>(src) + q);
+    };
+    copy(&p, &B.p, (int)offsetof(Params<float>, link) / 16 * 16);   // members have no links
+    copy(&w, &B.w[ELECTRIC], sizeof(w));
+    const long long step = *B.counter + offset;
+    if (step >= B.target) return;
+    __syncthreads();
+    half_cta<ELECTRIC, false, V>(p, w, {step, step - B.probe_base}, (unsigned)((int)blockIdx.x + first - pre[g]));
+}
+
+// One member of a batch alone: its parameters are the launch's, which cost a CTA
+// no copy (a grid that fills the GPU by itself steps 1.3 times faster so).
+template <bool ELECTRIC, int V>
+__global__ void __launch_bounds__(kSweepThreads, V == 4 ? 5 : 7)
+    half_member(const __grid_constant__ Params<float> p, const __grid_constant__ Sweep w, const long long *counter,
+                long long target, long long probe_base, int offset)
+{
+    pdl_release();
+    const long long step = *counter + offset;
+    if (step >= target) return;
+    half_cta<ELECTRIC, false, V>(p, w, {step, step - probe_base}, blockIdx.x);
+}
+
+// The members' step counters after a chunk of k steps.
+__global__ void batch_advance(long long *counters, const long long *targets, int n, long long k)
+{
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n) return;
+    const long long c = counters[g], t = targets[g];
+    counters[g] = c + k < t ? c + k : (c < t ? t : c);
 }
 
 }  // namespace sbp

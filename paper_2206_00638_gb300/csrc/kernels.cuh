@@ -74,32 +74,33 @@ template <typename S> using compute_t = typename Compute<S>::type;
 // T = float).  Stored FP16 values are field / scale, one scale for E and one
 // for H; the curl coefficients below carry the ratio of the two scales, so a
 // kernel only converts on load and store.
+// What every node needs comes first, the lists that few nodes look at after it.
 template <typename T, typename S = T>
 struct Params {
     S *F[6];                // padded fields Ex..Hz: element (i,j,k) at k*sz + j*sy + i
     const float *eps;       // ghost-padded cell eps_r on the same layout: cell (cx,cy,cz) at (cx+1,cy+1,cz+1)
     const float *mu;        // same for mu_r (only read when MUVAR)
-    int n[3];
     long long sy, sz;
+    int n[3];
     int face[6];
-    Link link[6];
     Coef<T> B[3];           // H: dt/(mu0 h_a) (uniform mu) or 2 dt/(mu0 h_a) (scaled by 1/sum2 mu_r)
     Coef<T> A[3];           // E: 4 dt/(eps0 h_a), scaled by 1/sum4 eps_r of the node
     Coef<T> AJ;             // 4 dt/eps0, source term
-    double dt, eta0, eps0, mu0;
-    double h[3];
-    int nsrc, nprb;
-    Src src[kMaxSources];
-    Prb prb[kMaxProbes];
     T fscale[2];                       // physical value = stored value * fscale[E=0 / H=1]
     T uB, uA;                          // fscale[H]/fscale[E] and its inverse: B and A carry the
                                        // scale ratio; the absorbing-SAT gamma needs them without
+    int nsrc, nprb;
     T *probe_buf;
     long long probe_cap, probe_slot;   // sample slot of this step (skip if >= cap)
     long long step;                    // n: the E half-step injects J(t^{n+1/2})
+    double dt, eta0, eps0, mu0;
+    double h[3];
     double *partials;                  // energy partial sums, one per CTA of energy_sum
     int kchunk;
     int fdtd;                          // 1: plain Yee FDTD comparator (band kernels only)
+    Src src[kMaxSources];
+    Prb prb[kMaxProbes];
+    Link link[6];
 };
 
 // ---------------------------------------------------------------------------

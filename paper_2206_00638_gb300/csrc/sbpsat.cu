@@ -760,8 +760,6 @@ int set_fused_smem_attr()
         SBP_FUSED_ATTR(__half, 8, 128);
         SBP_FUSED_ATTR(__half, 12, 128);
 #undef SBP_FUSED_ATTR
-        SBP_CUDA(cudaFuncSetAttribute(sbp::fused_batched<8>, attr, sbp::FusedGeom<float, 8>::kSmem));
-        SBP_CUDA(cudaFuncSetAttribute(sbp::fused_batched<16>, attr, sbp::FusedGeom<float, 16>::kSmem));
         SBP_CUDA(cudaFuncSetAttribute(sbp::persistent_batched, attr, sbp::kFusedSmem));
         done[dev] = true;
     }
@@ -1225,35 +1223,39 @@ int autotune(sbp_sim *s, int trials, int *chosen, double *best_ms)
 
 }  // namespace
 
-// A batch: many single-block FP32 simulations advanced together, one launch
-// per kernel kind per step for all of them (see BatchGrid in fused.cuh).
+// A batch: many single-block FP32 simulations advanced together (half_batched in
+// halfstep.cuh, or one persistent launch per chunk, fused.cuh).
 struct sbp_batch {
     struct Member {
         sbp_sim *s;
         long long target;        // absolute step index at which the member stops
         double *mirror;          // pinned host copy of the latest energy sample (serving), or null
     };
+    struct Group {                      // members that run a chunk together
+        int first, n, v;
+        unsigned ctas[2];
+        const sbp::BatchHalf *alone;    // the member (staging) when it runs by itself
+    };
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;  // private stream the graph is captured on (capture runs nothing)
-    cudaStream_t side = nullptr;        // band H -> band E beside the one-pass step
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int device = 0;
     std::vector<Member> m;
-    sbp::BatchGrid *d_grids = nullptr;
-    int *d_pre = nullptr;               // four prefix tables of cap+1 ints: fused, band H, band E CTAs,
-                                        // persistent-kernel items
-    long long *d_counters = nullptr;
+    std::vector<Group> groups;
+    sbp::BatchHalf *d_half = nullptr;   // members in group order
+    sbp::BatchGrid *d_grids = nullptr;  // members of a persistent batch
+    int *d_pre = nullptr;               // four prefix tables of cap+1 ints: CTAs of half-step H and E; persistent:
+                                        // fused, band H, band E CTAs and items
+    long long *d_counters = nullptr;    // steps taken, then targets (cap each)
     int cap = 0;
-    int nf = 0, nh = 0, ne = 0;         // CTAs per launch
-    int rows = sbp::kFTY;               // tile rows of the per-step one-pass launch (8 or 16)
     int ni = 0;                         // persistent-kernel items per step
-    sbp::BatchGrid *h_grids = nullptr;  // pinned staging of the uploads
+    sbp::BatchHalf *h_half = nullptr;   // pinned staging of the uploads
+    sbp::BatchGrid *h_grids = nullptr;
     int *h_pre = nullptr;
     long long *h_counters = nullptr;
     cudaEvent_t staged = nullptr;       // the last upload has left the staging buffers
     bool dirty = true;
     bool use_graph = true;
-    bool persistent = false;            // one persistent launch per chunk (else three launches per step)
+    bool persistent = false;            // one persistent launch per chunk (else two launches per group and step)
     unsigned *d_sched = nullptr;        // persistent kernel: ticket counter, 2 counters per member, error flag
     int *h_err = nullptr;               // pinned copy of the persistent kernel's error flag
     int resident = 0;                   // CTAs of the persistent kernel resident at once
@@ -1264,67 +1266,127 @@ struct sbp_batch {
 
 namespace {
 
+void batch_free_tables(sbp_batch *b)
+{
+    if (b->d_half) cudaFree(b->d_half);
+    if (b->d_grids) cudaFree(b->d_grids);
+    if (b->d_pre) cudaFree(b->d_pre);
+    if (b->d_counters) cudaFree(b->d_counters);
+    if (b->d_sched) cudaFree(b->d_sched);
+    if (b->h_half) cudaFreeHost(b->h_half);
+    if (b->h_grids) cudaFreeHost(b->h_grids);
+    if (b->h_pre) cudaFreeHost(b->h_pre);
+    if (b->h_counters) cudaFreeHost(b->h_counters);
+    b->d_half = nullptr; b->d_grids = nullptr; b->d_pre = nullptr; b->d_counters = nullptr; b->d_sched = nullptr;
+    b->h_half = nullptr; b->h_grids = nullptr; b->h_pre = nullptr; b->h_counters = nullptr;
+}
+
 int batch_reserve(sbp_batch *b, int n)
 {
     if (n <= b->cap) return SBP_OK;
     const int cap = std::max(n, 2 * b->cap + 4);
     SBP_CUDA(cudaStreamSynchronize(b->stream));
-    if (b->d_grids) cudaFree(b->d_grids);
-    if (b->d_pre) cudaFree(b->d_pre);
-    if (b->d_counters) cudaFree(b->d_counters);
-    if (b->h_grids) cudaFreeHost(b->h_grids);
-    if (b->h_pre) cudaFreeHost(b->h_pre);
-    if (b->h_counters) cudaFreeHost(b->h_counters);
-    b->d_grids = nullptr; b->d_pre = nullptr; b->d_counters = nullptr;
-    b->h_grids = nullptr; b->h_pre = nullptr; b->h_counters = nullptr;
-    SBP_CUDA(cudaMalloc(&b->d_grids, sizeof(sbp::BatchGrid) * cap));
+    batch_free_tables(b);
+    b->cap = 0;
+    const auto pinned = cudaHostAllocDefault;
+    if (b->persistent) {
+        SBP_CUDA(cudaMalloc(&b->d_grids, sizeof(sbp::BatchGrid) * cap));
+        SBP_CUDA(cudaHostAlloc((void **)&b->h_grids, sizeof(sbp::BatchGrid) * cap, pinned));
+        SBP_CUDA(cudaMalloc(&b->d_sched, sizeof(unsigned) * (2 * cap + 2)));
+        SBP_CUDA(cudaMemsetAsync(b->d_sched, 0, sizeof(unsigned) * (2 * cap + 2), b->stream));
+    } else {
+        SBP_CUDA(cudaMalloc(&b->d_half, sizeof(sbp::BatchHalf) * cap));
+        SBP_CUDA(cudaHostAlloc((void **)&b->h_half, sizeof(sbp::BatchHalf) * cap, pinned));
+    }
     SBP_CUDA(cudaMalloc(&b->d_pre, sizeof(int) * 4 * (cap + 1)));
-    SBP_CUDA(cudaMalloc(&b->d_counters, sizeof(long long) * cap));
-    if (b->d_sched) cudaFree(b->d_sched);
-    b->d_sched = nullptr;
-    SBP_CUDA(cudaMalloc(&b->d_sched, sizeof(unsigned) * (2 * cap + 2)));
-    SBP_CUDA(cudaMemsetAsync(b->d_sched, 0, sizeof(unsigned) * (2 * cap + 2), b->stream));
-    SBP_CUDA(cudaHostAlloc((void **)&b->h_grids, sizeof(sbp::BatchGrid) * cap, cudaHostAllocDefault));
-    SBP_CUDA(cudaHostAlloc((void **)&b->h_pre, sizeof(int) * 4 * (cap + 1), cudaHostAllocDefault));
-    SBP_CUDA(cudaHostAlloc((void **)&b->h_counters, sizeof(long long) * cap, cudaHostAllocDefault));
+    SBP_CUDA(cudaMalloc(&b->d_counters, sizeof(long long) * 2 * cap));
+    SBP_CUDA(cudaHostAlloc((void **)&b->h_pre, sizeof(int) * 4 * (cap + 1), pinned));
+    SBP_CUDA(cudaHostAlloc((void **)&b->h_counters, sizeof(long long) * 2 * cap, pinned));
     if (!b->staged) SBP_CUDA(cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming));
     b->cap = cap;
     if (b->gexec) { cudaGraphExecDestroy(b->gexec); b->gexec = nullptr; }
     return SBP_OK;
 }
 
-// Upload every member's parameters, prefix tables and step counters.
-constexpr int kBatchDepth = 64;   // z-planes per CTA of the batched one-pass step
+constexpr int kBatchDepth = 64;   // z-planes per CTA of a persistent batch's one-pass tiles
 
+// Bytes of fields and cells that a group of batch members holds in L2 while it
+// runs a chunk.  On this L2 (129 MB) a copy inside 64 MB moves 10.9 TB/s, inside
+// 96 MB 9.4 and inside 128 MB 7.5 (DRAM: 6.8).  24 grids of up to 192 cells per
+// axis, all batched: 80 MB 991 us per step, 60 MB 996, 110 MB 1020, 140 MB 1146,
+// one grid per group 1019.
+constexpr size_t kGroupBytes = 80u << 20;
+// A member of more bytes than this steps by itself: it fills the GPU, and its
+// parameters come with its launches.  The same 24 grids: 800 us per step (935
+// with the rule off); 48 grids of up to 96 cells 397 us, 418 with the line at
+// 8 MB and 471 with no batched launches; 32 of up to 64 cells 176, 176 and 245.
+constexpr size_t kAloneBytes = 24u << 20;
+
+// Members in group order: by vector width (a launch has one), then by size, as
+// many to a group as fit kGroupBytes.
+int batch_groups(sbp_batch *b)
+{
+    auto bytes = [](const sbp_sim *s) { return 7 * s->field_elems * sizeof(float); };
+    std::stable_sort(b->m.begin(), b->m.end(), [&](const sbp_batch::Member &x, const sbp_batch::Member &y) {
+        return x.s->sweep_v != y.s->sweep_v ? x.s->sweep_v < y.s->sweep_v : bytes(x.s) < bytes(y.s);
+    });
+    b->groups.clear();
+    size_t held = 0;
+    for (int g = 0; g < (int)b->m.size(); g++) {
+        const sbp_sim *s = b->m[g].s;
+        const bool alone = bytes(s) > kAloneBytes;
+        if (b->groups.empty() || b->groups.back().v != s->sweep_v || alone || b->groups.back().alone ||
+            held + bytes(s) > kGroupBytes) {
+            b->groups.push_back({g, 0, s->sweep_v, {0u, 0u}, alone ? b->h_half + g : nullptr});
+            held = 0;
+        }
+        sbp_batch::Group &G = b->groups.back();
+        held += bytes(s);
+        G.n++;
+        for (int h = 0; h < 2; h++) {
+            if ((long long)G.ctas[h] + s->sweep[h].ctas > INT32_MAX) return SBP_ECAPACITY;
+            G.ctas[h] += s->sweep[h].ctas;
+        }
+    }
+    return SBP_OK;
+}
+
+// Upload every member's parameters, prefix tables and step counters.
 int batch_rebuild(sbp_batch *b)
 {
     const int n = (int)b->m.size();
     int rc = batch_reserve(b, std::max(n, 1));
     if (rc) return rc;
+    if (!b->persistent && (rc = batch_groups(b))) return rc;
     // the previous upload must have left the pinned staging buffers
     SBP_CUDA(cudaEventSynchronize(b->staged));
-    sbp::BatchGrid *hg = b->h_grids;
     int *pre = b->h_pre;
     long long *cnt = b->h_counters;
     std::memset(pre, 0, sizeof(int) * 4 * (b->cap + 1));
     int *pf = pre, *ph = pre + (b->cap + 1), *pe = pre + 2 * (b->cap + 1), *pi = pre + 3 * (b->cap + 1);
-    // 16-row tiles (one 512-thread CTA per SM, which leaves room for the band
-    // kernels beside it) when every member has a full one, and the per-step
-    // path runs; else 8 rows (the persistent kernel always runs 8)
-    int rows = b->persistent ? sbp::kFTY : 16;
-    if (const char *env = std::getenv("SBP_FUSED_ROWS"))
-        if (std::atoi(env) == 8) rows = sbp::kFTY;
-    for (int g = 0; g < n; g++)
-        if (b->m[g].s->n[1] - 5 < 15) rows = sbp::kFTY;
-    b->rows = rows;
     for (int g = 0; g < n; g++) {
         sbp_sim *s = b->m[g].s;
-        sbp::BatchGrid &G = hg[g];
+        cnt[g] = s->step;
+        cnt[b->cap + g] = b->m[g].target;
+        if (!b->persistent) {
+            sbp::BatchHalf &H = b->h_half[g];
+            if ((rc = make_params<float>(s, H.p, s->cur, s->cur))) return rc;
+            for (int h = 0; h < 2; h++) static_cast<sbp::Sweep &>(H.w[h]) = s->sweep[h];
+            H.counter = b->d_counters + g;
+            H.target = b->m[g].target;
+            H.probe_base = s->probe_base;
+            const long long nh = (long long)pf[g] + s->sweep[0].ctas, ne = (long long)ph[g] + s->sweep[1].ctas;
+            if (nh > INT32_MAX || ne > INT32_MAX) return SBP_ECAPACITY;
+            pf[g + 1] = (int)nh;
+            ph[g + 1] = (int)ne;
+            continue;
+        }
+        sbp::BatchGrid &G = b->h_grids[g];
         std::memset(static_cast<void *>(&G), 0, sizeof(G));
-        // every member runs the batch's tile: 64 columns and the batch's height
-        // (its TMA boxes are re-encoded when that differs from the member's own)
-        if ((s->fused_rows != rows || s->fused_width != sbp::kFTX) &&
-            (rc = set_tile(s, sbp::kFTX, rows, s->fused_kchunk)))
+        // every member runs the persistent kernel's tile (its TMA boxes are
+        // re-encoded when that differs from the member's own)
+        if ((s->fused_rows != sbp::kFTY || s->fused_width != sbp::kFTX) &&
+            (rc = set_tile(s, sbp::kFTX, sbp::kFTY, s->fused_kchunk)))
             return rc;
         for (int c = 0; c < 2; c++) {
             G.maps[c] = s->maps[c];
@@ -1350,7 +1412,6 @@ int batch_rebuild(sbp_batch *b)
         G.fp[0].kchunk = G.fp[1].kchunk = depth;
         G.tiles[0] = s->fused_grid.x; G.tiles[1] = s->fused_grid.y;
         G.tiles[2] = (s->n[2] - 5 + depth - 1) / depth;
-        cnt[g] = s->step;
         const long long nfg = (long long)G.tiles[0] * G.tiles[1] * G.tiles[2];
         const long long nhg = G.bh.ctas;
         const long long neg = G.be.ctas;
@@ -1361,12 +1422,15 @@ int batch_rebuild(sbp_batch *b)
         pe[g + 1] = pe[g] + (int)neg;
         pi[g + 1] = pi[g] + sbp::band_items((int)nhg) + (int)nfg + sbp::band_items((int)neg);
     }
-    b->nf = pf[n]; b->nh = ph[n]; b->ne = pe[n]; b->ni = pi[n];
+    b->ni = pi[n];
     if (n > 0) {
         // stream-ordered behind the chunks already queued, which read the old tables
-        SBP_CUDA(cudaMemcpyAsync(b->d_grids, hg, sizeof(sbp::BatchGrid) * n, cudaMemcpyHostToDevice, b->stream));
+        if (b->persistent)
+            SBP_CUDA(cudaMemcpyAsync(b->d_grids, b->h_grids, sizeof(sbp::BatchGrid) * n, cudaMemcpyHostToDevice, b->stream));
+        else
+            SBP_CUDA(cudaMemcpyAsync(b->d_half, b->h_half, sizeof(sbp::BatchHalf) * n, cudaMemcpyHostToDevice, b->stream));
         SBP_CUDA(cudaMemcpyAsync(b->d_pre, pre, sizeof(int) * 4 * (b->cap + 1), cudaMemcpyHostToDevice, b->stream));
-        SBP_CUDA(cudaMemcpyAsync(b->d_counters, cnt, sizeof(long long) * n, cudaMemcpyHostToDevice, b->stream));
+        SBP_CUDA(cudaMemcpyAsync(b->d_counters, cnt, sizeof(long long) * 2 * b->cap, cudaMemcpyHostToDevice, b->stream));
         SBP_CUDA(cudaEventRecord(b->staged, b->stream));
     }
     b->gstale = true;                   // the graph is re-recorded and updated in place at the next chunk
@@ -1374,11 +1438,38 @@ int batch_rebuild(sbp_batch *b)
     return SBP_OK;
 }
 
+// One half-step of a group at offset `offset` of a chunk.  first: the chunk's
+// first launch, which waits for everything before it (tables and counters); the
+// others may start while the launch before still runs.
+template <bool ELECTRIC, int V>
+int launch_half_batched(const sbp_batch *b, const sbp_batch::Group &G, int offset, bool first)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G.ctas[ELECTRIC]);
+    cfg.blockDim = dim3(sbp::kSweepThreads);
+    cfg.stream = b->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = first ? 0 : 1;
+    if (G.alone) {
+        const sbp::BatchHalf &H = G.alone[0];
+        SBP_CUDA(cudaLaunchKernelEx(&cfg, sbp::half_member<ELECTRIC, V>, H.p,
+                                    static_cast<const sbp::Sweep &>(H.w[ELECTRIC]), H.counter, H.target, H.probe_base,
+                                    offset));
+        return SBP_OK;
+    }
+    const sbp::BatchHalf *grids = b->d_half + G.first;
+    const int *pre = b->d_pre + (ELECTRIC ? b->cap + 1 : 0) + G.first;
+    SBP_CUDA(cudaLaunchKernelEx(&cfg, sbp::half_batched<ELECTRIC, V>, grids, pre, G.n, offset));
+    return SBP_OK;
+}
+
 // K steps of every member: offsets 0..K-1, then the counters advance by K.
 int batch_launch_chunk(sbp_batch *b, long long K)
 {
     const int n = (int)b->m.size();
-    const int *pf = b->d_pre, *ph = b->d_pre + (b->cap + 1), *pe = b->d_pre + 2 * (b->cap + 1);
     if (b->persistent) {
         // one launch for the whole chunk: CTAs take (step, item) tickets in
         // order, items wait only for their own grid's previous step (see
@@ -1402,25 +1493,21 @@ int batch_launch_chunk(sbp_batch *b, long long K)
             SBP_CUDA(cudaGetLastError());
         }
     } else {
-        // per step: the one-pass interior step on the batch stream, band H then
-        // band E beside it on the side stream (band E reads only band H's output,
-        // which includes the first interior H layer), joined before the next step
-        for (long long o = 0; o < K; o++) {
-            SBP_CUDA(cudaEventRecord(b->ev_fork, b->stream));
-            if (b->nf > 0 && b->rows == 16)
-                sbp::fused_batched<16><<<b->nf, 16 * 32, sbp::FusedGeom<float, 16>::kSmem, b->stream>>>(
-                    b->d_grids, pf, n, (int)o);
-            else if (b->nf > 0)
-                sbp::fused_batched<8><<<b->nf, 8 * 32, sbp::FusedGeom<float, 8>::kSmem, b->stream>>>(
-                    b->d_grids, pf, n, (int)o);
-            SBP_CUDA(cudaStreamWaitEvent(b->side, b->ev_fork, 0));
-            if (b->nh > 0) sbp::band_h_batched<<<b->nh, 256, 0, b->side>>>(b->d_grids, ph, n, (int)o);
-            if (b->ne > 0) sbp::band_e_batched<<<b->ne, 256, 0, b->side>>>(b->d_grids, pe, n, (int)o);
-            SBP_CUDA(cudaEventRecord(b->ev_join, b->side));
-            SBP_CUDA(cudaStreamWaitEvent(b->stream, b->ev_join, 0));
-        }
+        // group by group, each through all K steps: its fields stay in L2
+        for (const sbp_batch::Group &G : b->groups)
+            for (long long o = 0; o < K; o++) {
+                const bool first = G.first == 0 && o == 0;
+                int rc = G.v == 1   ? launch_half_batched<false, 1>(b, G, (int)o, first)
+                         : G.v == 2 ? launch_half_batched<false, 2>(b, G, (int)o, first)
+                                    : launch_half_batched<false, 4>(b, G, (int)o, first);
+                if (!rc)
+                    rc = G.v == 1   ? launch_half_batched<true, 1>(b, G, (int)o, false)
+                         : G.v == 2 ? launch_half_batched<true, 2>(b, G, (int)o, false)
+                                    : launch_half_batched<true, 4>(b, G, (int)o, false);
+                if (rc) return rc;
+            }
     }
-    sbp::batch_advance<<<(n + 127) / 128, 128, 0, b->stream>>>(b->d_grids, n, K);
+    sbp::batch_advance<<<(n + 127) / 128, 128, 0, b->stream>>>(b->d_counters, b->d_counters + b->cap, n, K);
     SBP_CUDA(cudaGetLastError());
     return SBP_OK;
 }
@@ -1986,15 +2073,8 @@ int sbp_batch_create(void *cuda_stream, int flags, sbp_batch **out)
     }
     *b->h_err = 0;
     b->resident = std::max(1, per_sm * sms);
-    if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+    if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
         (void)cudaGetLastError();
-        if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-        if (b->side) cudaStreamDestroy(b->side);
-        if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-        if (b->ev_join) cudaEventDestroy(b->ev_join);
         delete b;
         return SBP_ECUDA;
     }
@@ -2108,7 +2188,7 @@ int sbp_batch_step(sbp_batch *b, int64_t nsteps)
     for (auto &m : b->m) {
         const long long done = std::min<long long>(nsteps, std::max<long long>(0, m.target - m.s->step));
         m.s->step += done;
-        m.s->cur ^= (int)(done & 1);
+        if (b->persistent) m.s->cur ^= (int)(done & 1);
         if (done > 0 && (rc = batch_sample_energy(b, m))) return rc;
     }
     return SBP_OK;
@@ -2123,16 +2203,7 @@ int sbp_batch_destroy(sbp_batch *b)
     cudaStreamSynchronize(b->stream);
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-    if (b->side) cudaStreamDestroy(b->side);
-    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-    if (b->ev_join) cudaEventDestroy(b->ev_join);
-    if (b->d_grids) cudaFree(b->d_grids);
-    if (b->d_pre) cudaFree(b->d_pre);
-    if (b->d_counters) cudaFree(b->d_counters);
-    if (b->h_grids) cudaFreeHost(b->h_grids);
-    if (b->h_pre) cudaFreeHost(b->h_pre);
-    if (b->h_counters) cudaFreeHost(b->h_counters);
-    if (b->d_sched) cudaFree(b->d_sched);
+    batch_free_tables(b);
     if (b->h_err) cudaFreeHost(b->h_err);
     if (b->staged) cudaEventDestroy(b->staged);
     delete b;

@@ -429,14 +429,14 @@ def from_workload(w, precision=FP32, stream=None, torch_memory=True, energy_ever
 
 
 class Batch:
-    """Continuous batching of many simulations: one launch per kernel kind per step covers every
-    member (wraps ``sbp_batch``).  Members must be created on the batch's stream."""
+    """Continuous batching of many simulations (wraps ``sbp_batch``): small members share launches,
+    groups that fit L2 run a chunk one after another.  Members must be created on the batch's stream."""
 
     GRAPHS, PERSISTENT = 1, 2
 
     def __init__(self, stream=None, use_graphs=True, persistent=False):
         """use_graphs: replay each chunk as a CUDA graph; persistent: one persistent launch per
-        chunk instead of three launches per step."""
+        chunk instead of two launches per group of members and step."""
         self.stream = _stream_ptr(stream)
         h = C.c_void_p()
         flags = (self.GRAPHS if use_graphs else 0) | (self.PERSISTENT if persistent else 0)

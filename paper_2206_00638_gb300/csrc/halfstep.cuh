@@ -27,6 +27,14 @@ namespace sbp {
 
 constexpr int kSweepThreads = 128;        // threads of a CTA
 
+// CTAs of a half-step that fit an SM, by registers: 72 a thread in FP32 (76-80 left
+// to the compiler cost 8 % at 117 x 96 x 131), 96 for E in vectors of 4, 112 and
+// more in FP64.
+template <typename T, int V> constexpr int half_ctas(bool electric)
+{
+    return sizeof(T) == 8 ? 4 : V == 4 && electric ? 5 : 7;
+}
+
 // n / d for n < 2^31, with the multiplier of d found on the host.
 struct FastDiv { unsigned mul, shift; };
 __device__ __forceinline__ unsigned operator/(unsigned n, const FastDiv &d) { return (__umulhi(n, d.mul) + n) >> d.shift; }
@@ -72,27 +80,22 @@ __device__ __forceinline__ void ldv(const S *p, compute_t<S> (&v)[V])
         }
     }
 }
-// Store v (already rounded to the storage type), or its first `count` elements.
+// Store v (already rounded to the storage type).
 template <int V, typename S, typename T>
-__device__ __forceinline__ void stv(S *p, const T (&v)[V], int count)
+__device__ __forceinline__ void stv(S *p, const T (&v)[V])
 {
-    constexpr int bytes = V * (int)sizeof(S);
-    if constexpr (V > 1) {
-        if (count >= V) {
-            using W = typename std::conditional<bytes == 16, uint4, uint2>::type;
-            union { W w; S s[V]; } u;
+    if constexpr (V == 1) {
+        st_s(p, v[0]);
+    } else {
+        using W = typename std::conditional<V * sizeof(S) == 16, uint4, uint2>::type;
+        union { W w; S s[V]; } u;
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                if constexpr (std::is_same<S, __half>::value) u.s[q] = __float2half_rn(v[q]);
-                else u.s[q] = v[q];
-            }
-            *reinterpret_cast<W *>(p) = u.w;
-            return;
+        for (int q = 0; q < V; ++q) {
+            if constexpr (std::is_same<S, __half>::value) u.s[q] = __float2half_rn(v[q]);
+            else u.s[q] = v[q];
         }
+        *reinterpret_cast<W *>(p) = u.w;
     }
-#pragma unroll
-    for (int q = 0; q < V; ++q)
-        if (q < count) st_s(p + q, v[q]);
 }
 // Cell values (FP32) in the arithmetic type.
 template <int V, typename T>
@@ -127,26 +130,45 @@ __device__ __forceinline__ T advance_plain(T old, const Coef<T> &c0, T d0, const
     }
 }
 
-// Probes of components c0..c0+2 near a warp's rows and planes (bit per probe);
-// every lane of the warp calls it.
-__device__ __forceinline__ unsigned long long rows_probe_mask(const Prb *prb, int nprb, int c0, int k0, int k1, int j0,
-                                                              int j1, int lane)
-{
-    unsigned long long m = 0ull;
-    for (int q0 = 0; q0 < nprb; q0 += 32) {
-        const int q = q0 + lane;
-        bool hit = false;
-        if (q < nprb) {
-            const Prb P = prb[q];
-            hit = P.comp >= c0 && P.comp <= c0 + 2 && P.k >= k0 && P.k <= k1 && P.j >= j0 && P.j <= j1;
-        }
-        m |= (unsigned long long)__ballot_sync(0xffffffffu, hit) << q0;
-    }
-    return m;
-}
-
 // Step index and probe sample slot of a launch.
 struct When { long long step, slot; };
+
+// Sources and probes that some node of a warp may hold: source values (null for
+// none) and a bit per probe.
+struct Marks { const double *J; unsigned long long pm; };
+
+__device__ __forceinline__ bool meets(const int (&box)[6], int i0, int i1, int j, int k0, int k1)
+{
+    return i0 <= box[3] && i1 >= box[0] && j <= box[4] && j >= box[1] && k0 <= box[5] && k1 >= box[2];
+}
+
+// The marks of a warp whose lanes hold nodes i0..i1 of row j in planes k0..k1.
+// Nearly every warp is done after the test against the index boxes around all
+// probes and all sources.  Every lane of the warp calls it.
+template <bool ELECTRIC, typename T, typename S>
+__device__ __forceinline__ Marks find_marks(const Params<T, S> &p, When when, int i0, int i1, int j, int k0, int k1)
+{
+    Marks r = {nullptr, 0ull};
+    const bool near_p = meets(p.pbox[ELECTRIC ? 0 : 1], i0, i1, j, k0, k1);
+    const bool near_s = ELECTRIC && meets(p.sbox, i0, i1, j, k0, k1);
+    if (!__any_sync(0xffffffffu, near_p || near_s)) return r;
+    constexpr int c0 = ELECTRIC ? 0 : 3;
+    const int lane = threadIdx.x & 31;
+    const int ja = __reduce_min_sync(0xffffffffu, j), jb = __reduce_max_sync(0xffffffffu, j);
+    k0 = __reduce_min_sync(0xffffffffu, k0);
+    k1 = __reduce_max_sync(0xffffffffu, k1);
+    for (int q0 = 0; q0 < p.nprb; q0 += 32) {
+        const int q = q0 + lane;
+        bool hit = false;
+        if (q < p.nprb) {
+            const Prb P = p.prb[q];
+            hit = P.comp >= c0 && P.comp <= c0 + 2 && P.k >= k0 && P.k <= k1 && P.j >= ja && P.j <= jb;
+        }
+        r.pm |= (unsigned long long)__ballot_sync(0xffffffffu, hit) << q0;
+    }
+    if (ELECTRIC) r.J = source_values(p, when.step, lane, k0, k1, ja, jb, 0, INT32_MAX);
+    return r;
+}
 
 template <int V, typename T, typename S>
 __device__ __forceinline__ void vec_probes(const Params<T, S> &p, When t, unsigned long long m, int c0, int i0, int j, int k,
@@ -164,8 +186,8 @@ __device__ __forceinline__ void vec_probes(const Params<T, S> &p, When t, unsign
     }
 }
 
-// First x, row and plane range of a box thread, and the rows of its warp.
-struct VecPlace { int i0, j, jmin, jmax, k0, k1; bool valid; };
+// First x, row and plane range of a box thread.
+struct VecPlace { int i0, j, k0, k1; bool valid; };
 
 template <int V>
 __device__ __forceinline__ VecPlace vec_place(const Sweep &w, unsigned cta, int chunk)
@@ -176,46 +198,50 @@ __device__ __forceinline__ VecPlace vec_place(const Sweep &w, unsigned cta, int 
     const unsigned tc = min(t, w.vecs - 1u), row = tc / w.dnv;
     r.j = w.lo[1] + (int)row;
     r.i0 = w.lo[0] + V * (int)(tc - row * w.nv);
-    r.jmin = __shfl_sync(0xffffffffu, r.j, 0);
-    r.jmax = __shfl_sync(0xffffffffu, r.j, 31);
     r.k0 = max(chunk * w.kz, w.lo[2]);
     r.k1 = min(chunk * w.kz + w.kz - 1, w.hi[2]);
     return r;
 }
 
-template <typename T, typename S, bool MUVAR, int V>
+// I: the type of an element index (unsigned, or long long for arrays of 2^32
+// elements and more; unsigned sums wrap, so offsets may be negative).  One
+// 32-bit addition and one widening multiply-add make an address, where 64-bit
+// sums take twice that, and the half-steps of grids that stay in L2 are bound by
+// their instructions.
+template <typename I, typename T, typename S, bool MUVAR, int V>
 __device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, When when, unsigned cta, int chunk)
 {
     const VecPlace r = vec_place<V>(w, cta, chunk);
     if (r.k0 > r.k1) return;
-    const unsigned long long pm =
-        p.nprb ? rows_probe_mask(p.prb, p.nprb, 3, r.k0, r.k1, r.jmin, r.jmax, threadIdx.x & 31) : 0ull;
+    const unsigned long long pm = find_marks<false>(p, when, r.i0, r.i0 + V - 1, r.j, r.k0, r.k1).pm;
     if (!r.valid) return;
-    const long long sy = p.sy, sz = p.sz;
-    long long o = (long long)r.k0 * sz + (long long)r.j * sy + r.i0;
+    const I sy = (I)p.sy, sz = (I)p.sz;
+    I o = (I)r.k0 * sz + (I)r.j * sy + (I)r.i0;
     const S *const Ex = p.F[0], *const Ey = p.F[1], *const Ez = p.F[2];
     S *const Hx = p.F[3], *const Hy = p.F[4], *const Hz = p.F[5];
     const Coef<T> Bx = p.B[0], By = p.B[1], Bz = p.B[2];
     pdl_wait();
     T exm[V], eym[V], m0[V];
-    ldv<V>(Ex + o - sz, exm);
-    ldv<V>(Ey + o - sz, eym);
+    ldv<V>(Ex + (I)(o - sz), exm);
+    ldv<V>(Ey + (I)(o - sz), eym);
     if constexpr (MUVAR) ldcells<V>(p.mu + o, m0);
     for (int k = r.k0; k <= r.k1; ++k, o += sz) {
         T ex[V], ey[V], ez[V], exj[V], ezj[V], hx[V], hy[V], hz[V];
+        const S *const pey = Ey + o, *const pez = Ez + o;
+        const I oj = o - sy;
         ldv<V>(Ex + o, ex);
-        ldv<V>(Ey + o, ey);
-        ldv<V>(Ez + o, ez);
-        ldv<V>(Ex + o - sy, exj);
-        ldv<V>(Ez + o - sy, ezj);
-        const T eyl = ld_s(Ey + o - 1), ezl = ld_s(Ez + o - 1);
+        ldv<V>(pey, ey);
+        ldv<V>(pez, ez);
+        ldv<V>(Ex + oj, exj);
+        ldv<V>(Ez + oj, ezj);
+        const T eyl = ld_s(pey - 1), ezl = ld_s(pez - 1);
         ldv<V>(Hx + o, hx);
         ldv<V>(Hy + o, hy);
         ldv<V>(Hz + o, hz);
         T mj[V], mk[V], mr = T(0);
         if constexpr (MUVAR) {
-            ldcells<V>(p.mu + o + sy, mj);
-            ldcells<V>(p.mu + o + sz, mk);
+            ldcells<V>(p.mu + (I)(o + sy), mj);
+            ldcells<V>(p.mu + (I)(o + sz), mk);
             mr = widen<T>(__ldg(p.mu + o + V));
         }
 #pragma unroll
@@ -239,9 +265,9 @@ __device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, Whe
                 hz[q] = quant<S>(advance_plain<S>(hz[q], By, d4, Bx, d5));
             }
         }
-        stv<V>(Hx + o, hx, V);
-        stv<V>(Hy + o, hy, V);
-        stv<V>(Hz + o, hz, V);
+        stv<V>(Hx + o, hx);
+        stv<V>(Hy + o, hy);
+        stv<V>(Hz + o, hz);
         if (pm) vec_probes<V>(p, when, pm, 3, r.i0, r.j, k, hx, hy, hz);
 #pragma unroll
         for (int q = 0; q < V; ++q) {
@@ -254,13 +280,14 @@ __device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, Whe
 
 // Pair sums of the eps cells (j, j+1; i, i+1) of one plane, from which the node
 // sums of cell_sum are built in its association.
-template <int V, typename T>
-__device__ __forceinline__ void eps_pairs(const float *eps, long long o, long long sy, T (&a)[V], T (&b)[V], T (&c)[V])
+template <int V, typename I, typename T>
+__device__ __forceinline__ void eps_pairs(const float *eps, I o, I sy, T (&a)[V], T (&b)[V], T (&c)[V])
 {
     T f[V], g[V];
-    ldcells<V>(eps + o, f);
-    ldcells<V>(eps + o + sy, g);
-    const T fr = widen<T>(__ldg(eps + o + V)), gr = widen<T>(__ldg(eps + o + sy + V));
+    const float *const pf = eps + o, *const pg = eps + (I)(o + sy);
+    ldcells<V>(pf, f);
+    ldcells<V>(pg, g);
+    const T fr = widen<T>(__ldg(pf + V)), gr = widen<T>(__ldg(pg + V));
 #pragma unroll
     for (int q = 0; q < V; ++q) {
         const int n = q + 1 < V ? q + 1 : q;
@@ -270,18 +297,34 @@ __device__ __forceinline__ void eps_pairs(const float *eps, long long o, long lo
     }
 }
 
-template <typename T, typename S, int V>
+// The current density of the warp's sources on V nodes of the three components.
+template <int V, typename T, typename S, typename A>
+__device__ __forceinline__ void vec_sources(const Params<T, S> &p, const double *J, int i0, int j, int k, A (&a)[V],
+                                            A (&b)[V], A (&c)[V])
+{
+    for (int s = 0; s < p.nsrc; ++s) {
+        const Src &P = p.src[s];
+        if ((P.k >= 0 && P.k != k) || (P.j >= 0 && P.j != j)) continue;
+        const T v = T(J[s]);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            if (P.i >= 0 && P.i != i0 + q) continue;
+            if (P.comp == 0) a[q].add(p.AJ, v, T(-1));
+            else if (P.comp == 1) b[q].add(p.AJ, v, T(-1));
+            else c[q].add(p.AJ, v, T(-1));
+        }
+    }
+}
+
+template <typename I, typename T, typename S, int V>
 __device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, When when, unsigned cta, int chunk)
 {
     const VecPlace r = vec_place<V>(w, cta, chunk);
     if (r.k0 > r.k1) return;
-    const int lane = threadIdx.x & 31;
-    const unsigned long long pm =
-        p.nprb ? rows_probe_mask(p.prb, p.nprb, 0, r.k0, r.k1, r.jmin, r.jmax, lane) : 0ull;
-    const double *const J = source_values(p, when.step, lane, r.k0, r.k1, r.jmin, r.jmax, 0, INT32_MAX);
+    const Marks marks = find_marks<true>(p, when, r.i0, r.i0 + V - 1, r.j, r.k0, r.k1);
     if (!r.valid) return;
-    const long long sy = p.sy, sz = p.sz;
-    long long o = (long long)r.k0 * sz + (long long)r.j * sy + r.i0;
+    const I sy = (I)p.sy, sz = (I)p.sz;
+    I o = (I)r.k0 * sz + (I)r.j * sy + (I)r.i0;
     S *const Ex = p.F[0], *const Ey = p.F[1], *const Ez = p.F[2];
     const S *const Hx = p.F[3], *const Hy = p.F[4], *const Hz = p.F[5];
     const Coef<T> Ax = p.A[0], Ay = p.A[1], Az = p.A[2];
@@ -291,69 +334,68 @@ __device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, Whe
     T hx[V], hy[V];
     ldv<V>(Hx + o, hx);
     ldv<V>(Hy + o, hy);
+    T hyr = ld_s(Hy + o + V);
     for (int k = r.k0; k <= r.k1; ++k, o += sz) {
         T hxn[V], hyn[V], hz[V], hzj[V], hxj[V], ex[V], ey[V], ez[V], na[V], nb[V], nc[V];
-        ldv<V>(Hx + o + sz, hxn);
-        ldv<V>(Hy + o + sz, hyn);
-        ldv<V>(Hz + o, hz);
-        ldv<V>(Hz + o + sy, hzj);
-        ldv<V>(Hx + o + sy, hxj);
-        const T hyr = ld_s(Hy + o + V), hzr = ld_s(Hz + o + V);
+        const I oz = o + sz, oj = o + sy;
+        const S *const phy = Hy + oz, *const phz = Hz + o;
+        ldv<V>(Hx + oz, hxn);
+        ldv<V>(phy, hyn);
+        const T hyrn = ld_s(phy + V), hzr = ld_s(phz + V);
+        ldv<V>(phz, hz);
+        ldv<V>(Hz + oj, hzj);
+        ldv<V>(Hx + oj, hxj);
         ldv<V>(Ex + o, ex);
         ldv<V>(Ey + o, ey);
         ldv<V>(Ez + o, ez);
-        eps_pairs<V>(p.eps, o + sz, sy, na, nb, nc);
+        eps_pairs<V>(p.eps, oz, sy, na, nb, nc);
+        typename AccOf<T, S>::type a[V], b[V], c[V];
 #pragma unroll
         for (int q = 0; q < V; ++q) {
             const int n = q + 1 < V ? q + 1 : q;
             const T hyi = q + 1 < V ? hy[n] : hyr, hzi = q + 1 < V ? hz[n] : hzr;
-            typename AccOf<T, S>::type a, b, c;
-            a.add(Ay, hzj[q] - hz[q]); a.add(Az, hyn[q] - hy[q], T(-1));
-            b.add(Az, hxn[q] - hx[q]); b.add(Ax, hzi - hz[q], T(-1));
-            c.add(Ax, hyi - hy[q]);    c.add(Ay, hxj[q] - hx[q], T(-1));
-            if (J) {
-                for (int s = 0; s < p.nsrc; ++s) {
-                    const Src &P = p.src[s];
-                    if ((P.k >= 0 && P.k != k) || (P.j >= 0 && P.j != r.j) || (P.i >= 0 && P.i != r.i0 + q)) continue;
-                    if (P.comp == 0) a.add(p.AJ, T(J[s]), T(-1));
-                    else if (P.comp == 1) b.add(p.AJ, T(J[s]), T(-1));
-                    else c.add(p.AJ, T(J[s]), T(-1));
-                }
-            }
-            ex[q] = quant<S>(add_scaled(ex[q], a, qa[q] + na[q]));
-            ey[q] = quant<S>(add_scaled(ey[q], b, qb[q] + nb[q]));
-            ez[q] = quant<S>(add_scaled(ez[q], c, qb[q] + qc[q]));
+            a[q].add(Ay, hzj[q] - hz[q]); a[q].add(Az, hyn[q] - hy[q], T(-1));
+            b[q].add(Az, hxn[q] - hx[q]); b[q].add(Ax, hzi - hz[q], T(-1));
+            c[q].add(Ax, hyi - hy[q]);    c[q].add(Ay, hxj[q] - hx[q], T(-1));
         }
-        stv<V>(Ex + o, ex, V);
-        stv<V>(Ey + o, ey, V);
-        stv<V>(Ez + o, ez, V);
-        if (pm) vec_probes<V>(p, when, pm, 0, r.i0, r.j, k, ex, ey, ez);
+        if (marks.J) vec_sources<V>(p, marks.J, r.i0, r.j, k, a, b, c);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            ex[q] = quant<S>(add_scaled(ex[q], a[q], qa[q] + na[q]));
+            ey[q] = quant<S>(add_scaled(ey[q], b[q], qb[q] + nb[q]));
+            ez[q] = quant<S>(add_scaled(ez[q], c[q], qb[q] + qc[q]));
+        }
+        stv<V>(Ex + o, ex);
+        stv<V>(Ey + o, ey);
+        stv<V>(Ez + o, ez);
+        if (marks.pm) vec_probes<V>(p, when, marks.pm, 0, r.i0, r.j, k, ex, ey, ez);
 #pragma unroll
         for (int q = 0; q < V; ++q) {
             hx[q] = hxn[q]; hy[q] = hyn[q];
             qa[q] = na[q]; qb[q] = nb[q]; qc[q] = nc[q];
         }
+        hyr = hyrn;
     }
 }
 
 // --- rim CTAs ----------------------------------------------------------------
 // One axis of a rim node: its D row there (offset of the first entry from the
 // node, coefficients) and the face it lies on (side -1 / +1, 0 for none).
-template <typename T> struct RimAxis {
-    long long off, st;
+template <typename I, typename T> struct RimAxis {
+    I off, st;
     T k[3];
     int side, type;
 };
 
-template <bool ELECTRIC, typename T, typename S>
-__device__ __forceinline__ RimAxis<T> rim_axis(const Params<T, S> &p, int a, int r)
+template <bool ELECTRIC, typename I, typename T, typename S>
+__device__ __forceinline__ RimAxis<I, T> rim_axis(const Params<T, S> &p, int a, int r)
 {
     const int n = p.n[a], last = n + (ELECTRIC ? 0 : 1);
-    RimAxis<T> x;
-    x.st = a == 0 ? 1 : a == 1 ? p.sy : p.sz;
+    RimAxis<I, T> x;
+    x.st = a == 0 ? I(1) : a == 1 ? (I)p.sy : (I)p.sz;
     if constexpr (ELECTRIC) dplus_coefs(r, n, x.k);
     else dminus_coefs(r, n, x.k);
-    x.off = (long long)((ELECTRIC ? dplus_start(r, n) : dminus_start(r, n)) - r) * x.st;
+    x.off = (I)((ELECTRIC ? dplus_start(r, n) : dminus_start(r, n)) - r) * x.st;
     x.side = r == 0 ? -1 : r == last ? 1 : 0;
     x.type = x.side ? p.face[2 * a + (x.side > 0)] : (ELECTRIC ? kPEC : kPMC);   // the type without a penalty
     return x;
@@ -361,8 +403,8 @@ __device__ __forceinline__ RimAxis<T> rim_axis(const Params<T, S> &p, int a, int
 
 // The row on its entries.  A two-point row gives the same bits either way; FP64,
 // whose pipe is the narrow one, takes the single subtraction.
-template <typename T>
-__device__ __forceinline__ T rim_row(const RimAxis<T> &x, const Tri<T> &v)
+template <typename I, typename T>
+__device__ __forceinline__ T rim_row(const RimAxis<I, T> &x, const Tri<T> &v)
 {
     if constexpr (std::is_same<T, double>::value)
         if (x.k[2] == T(0)) return v.b - v.a;
@@ -399,8 +441,8 @@ __device__ __noinline__ T rim_gamma(const Params<T, S> &p, int a, T se, T sm)
 // New value of component C at a rim node, in the operation order of h_apply /
 // e_apply.  v[t]: the entries of the two curl terms; se: sum of the node's eps
 // cells (4 for E, 2 for H, there only read on an absorbing face).
-template <typename T, int C, bool MUVAR, typename S>
-__device__ __forceinline__ T rim_apply(const Params<T, S> &p, const RimAxis<T> (&ax)[3], const int (&idx)[3], T old,
+template <typename T, int C, bool MUVAR, typename I, typename S>
+__device__ __forceinline__ T rim_apply(const Params<T, S> &p, const RimAxis<I, T> (&ax)[3], const int (&idx)[3], T old,
                                        const Tri<T> (&v)[2], T se, T sm, const double *J)
 {
     constexpr bool electric = C < 3;
@@ -431,31 +473,52 @@ __device__ __forceinline__ T rim_apply(const Params<T, S> &p, const RimAxis<T> (
 }
 
 // The entries of component C's two curl terms (a third entry only on closure rows).
-template <int C, typename T, typename S>
-__device__ __forceinline__ void rim_gather(const Params<T, S> &p, const RimAxis<T> (&ax)[3], long long o, Tri<T> (&v)[2])
+template <int C, typename I, typename T, typename S>
+__device__ __forceinline__ void rim_gather(const Params<T, S> &p, const RimAxis<I, T> (&ax)[3], I o, Tri<T> (&v)[2])
 {
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-        const RimAxis<T> &x = ax[curl_axis(C, t)];
-        const S *const q = p.F[curl_comp(C, t)] + (o + x.off);
-        v[t].a = ld_s(q);
-        v[t].b = ld_s(q + x.st);
-        v[t].c = x.k[2] != T(0) ? ld_s(q + 2 * x.st) : T(0);
+        const RimAxis<I, T> &x = ax[curl_axis(C, t)];
+        const S *const F = p.F[curl_comp(C, t)];
+        const I q = o + x.off;
+        v[t].a = ld_s(F + q);
+        v[t].b = ld_s(F + (I)(q + x.st));
+        v[t].c = x.k[2] != T(0) ? ld_s(F + (I)(q + x.st + x.st)) : T(0);
     }
 }
 
-// One rim node of a half-step (J, pm: the warp's sources and probes).  One code
-// for every rim node: variants for the row ends and for the layers took a
-// quarter fewer instructions and 15 % more time, waiting for instruction fetch.
-template <typename T, typename S, bool ELECTRIC, bool MUVAR>
-__device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i, int j, int k, const double *J,
-                                         unsigned long long pm)
+// Sums of the cells around a node of the three E components (four cells each) or
+// the three H components (two each), in the association of cell_sum.
+template <bool ELECTRIC, typename I, typename T>
+__device__ __forceinline__ void rim_cells(const float *m, I o, I sy, I sz, T &x, T &y, T &z)
+{
+    const float *const py = m + (I)(o + sy), *const pz = m + (I)(o + sz);
+    const T c = widen<T>(__ldg(m + o)), cx = widen<T>(__ldg(m + o + 1)), cy = widen<T>(__ldg(py));
+    const T cz = widen<T>(__ldg(pz));
+    if constexpr (ELECTRIC) {
+        const T cxy = widen<T>(__ldg(py + 1)), cxz = widen<T>(__ldg(pz + 1));
+        const T cyz = widen<T>(__ldg(m + (I)(o + sy + sz)));
+        x = (c + cy) + (cz + cyz);
+        y = (c + cx) + (cz + cxz);
+        z = (c + cx) + (cy + cxy);
+    } else {
+        x = c + cx;
+        y = c + cy;
+        z = c + cz;
+    }
+}
+
+// One rim node of a half-step.  One code for every rim node: variants for the
+// row ends and for the layers took a quarter fewer instructions and 15 % more
+// time, waiting for instruction fetch.
+template <typename I, typename T, typename S, bool ELECTRIC, bool MUVAR>
+__device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i, int j, int k, Marks marks)
 {
     constexpr int c0 = ELECTRIC ? 0 : 3;
     const int idx[3] = {i, j, k};
-    const RimAxis<T> ax[3] = {rim_axis<ELECTRIC, T>(p, 0, i), rim_axis<ELECTRIC, T>(p, 1, j),
-                              rim_axis<ELECTRIC, T>(p, 2, k)};
-    const long long o = (long long)k * p.sz + (long long)j * p.sy + i;
+    const RimAxis<I, T> ax[3] = {rim_axis<ELECTRIC, I, T>(p, 0, i), rim_axis<ELECTRIC, I, T>(p, 1, j),
+                                 rim_axis<ELECTRIC, I, T>(p, 2, k)};
+    const I sy = (I)p.sy, sz = (I)p.sz, o = (I)k * sz + (I)j * sy + (I)i;
     const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
     const bool abs = ax[0].type == kABS || ax[1].type == kABS || ax[2].type == kABS;
     pdl_wait();
@@ -463,35 +526,28 @@ __device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i
     rim_gather<c0>(p, ax, o, vx);
     rim_gather<c0 + 1>(p, ax, o, vy);
     rim_gather<c0 + 2>(p, ax, o, vz);
-    T x = ld_s(p.F[c0] + o), y = ld_s(p.F[c0 + 1] + o), z = ld_s(p.F[c0 + 2] + o);
+    S *const X = p.F[c0] + o, *const Y = p.F[c0 + 1] + o, *const Z = p.F[c0 + 2] + o;
+    T x = ld_s(X), y = ld_s(Y), z = ld_s(Z);
     T ex = T(0), ey = T(0), ez = T(0), mx = T(0), my = T(0), mz = T(0);
-    if (ELECTRIC || abs) {
-        ex = cell_sum<c0, T>(p.eps, o, p.sy, p.sz);
-        ey = cell_sum<c0 + 1, T>(p.eps, o, p.sy, p.sz);
-        ez = cell_sum<c0 + 2, T>(p.eps, o, p.sy, p.sz);
-    }
-    if (MUVAR && (!ELECTRIC || abs)) {
-        mx = cell_sum<c0, T>(p.mu, o, p.sy, p.sz);
-        my = cell_sum<c0 + 1, T>(p.mu, o, p.sy, p.sz);
-        mz = cell_sum<c0 + 2, T>(p.mu, o, p.sy, p.sz);
-    }
-    x = rim_apply<T, c0, MUVAR>(p, ax, idx, x, vx, ex, mx, J);
-    y = rim_apply<T, c0 + 1, MUVAR>(p, ax, idx, y, vy, ey, my, J);
-    z = rim_apply<T, c0 + 2, MUVAR>(p, ax, idx, z, vz, ez, mz, J);
+    if (ELECTRIC || abs) rim_cells<ELECTRIC>(p.eps, o, sy, sz, ex, ey, ez);
+    if (MUVAR && (!ELECTRIC || abs)) rim_cells<ELECTRIC>(p.mu, o, sy, sz, mx, my, mz);
+    x = rim_apply<T, c0, MUVAR>(p, ax, idx, x, vx, ex, mx, marks.J);
+    y = rim_apply<T, c0 + 1, MUVAR>(p, ax, idx, y, vy, ey, my, marks.J);
+    z = rim_apply<T, c0 + 2, MUVAR>(p, ax, idx, z, vz, ez, mz, marks.J);
     // nodes of each component (Table I); the others are not stored and hold no probe
     const int e = ELECTRIC ? 1 : 0;
-    if (i <= nx + e && j <= ny + 1 - e && k <= nz + 1 - e) st_s(p.F[c0] + o, x);
-    if (i <= nx + 1 - e && j <= ny + e && k <= nz + 1 - e) st_s(p.F[c0 + 1] + o, y);
-    if (i <= nx + 1 - e && j <= ny + 1 - e && k <= nz + e) st_s(p.F[c0 + 2] + o, z);
-    if (pm) {
+    if (i <= nx + e && j <= ny + 1 - e && k <= nz + 1 - e) st_s(X, x);
+    if (i <= nx + 1 - e && j <= ny + e && k <= nz + 1 - e) st_s(Y, y);
+    if (i <= nx + 1 - e && j <= ny + 1 - e && k <= nz + e) st_s(Z, z);
+    if (marks.pm) {
         const T a[1] = {x}, b[1] = {y}, c[1] = {z};
-        vec_probes<1>(p, when, pm, c0, i, j, k, a, b, c);
+        vec_probes<1>(p, when, marks.pm, c0, i, j, k, a, b, c);
     }
 }
 
 // Rim CTAs: the planes below and above the box first, then per z-chunk the y
 // layers and the row ends of its box planes.
-template <typename T, typename S, bool ELECTRIC, bool MUVAR>
+template <typename I, typename T, typename S, bool ELECTRIC, bool MUVAR>
 __device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w, When when, unsigned cta, unsigned q,
                                           int chunk)
 {
@@ -523,46 +579,37 @@ __device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w,
             j = w.lo[1] + (int)row;
         }
     }
-    unsigned long long pm = 0ull;
-    const double *J = nullptr;
-    if (p.nprb || (ELECTRIC && p.nsrc)) {
-        const int lane = threadIdx.x & 31;
-        const int jmin = __reduce_min_sync(0xffffffffu, j), jmax = __reduce_max_sync(0xffffffffu, j);
-        const int kmin = __reduce_min_sync(0xffffffffu, k), kmax = __reduce_max_sync(0xffffffffu, k);
-        if (p.nprb) pm = rows_probe_mask(p.prb, p.nprb, ELECTRIC ? 0 : 3, kmin, kmax, jmin, jmax, lane);
-        if (ELECTRIC) J = source_values(p, when.step, lane, kmin, kmax, jmin, jmax, 0, INT32_MAX);
-    }
-    if (t >= count) return;
-    rim_node<T, S, ELECTRIC, MUVAR>(p, when, i, j, k, J, pm);
+    const Marks marks = find_marks<ELECTRIC>(p, when, i, i, j, k, k);
+    if (t < count) rim_node<I, T, S, ELECTRIC, MUVAR>(p, when, i, j, k, marks);
 }
 
 // CTA `cta` of a half-step's work list.
-template <bool ELECTRIC, bool MUVAR, int V, typename T, typename S>
+template <bool ELECTRIC, bool MUVAR, int V, typename I, typename T, typename S>
 __device__ __forceinline__ void half_cta(const Params<T, S> &p, const Sweep &w, When when, unsigned cta)
 {
     const unsigned r = cta < w.cz ? 0u : cta - w.cz, chunk = r / w.dchunk, q = r - chunk * w.cchunk;
     if (cta >= w.cz && q < w.cbox) {
-        if constexpr (ELECTRIC) box_e<T, S, V>(p, w, when, q, (int)chunk);
-        else box_h<T, S, MUVAR, V>(p, w, when, q, (int)chunk);
+        if constexpr (ELECTRIC) box_e<I, T, S, V>(p, w, when, q, (int)chunk);
+        else box_h<I, T, S, MUVAR, V>(p, w, when, q, (int)chunk);
     } else {
-        sweep_rim<T, S, ELECTRIC, MUVAR>(p, w, when, cta, q, (int)chunk);
+        sweep_rim<I, T, S, ELECTRIC, MUVAR>(p, w, when, cta, q, (int)chunk);
     }
 }
 
-template <typename T, typename S, bool MUVAR, int V>
-__global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 4 : 5)
+template <typename I, typename T, typename S, bool MUVAR, int V>
+__global__ void __launch_bounds__(kSweepThreads, half_ctas<T, V>(false))
     half_h(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
 {
     pdl_release();
-    half_cta<false, MUVAR, V>(p, w, {p.step, p.probe_slot}, blockIdx.x);
+    half_cta<false, MUVAR, V, I>(p, w, {p.step, p.probe_slot}, blockIdx.x);
 }
 
-template <typename T, typename S, bool MUVAR, int V>
-__global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 4 : 5)
+template <typename I, typename T, typename S, bool MUVAR, int V>
+__global__ void __launch_bounds__(kSweepThreads, half_ctas<T, V>(true))
     half_e(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
 {
     pdl_release();
-    half_cta<true, MUVAR, V>(p, w, {p.step, p.probe_slot}, blockIdx.x);
+    half_cta<true, MUVAR, V, I>(p, w, {p.step, p.probe_slot}, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -579,7 +626,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 4 : 5)
 // L2 together, through all its steps, then the next group.
 // ---------------------------------------------------------------------------
 struct alignas(16) BatchSweep : Sweep {};
-static_assert(sizeof(BatchSweep) % 16 == 0 && offsetof(Params<float>, link) % 16 == 0, "copied in 16-byte units");
+static_assert(sizeof(BatchSweep) % 16 == 0, "copied in 16-byte units");
 
 struct alignas(16) BatchHalf {
     alignas(16) Params<float> p;  // the member's fields, in place (step and probe slot come from the counter)
@@ -590,7 +637,7 @@ struct alignas(16) BatchHalf {
 };
 
 template <bool ELECTRIC, int V>
-__global__ void __launch_bounds__(kSweepThreads, V == 4 ? 5 : 7)
+__global__ void __launch_bounds__(kSweepThreads, half_ctas<float, V>(ELECTRIC))
     half_batched(const BatchHalf *grids, const int *pre, int n, int offset)
 {
     __shared__ __align__(16) Params<float> p;
@@ -604,25 +651,25 @@ __global__ void __launch_bounds__(kSweepThreads, V == 4 ? 5 : 7)
         for (int q = threadIdx.x; q < bytes / 16; q += kSweepThreads)
             static_cast<uint4 *>(dst)[q] = __ldg(static_cast<const uint4 *>(src) + q);
     };
-    copy(&p, &B.p, (int)offsetof(Params<float>, link) / 16 * 16);   // members have no links
+    copy(&p, &B.p, ((int)offsetof(Params<float>, link) + 15) / 16 * 16);   // members have no links
     copy(&w, &B.w[ELECTRIC], sizeof(w));
     const long long step = *B.counter + offset;
     if (step >= B.target) return;
     __syncthreads();
-    half_cta<ELECTRIC, false, V>(p, w, {step, step - B.probe_base}, (unsigned)((int)blockIdx.x + first - pre[g]));
+    half_cta<ELECTRIC, false, V, unsigned>(p, w, {step, step - B.probe_base}, (unsigned)((int)blockIdx.x + first - pre[g]));
 }
 
 // One member of a batch alone: its parameters are the launch's, which cost a CTA
 // no copy (a grid that fills the GPU by itself steps 1.3 times faster so).
 template <bool ELECTRIC, int V>
-__global__ void __launch_bounds__(kSweepThreads, V == 4 ? 5 : 7)
+__global__ void __launch_bounds__(kSweepThreads, half_ctas<float, V>(ELECTRIC))
     half_member(const __grid_constant__ Params<float> p, const __grid_constant__ Sweep w, const long long *counter,
                 long long target, long long probe_base, int offset)
 {
     pdl_release();
     const long long step = *counter + offset;
     if (step >= target) return;
-    half_cta<ELECTRIC, false, V>(p, w, {step, step - probe_base}, blockIdx.x);
+    half_cta<ELECTRIC, false, V, unsigned>(p, w, {step, step - probe_base}, blockIdx.x);
 }
 
 // The members' step counters after a chunk of k steps.

@@ -90,6 +90,7 @@ struct Params {
     T uB, uA;                          // fscale[H]/fscale[E] and its inverse: B and A carry the
                                        // scale ratio; the absorbing-SAT gamma needs them without
     int nsrc, nprb;
+    int pbox[2][6], sbox[6];           // index boxes (low, high per axis) around the probes of E, of H, and the sources
     T *probe_buf;
     long long probe_cap, probe_slot;   // sample slot of this step (skip if >= cap)
     long long step;                    // n: the E half-step injects J(t^{n+1/2})

@@ -108,6 +108,7 @@ struct sbp_sim {
     sbp::Band band_hb, band_eb;
     sbp::Sweep sweep[2];                  // in-place half-steps: work lists (H, E) and vector width
     int sweep_v = 1;
+    bool sweep_big = false;               // element indices need 64 bits
     float *eps = nullptr;
     float *mu = nullptr;
     double *partials = nullptr;
@@ -469,6 +470,11 @@ int choose_sweep(sbp_sim *s)
     else if (nodes > 64000000) kz = 16;
     else if (nodes > 4000000) kz = 8;
     else if (v == 4 && s->prec == SBP_FP32) v = 2;
+    // arrays of 2^32 elements and more (with room for the offsets past the last
+    // plane) index with 64 bits; tests ask for it on small grids
+    s->sweep_big = s->field_elems + 2 * (size_t)s->sz >= (1ull << 32);
+    if (const char *env = std::getenv("SBP_STEP_PATH")) s->sweep_big = s->sweep_big || std::strcmp(env, "inplace64") == 0;
+    if (s->sweep_big && s->prec != SBP_FP64) v = 4;
     s->sweep_v = v;
     int rc = make_sweep(s->n, false, v, kz, s->sweep[0]);
     return rc ? rc : make_sweep(s->n, true, v, kz, s->sweep[1]);
@@ -656,6 +662,17 @@ int make_params(const sbp_sim *s, sbp::Params<T, S> &p, int eset, int hset)
     for (int q = 0; q < p.nsrc; q++) p.src[q] = s->src[q];
     p.nprb = (int)s->prb.size();
     for (int q = 0; q < p.nprb; q++) p.prb[q] = s->prb[q];
+    for (int *box : {p.pbox[0], p.pbox[1], p.sbox})
+        for (int a = 0; a < 3; a++) { box[a] = INT_MAX; box[3 + a] = -1; }
+    auto stretch = [](int *box, int a, int lo, int hi) { box[a] = std::min(box[a], lo); box[3 + a] = std::max(box[3 + a], hi); };
+    for (const sbp::Prb &q : s->prb) {
+        const int at[3] = {q.i, q.j, q.k};
+        for (int a = 0; a < 3; a++) stretch(p.pbox[q.comp >= 3], a, at[a], at[a]);
+    }
+    for (const sbp::Src &q : s->src) {
+        const int at[3] = {q.i, q.j, q.k};
+        for (int a = 0; a < 3; a++) stretch(p.sbox, a, std::max(at[a], 0), at[a] < 0 ? INT_MAX : at[a]);
+    }
     p.probe_buf = static_cast<T *>(s->probe_buf);   // samples in the arithmetic type
     p.probe_cap = s->probe_buf ? s->probe_cap : 0;
     p.probe_slot = s->step - s->probe_base;
@@ -685,7 +702,7 @@ int launch_dependent(K kernel, cudaStream_t st, const P &p, const sbp::Sweep &w)
 }
 
 // One in-place half-step of the current set (h: H, else E).
-template <typename T, typename S, int V>
+template <typename I, typename T, typename S, int V>
 int launch_half_t(const sbp_sim *s, bool h)
 {
     sbp::Params<T, S> p;
@@ -693,20 +710,25 @@ int launch_half_t(const sbp_sim *s, bool h)
     if (rc) return rc;
     const sbp::Sweep &w = s->sweep[h ? 0 : 1];
     if (s->mu)
-        return h ? launch_dependent(sbp::half_h<T, S, true, V>, s->stream, p, w)
-                 : launch_dependent(sbp::half_e<T, S, true, V>, s->stream, p, w);
-    return h ? launch_dependent(sbp::half_h<T, S, false, V>, s->stream, p, w)
-             : launch_dependent(sbp::half_e<T, S, false, V>, s->stream, p, w);
+        return h ? launch_dependent(sbp::half_h<I, T, S, true, V>, s->stream, p, w)
+                 : launch_dependent(sbp::half_e<I, T, S, true, V>, s->stream, p, w);
+    return h ? launch_dependent(sbp::half_h<I, T, S, false, V>, s->stream, p, w)
+             : launch_dependent(sbp::half_e<I, T, S, false, V>, s->stream, p, w);
 }
 
 int launch_half(const sbp_sim *s, bool h)
 {
+    using U = unsigned;
+    using L = long long;
     const int v = s->sweep_v;
-    if (s->prec == SBP_FP64) return launch_half_t<double, double, 1>(s, h);
+    if (s->prec == SBP_FP64)
+        return s->sweep_big ? launch_half_t<L, double, double, 1>(s, h) : launch_half_t<U, double, double, 1>(s, h);
     if (s->prec == SBP_FP32_FP16STORE)
-        return v > 1 ? launch_half_t<float, __half, 4>(s, h) : launch_half_t<float, __half, 1>(s, h);
-    return v == 4 ? launch_half_t<float, float, 4>(s, h)
-         : v == 2 ? launch_half_t<float, float, 2>(s, h) : launch_half_t<float, float, 1>(s, h);
+        return s->sweep_big ? launch_half_t<L, float, __half, 4>(s, h)
+             : v > 1        ? launch_half_t<U, float, __half, 4>(s, h) : launch_half_t<U, float, __half, 1>(s, h);
+    return s->sweep_big ? launch_half_t<L, float, float, 4>(s, h)
+         : v == 4       ? launch_half_t<U, float, float, 4>(s, h)
+         : v == 2       ? launch_half_t<U, float, float, 2>(s, h) : launch_half_t<U, float, float, 1>(s, h);
 }
 
 // Parameters of the one-pass interior step reading set `old`, writing set old^1.

@@ -39,10 +39,10 @@ def test_against_oracle(n, mu, precision):
 def test_bitwise_equal_to_one_pass(n, precision, monkeypatch):
     w = wl.random_box(n, faces=(A, M, P, A, P, M), seed=5)
     out = []
-    for path in ("onepass", "inplace"):
+    for path in ("onepass", "inplace", "inplace64"):
         monkeypatch.setenv("SBP_STEP_PATH", path)
         s = parity.gpu_run(w, 9, precision)[0]
         out.append([s.field(c) for c in range(6)] + [s.probes()])
         s.close()
-    for a, b in zip(*out):
-        assert np.array_equal(a, b)
+    for a, b, c in zip(*out):
+        assert np.array_equal(a, b) and np.array_equal(a, c)

@@ -508,11 +508,13 @@ __device__ __forceinline__ void rim_cells(const float *m, I o, I sy, I sz, T &x,
     }
 }
 
-// One rim node of a half-step.  One code for every rim node: variants for the
+// One rim node of a half-step, its new values to `out` (in place, or the new set
+// of a one-pass step).  One code for every rim node: variants for the
 // row ends and for the layers took a quarter fewer instructions and 15 % more
 // time, waiting for instruction fetch.
 template <typename I, typename T, typename S, bool ELECTRIC, bool MUVAR>
-__device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i, int j, int k, Marks marks)
+__device__ __forceinline__ void rim_node(const Params<T, S> &p, S *const (&out)[3], When when, int i, int j, int k,
+                                         Marks marks)
 {
     constexpr int c0 = ELECTRIC ? 0 : 3;
     const int idx[3] = {i, j, k};
@@ -526,8 +528,7 @@ __device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i
     rim_gather<c0>(p, ax, o, vx);
     rim_gather<c0 + 1>(p, ax, o, vy);
     rim_gather<c0 + 2>(p, ax, o, vz);
-    S *const X = p.F[c0] + o, *const Y = p.F[c0 + 1] + o, *const Z = p.F[c0 + 2] + o;
-    T x = ld_s(X), y = ld_s(Y), z = ld_s(Z);
+    T x = ld_s(p.F[c0] + o), y = ld_s(p.F[c0 + 1] + o), z = ld_s(p.F[c0 + 2] + o);
     T ex = T(0), ey = T(0), ez = T(0), mx = T(0), my = T(0), mz = T(0);
     if (ELECTRIC || abs) rim_cells<ELECTRIC>(p.eps, o, sy, sz, ex, ey, ez);
     if (MUVAR && (!ELECTRIC || abs)) rim_cells<ELECTRIC>(p.mu, o, sy, sz, mx, my, mz);
@@ -536,9 +537,9 @@ __device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i
     z = rim_apply<T, c0 + 2, MUVAR>(p, ax, idx, z, vz, ez, mz, marks.J);
     // nodes of each component (Table I); the others are not stored and hold no probe
     const int e = ELECTRIC ? 1 : 0;
-    if (i <= nx + e && j <= ny + 1 - e && k <= nz + 1 - e) st_s(X, x);
-    if (i <= nx + 1 - e && j <= ny + e && k <= nz + 1 - e) st_s(Y, y);
-    if (i <= nx + 1 - e && j <= ny + 1 - e && k <= nz + e) st_s(Z, z);
+    if (i <= nx + e && j <= ny + 1 - e && k <= nz + 1 - e) st_s(out[0] + o, x);
+    if (i <= nx + 1 - e && j <= ny + e && k <= nz + 1 - e) st_s(out[1] + o, y);
+    if (i <= nx + 1 - e && j <= ny + 1 - e && k <= nz + e) st_s(out[2] + o, z);
     if (marks.pm) {
         const T a[1] = {x}, b[1] = {y}, c[1] = {z};
         vec_probes<1>(p, when, marks.pm, c0, i, j, k, a, b, c);
@@ -548,8 +549,8 @@ __device__ __forceinline__ void rim_node(const Params<T, S> &p, When when, int i
 // Rim CTAs: the planes below and above the box first, then per z-chunk the y
 // layers and the row ends of its box planes.
 template <typename I, typename T, typename S, bool ELECTRIC, bool MUVAR>
-__device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w, When when, unsigned cta, unsigned q,
-                                          int chunk)
+__device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w, S *const (&out)[3], When when, unsigned cta,
+                                          unsigned q, int chunk)
 {
     unsigned t, count;
     int i, j, k;
@@ -580,7 +581,7 @@ __device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w,
         }
     }
     const Marks marks = find_marks<ELECTRIC>(p, when, i, i, j, k, k);
-    if (t < count) rim_node<I, T, S, ELECTRIC, MUVAR>(p, when, i, j, k, marks);
+    if (t < count) rim_node<I, T, S, ELECTRIC, MUVAR>(p, out, when, i, j, k, marks);
 }
 
 // CTA `cta` of a half-step's work list.
@@ -592,8 +593,26 @@ __device__ __forceinline__ void half_cta(const Params<T, S> &p, const Sweep &w, 
         if constexpr (ELECTRIC) box_e<I, T, S, V>(p, w, when, q, (int)chunk);
         else box_h<I, T, S, MUVAR, V>(p, w, when, q, (int)chunk);
     } else {
-        sweep_rim<I, T, S, ELECTRIC, MUVAR>(p, w, when, cta, q, (int)chunk);
+        constexpr int c0 = ELECTRIC ? 0 : 3;
+        S *const out[3] = {p.F[c0], p.F[c0 + 1], p.F[c0 + 2]};
+        sweep_rim<I, T, S, ELECTRIC, MUVAR>(p, w, out, when, cta, q, (int)chunk);
     }
+}
+
+// The nodes of a half-step that the one-pass kernel leaves out (a work list
+// without box CTAs), from the old set to the new one.
+//
+// One node per thread with every load first, where the slab kernels (band_h,
+// band_e) took a warp's nodes through code for its slab with 64-bit addresses: at
+// 512^3 130 + 140 us a step alone (157 + 170 before), beside the one-pass kernel
+// the step takes 1423 us (1471).
+template <bool ELECTRIC, typename S>
+__global__ void __launch_bounds__(kSweepThreads, 7)
+    rim_step(const __grid_constant__ Params<float, S> p, const __grid_constant__ Sweep w, S *x, S *y, S *z)
+{
+    const unsigned cta = blockIdx.x, r = cta < w.cz ? 0u : cta - w.cz, chunk = r / w.dchunk, q = r - chunk * w.cchunk;
+    S *const out[3] = {x, y, z};
+    sweep_rim<unsigned, float, S, ELECTRIC, false>(p, w, out, {p.step, p.probe_slot}, cta, q, (int)chunk);
 }
 
 template <typename I, typename T, typename S, bool MUVAR, int V>

@@ -107,6 +107,7 @@ struct sbp_sim {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     sbp::Band band_hb, band_eb;
     sbp::Sweep sweep[2];                  // in-place half-steps: work lists (H, E) and vector width
+    sbp::Sweep rim[2];                    // one-pass step: the nodes outside its kernel (H, E)
     int sweep_v = 1;
     bool sweep_big = false;               // element indices need 64 bits
     float *eps = nullptr;
@@ -411,8 +412,10 @@ sbp::FastDiv fast_div(unsigned d)
 }
 
 // Work list of an in-place half-step (electric: of E, else of H) of an n-cell
-// grid: vectors of v nodes, z-chunks of kz planes.
-int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w)
+// grid: vectors of v nodes, z-chunks of kz planes.  onepass: the part of a
+// one-pass step outside its kernel instead (H outside [4, n-3]^3, E outside
+// [3, n-3]^3), no box CTAs.
+int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool onepass = false)
 {
     std::memset(&w, 0, sizeof(w));
     long long box[3];
@@ -421,13 +424,14 @@ int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w)
         const int lo = electric ? 2 : 3, hi = n[a] - 2;
         w.lo[a] = a ? lo : (lo + v - 1) / v * v;
         w.hi[a] = std::max(a ? hi : (hi + 1) / v * v - 1, w.lo[a] - 1);
+        if (onepass) { w.lo[a] = electric ? 3 : 4; w.hi[a] = n[a] - 3; }
         box[a] = w.hi[a] - w.lo[a] + 1;
     }
     const long long nv = box[0] / v, planes = n[2] + 2, rows = n[1] + 2, xs = n[0] + 2;
     const long long vecs = nv * box[1], zplanes = planes - box[2], ynodes = (rows - box[1]) * xs;
     const long long ends = xs - box[0], rim = ynodes + ends * box[1];
     auto ctas_of = [&](long long items) { return (items + sbp::kSweepThreads - 1) / sbp::kSweepThreads; };
-    const long long cz = ctas_of(zplanes * rows * xs), cbox = ctas_of(vecs), cchunk = cbox + ctas_of(kz * rim);
+    const long long cz = ctas_of(zplanes * rows * xs), cbox = onepass ? 0 : ctas_of(vecs), cchunk = cbox + ctas_of(kz * rim);
     const long long ctas = cz + cchunk * ((planes + kz - 1) / kz);
     if (std::max(std::max(zplanes * rows * xs, vecs), kz * rim) >= (1ll << 31) - 1024 || ctas >= (1ll << 31))
         return SBP_EINVAL;
@@ -453,23 +457,27 @@ int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w)
     return SBP_OK;
 }
 
-// Vector width and planes per z-chunk of the in-place half-steps, by the nodes
-// of the grid.  Measured per step, CTAs of 128 threads (256 are 0-10 % slower
-// everywhere: fewer warps fit beside the register use):
-//   125 k nodes (61 x 47 x 38)    V 1: 7.8 us; V 2: 13, too few threads
-//   1.6 M nodes (117 x 96 x 131)  V 2, 4 planes: 22.7 us; V 1 27.7; V 4 24.3;
-//                                 V 2, 2 planes: 24.7, 1 plane: 28.6 (CTAs start at about one per ns)
-//   17 M nodes (256^3)            V 4, 8 planes: 229 us; V 2: 234; V 4, 4 planes: 230
-//   512^3, FP16 storage           V 4, 16 planes: 1138 us, 8 planes: 1168
-// FP64 is bound by its pipe and runs one node per thread (two: 1 % slower).
+// Vector width (V) and planes per z-chunk of the in-place half-steps, by the
+// nodes of the grid.  us per step, FP32, as V:planes (CTAs of 128 threads; 256 are
+// slower everywhere, fewer warps fit beside the register use):
+//   nodes          1:1    1:2    2:2    2:4    2:8    4:4    4:8    4:16
+//   125 k          8.0   10.1   13
+//   0.29 M (64^3) 12.5   11.4    9.6    9.3   13.2   10.5   15.1   23.6
+//   0.57 M (82^3) 17.9   15.5   13.4   13.4   15.0   14.0   18.5   27.6
+//   1.6 M         35.2   28.9   23.4   21.8   23.5   22.7   27.0   36.1
+//   2.4 M         51.9   41.6   33.0   30.4   31.1   31.9   35.2   44.0
+//   2 x 3.7 M      197    165    126    122    125    117    123    136
+//   5.1 M          133    110   82.7   80.2   81.1   76.2   78.1   84.9
+//   17 M (256^3)   383    332    242    234    231    214    214    223
+// FP16 storage at 512^3: 4:16 1036, 4:8 1064.  FP64 is bound by its pipe: one node
+// per thread, 1 or 2 planes (2 nodes: 1 % slower).
 int choose_sweep(sbp_sim *s)
 {
     const long long nodes = (long long)(s->n[0] + 2) * (s->n[1] + 2) * (s->n[2] + 2);
-    int v = nodes < 200000 || s->prec == SBP_FP64 ? 1 : 4, kz = nodes < 200000 ? 1 : nodes < 600000 ? 2 : 4;
-    if (s->prec == SBP_FP64) kz = std::min(kz, 2);
-    else if (nodes > 64000000) kz = 16;
-    else if (nodes > 4000000) kz = 8;
-    else if (v == 4 && s->prec == SBP_FP32) v = 2;
+    int v = 4, kz = nodes > 64000000 ? 16 : 4;
+    if (nodes < 200000) v = kz = 1;
+    else if (s->prec == SBP_FP64) { v = 1; kz = 2; }
+    else if (nodes < 2500000 && s->prec == SBP_FP32) v = 2;
     // arrays of 2^32 elements and more (with room for the offsets past the last
     // plane) index with 64 bits; tests ask for it on small grids
     s->sweep_big = s->field_elems + 2 * (size_t)s->sz >= (1ull << 32);
@@ -482,11 +490,11 @@ int choose_sweep(sbp_sim *s)
 
 // Whether a step of this simulation runs the one-pass kernel (else the in-place
 // half-steps).  One pass moves 13 words per node instead of 19, but marches
-// planes behind a barrier and leaves the boundary to separate band launches, so
-// it pays where the grid is far larger than L2 (per step, FP32, one pass /
-// in place: 61 x 47 x 38 17.6 / 7.8 us, 117 x 96 x 131 39 / 22.7 us, 256^3 236 /
-// 229 us, 512^3 1483 / 1600 us).  With FP16 storage one pass is issue-bound
-// (512^3: 1337 / 1140 us) and never pays.
+// planes behind a barrier and leaves the boundary to launches of its own, so it
+// pays where the grid is far larger than L2 (per step, FP32, one pass / in place:
+// 61 x 47 x 38 17.6 / 7.8 us, 117 x 96 x 131 39 / 21.8 us, 256^3 236 / 214 us,
+// 512^3 1423 / 1600 us).  With FP16 storage one pass is issue-bound (512^3: 1337 /
+// 1036 us) and never pays.
 constexpr long long kOnePassNodes = 24000000;
 
 int setup(sbp_sim *s, const sbp_grid_desc *d, const Layout &L, char *ws)
@@ -523,6 +531,8 @@ int setup(sbp_sim *s, const sbp_grid_desc *d, const Layout &L, char *ws)
     s->fused_width = L.fused_width;
     s->fused_grid = L.fused_grid;
     if (int rc = choose_sweep(s)) return rc;
+    for (int e = 0; e < 2 && s->one_pass; e++)
+        if (int rc = make_sweep(s->n, e == 1, 1, 4, s->rim[e], true)) return rc;
     char *p = ws;
     for (int set = 0; set < (L.fused ? 2 : 1); set++)
         for (int c = 0; c < 6; c++) { s->set[set][c] = p; p += L.field_bytes; }
@@ -819,6 +829,9 @@ int launch_fused_interior_t(sbp_sim *s)
     return SBP_OK;
 }
 
+// The slab kernels keep the Yee comparator and arrays that need 64-bit indices.
+bool rim_runs(const sbp_sim *s) { return s->one_pass && !s->fdtd && !s->sweep_big; }
+
 // Band H (old -> new) on stream st.
 template <typename S>
 int launch_band_h_t(sbp_sim *s, cudaStream_t st)
@@ -829,7 +842,10 @@ int launch_band_h_t(sbp_sim *s, cudaStream_t st)
     if (rc) return rc;
     const sbp::Band &bh = s->band_hb;
     S **ns = reinterpret_cast<S **>(s->set[nw]);
-    sbp::band_h<float, false><<<bh.ctas, 256, 0, st>>>(p, bh, ns[3], ns[4], ns[5]);
+    if (rim_runs(s))
+        sbp::rim_step<false, S><<<s->rim[0].ctas, sbp::kSweepThreads, 0, st>>>(p, s->rim[0], ns[3], ns[4], ns[5]);
+    else
+        sbp::band_h<float, false><<<bh.ctas, 256, 0, st>>>(p, bh, ns[3], ns[4], ns[5]);
     SBP_CUDA(cudaGetLastError());
     return SBP_OK;
 }
@@ -844,7 +860,10 @@ int launch_band_e_t(sbp_sim *s, cudaStream_t st)
     if (rc) return rc;
     const sbp::Band &be = s->band_eb;
     S **ns = reinterpret_cast<S **>(s->set[nw]);
-    sbp::band_e<float, false><<<be.ctas, 256, 0, st>>>(p, be, ns[0], ns[1], ns[2]);
+    if (rim_runs(s))
+        sbp::rim_step<true, S><<<s->rim[1].ctas, sbp::kSweepThreads, 0, st>>>(p, s->rim[1], ns[0], ns[1], ns[2]);
+    else
+        sbp::band_e<float, false><<<be.ctas, 256, 0, st>>>(p, be, ns[0], ns[1], ns[2]);
     SBP_CUDA(cudaGetLastError());
     return SBP_OK;
 }

@@ -18,19 +18,21 @@ def fast_div(d):
     return lambda n: (((n * mul) >> 32) + n) >> sh
 
 
-def cover(n, electric, v, kz):
+def cover(n, electric, v, kz, onepass=False):
     lo, hi, box = [0] * 3, [0] * 3, [0] * 3
     for a in range(3):
         low, high = (2 if electric else 3), n[a] - 2
         lo[a] = low if a else (low + v - 1) // v * v
         hi[a] = max(high if a else (high + 1) // v * v - 1, lo[a] - 1)
+        if onepass:
+            lo[a], hi[a] = (3 if electric else 4), n[a] - 3
         box[a] = hi[a] - lo[a] + 1
     nv, planes, rows, xs = box[0] // v, n[2] + 2, n[1] + 2, n[0] + 2
     assert box[0] % v == 0
     vecs, zplanes, ynodes, ends = nv * box[1], planes - box[2], (rows - box[1]) * xs, xs - box[0]
     rim = ynodes + ends * box[1]
     ctas_of = lambda items: (items + THREADS - 1) // THREADS
-    cz, cbox = ctas_of(zplanes * rows * xs), ctas_of(vecs)
+    cz, cbox = ctas_of(zplanes * rows * xs), 0 if onepass else ctas_of(vecs)
     cchunk = cbox + ctas_of(kz * rim)
     chunks = (planes + kz - 1) // kz
     dnv, dxs, drows = fast_div(max(nv, 1)), fast_div(xs), fast_div(rows)
@@ -83,6 +85,16 @@ def test_every_node_once(electric, v):
         for kz in (1, 3, 16):
             hits = cover(n, electric, v, kz)
             assert hits.min() == 1 and hits.max() == 1, (n, kz)
+
+
+@pytest.mark.parametrize("electric", [False, True])
+def test_one_pass_leaves_the_rim(electric):
+    """Without box items: every node outside the one-pass box once, none inside."""
+    for n in [(8, 8, 8), (9, 8, 11), (12, 17, 8), (34, 9, 10), (21, 30, 26)]:
+        hits = cover(n, electric, 1, 4, onepass=True)
+        lo, hi = (3 if electric else 4), [m - 3 for m in n]
+        inner = hits[lo:hi[2] + 1, lo:hi[1] + 1, lo:hi[0] + 1]
+        assert inner.max(initial=0) == 0 and hits.sum() == hits.size - inner.size and hits.max() == 1
 
 
 def test_fast_division():

@@ -28,11 +28,11 @@ namespace sbp {
 constexpr int kSweepThreads = 128;        // threads of a CTA
 
 // CTAs of a half-step that fit an SM, by registers: 72 a thread in FP32 (76-80 left
-// to the compiler cost 8 % at 117 x 96 x 131), 96 for E in vectors of 4, 112 and
-// more in FP64.
+// to the compiler cost 8 % at 117 x 96 x 131), 80 for E in vectors of 4 (96: 512^3
+// in FP16 storage 1048 us per step, 997 now), 112 and more in FP64.
 template <typename T, int V> constexpr int half_ctas(bool electric)
 {
-    return sizeof(T) == 8 ? 4 : V == 4 && electric ? 5 : 7;
+    return sizeof(T) == 8 ? 4 : V == 4 && electric ? 6 : 7;
 }
 
 // n / d for n < 2^31, with the multiplier of d found on the host.
@@ -50,6 +50,7 @@ struct Sweep {
     unsigned ynodes, rim;     // rim nodes of a box plane: y layers, in all
     unsigned cz;              // CTAs of the planes below and above the box (first in the list)
     unsigned cbox, cchunk;    // box CTAs and all CTAs of a z-chunk
+    unsigned flip;            // last chunk when the chunks are taken from the last to the first, else 0
     unsigned ctas;
     FastDiv dnv, dxs, drows, dends, drim, dchunk;
 };
@@ -384,6 +385,7 @@ __device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, Whe
 template <typename I, typename T> struct RimAxis {
     I off, st;
     T k[3];
+    bool closure;             // a closure row: its third entry counts
     int side, type;
 };
 
@@ -395,6 +397,8 @@ __device__ __forceinline__ RimAxis<I, T> rim_axis(const Params<T, S> &p, int a, 
     x.st = a == 0 ? I(1) : a == 1 ? (I)p.sy : (I)p.sz;
     if constexpr (ELECTRIC) dplus_coefs(r, n, x.k);
     else dminus_coefs(r, n, x.k);
+    // (asked of the index, not of the coefficient: an FP64 comparison goes through the FP64 pipe)
+    x.closure = ELECTRIC ? r <= 1 || r >= n - 1 : r == 2 || r == n - 1 || r == n + 1;
     x.off = (I)((ELECTRIC ? dplus_start(r, n) : dminus_start(r, n)) - r) * x.st;
     x.side = r == 0 ? -1 : r == last ? 1 : 0;
     x.type = x.side ? p.face[2 * a + (x.side > 0)] : (ELECTRIC ? kPEC : kPMC);   // the type without a penalty
@@ -407,19 +411,8 @@ template <typename I, typename T>
 __device__ __forceinline__ T rim_row(const RimAxis<I, T> &x, const Tri<T> &v)
 {
     if constexpr (std::is_same<T, double>::value)
-        if (x.k[2] == T(0)) return v.b - v.a;
+        if (!x.closure) return v.b - v.a;
     return row_chain(x.k, v.a, v.b, v.c);
-}
-
-// The partner's value of field u at the face node that node (i, j, k) faces along a.
-template <typename T, typename S, bool ELECTRIC>
-__device__ __noinline__ T rim_partner(const Params<T, S> &p, int f, int u, int i, int j, int k)
-{
-    const Link &L = p.link[f];
-    const int a = f >> 1, nidx = L.side < 0 ? 0 : ELECTRIC ? L.n_norm + 1 : L.n_norm;
-    const long long on = (long long)(a == 0 ? nidx : i) + (long long)(a == 1 ? nidx : j) * L.sy +
-                         (long long)(a == 2 ? nidx : k) * L.sz;
-    return link_value<false, T, S>(L, u, on);
 }
 
 // Absorbing self term along axis a from the sums of the node's cells.  One copy,
@@ -439,26 +432,26 @@ __device__ __noinline__ T rim_gamma(const Params<T, S> &p, int a, T se, T sm)
     }
 }
 // New value of component C at a rim node, in the operation order of h_apply /
-// e_apply.  v[t]: the entries of the two curl terms; se: sum of the node's eps
-// cells (4 for E, 2 for H, there only read on an absorbing face).
+// e_apply.  v[t]: the entries of the two curl terms; nv[t]: the partner's values on
+// interface faces; se: sum of the node's eps cells (4 for E, 2 for H, there only
+// read on an absorbing face).
 template <typename T, int C, bool MUVAR, typename I, typename S>
 __device__ __forceinline__ T rim_apply(const Params<T, S> &p, const RimAxis<I, T> (&ax)[3], const int (&idx)[3], T old,
-                                       const Tri<T> (&v)[2], T se, T sm, const double *J)
+                                       const Tri<T> (&v)[2], const T (&nv)[2], T se, T sm, const double *J)
 {
     constexpr bool electric = C < 3;
     typename AccOf<T, S>::type acc;
     T gam = T(0);
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-        const int u = curl_comp(C, t), a = curl_axis(C, t), sg = curl_sign(t);
+        const int a = curl_axis(C, t), sg = curl_sign(t);
         const Coef<T> &cf = electric ? p.A[a] : p.B[a];
         acc.add(cf, rim_row(ax[a], v[t]), T(sg));
         if (ax[a].type == (electric ? kPEC : kPMC)) continue;
-        const T phi = T(-sg * ax[a].side);
+        const bool up = sg * ax[a].side < 0;           // phi = -sg * side
         T pv = ax[a].side < 0 ? v[t].a : v[t].c;
-        if (ax[a].type == kIFACE)
-            pv = pv - rim_partner<T, S, electric>(p, 2 * a + (ax[a].side > 0), u, idx[0], idx[1], idx[2]);
-        acc.add(cf, pv, ax[a].type == (electric ? kPMC : kPEC) ? T(2) * phi : phi);
+        if (ax[a].type == kIFACE) pv = pv - nv[t];
+        acc.add(cf, pv, ax[a].type == (electric ? kPMC : kPEC) ? (up ? T(2) : T(-2)) : (up ? T(1) : T(-1)));
         if (ax[a].type == kABS) gam += rim_gamma<T, S, electric, MUVAR>(p, a, se, sm);
     }
     if (electric && J) {
@@ -483,7 +476,21 @@ __device__ __forceinline__ void rim_gather(const Params<T, S> &p, const RimAxis<
         const I q = o + x.off;
         v[t].a = ld_s(F + q);
         v[t].b = ld_s(F + (I)(q + x.st));
-        v[t].c = x.k[2] != T(0) ? ld_s(F + (I)(q + x.st + x.st)) : T(0);
+        v[t].c = x.closure ? ld_s(F + (I)(q + x.st + x.st)) : T(0);
+    }
+}
+
+// The partner's values of component C's two curl fields, where the term's axis
+// faces an interface.  on: offsets of the node on the partner's faces per axis.
+template <int C, typename I, typename T, typename S>
+__device__ __forceinline__ void rim_partners(const Params<T, S> &p, const RimAxis<I, T> (&ax)[3], const long long (&on)[3],
+                                             T (&nv)[2])
+{
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int a = curl_axis(C, t);
+        if (ax[a].type == kIFACE)
+            nv[t] = link_value<false, T, S>(p.link[2 * a + (ax[a].side > 0)], curl_comp(C, t), on[a]);
     }
 }
 
@@ -529,12 +536,29 @@ __device__ __forceinline__ void rim_node(const Params<T, S> &p, S *const (&out)[
     rim_gather<c0 + 1>(p, ax, o, vy);
     rim_gather<c0 + 2>(p, ax, o, vz);
     T x = ld_s(p.F[c0] + o), y = ld_s(p.F[c0 + 1] + o), z = ld_s(p.F[c0 + 2] + o);
+    // partner values with the other loads: fetched one by one where each is used,
+    // they were most of a small periodic pair's half-step
+    T nx2[2] = {T(0), T(0)}, ny2[2] = {T(0), T(0)}, nz2[2] = {T(0), T(0)};
+    if (ax[0].type == kIFACE || ax[1].type == kIFACE || ax[2].type == kIFACE) {
+        long long on[3] = {0, 0, 0};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (ax[a].type != kIFACE) continue;
+            const Link &L = p.link[2 * a + (ax[a].side > 0)];
+            const int nidx = L.side < 0 ? 0 : ELECTRIC ? L.n_norm + 1 : L.n_norm;
+            on[a] = (long long)(a == 0 ? nidx : i) + (long long)(a == 1 ? nidx : j) * L.sy +
+                    (long long)(a == 2 ? nidx : k) * L.sz;
+        }
+        rim_partners<c0>(p, ax, on, nx2);
+        rim_partners<c0 + 1>(p, ax, on, ny2);
+        rim_partners<c0 + 2>(p, ax, on, nz2);
+    }
     T ex = T(0), ey = T(0), ez = T(0), mx = T(0), my = T(0), mz = T(0);
     if (ELECTRIC || abs) rim_cells<ELECTRIC>(p.eps, o, sy, sz, ex, ey, ez);
     if (MUVAR && (!ELECTRIC || abs)) rim_cells<ELECTRIC>(p.mu, o, sy, sz, mx, my, mz);
-    x = rim_apply<T, c0, MUVAR>(p, ax, idx, x, vx, ex, mx, marks.J);
-    y = rim_apply<T, c0 + 1, MUVAR>(p, ax, idx, y, vy, ey, my, marks.J);
-    z = rim_apply<T, c0 + 2, MUVAR>(p, ax, idx, z, vz, ez, mz, marks.J);
+    x = rim_apply<T, c0, MUVAR>(p, ax, idx, x, vx, nx2, ex, mx, marks.J);
+    y = rim_apply<T, c0 + 1, MUVAR>(p, ax, idx, y, vy, ny2, ey, my, marks.J);
+    z = rim_apply<T, c0 + 2, MUVAR>(p, ax, idx, z, vz, nz2, ez, mz, marks.J);
     // nodes of each component (Table I); the others are not stored and hold no probe
     const int e = ELECTRIC ? 1 : 0;
     if (i <= nx + e && j <= ny + 1 - e && k <= nz + 1 - e) st_s(out[0] + o, x);
@@ -588,7 +612,8 @@ __device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w,
 template <bool ELECTRIC, bool MUVAR, int V, typename I, typename T, typename S>
 __device__ __forceinline__ void half_cta(const Params<T, S> &p, const Sweep &w, When when, unsigned cta)
 {
-    const unsigned r = cta < w.cz ? 0u : cta - w.cz, chunk = r / w.dchunk, q = r - chunk * w.cchunk;
+    const unsigned r = cta < w.cz ? 0u : cta - w.cz, c = r / w.dchunk, q = r - c * w.cchunk;
+    const unsigned chunk = w.flip ? w.flip - c : c;
     if (cta >= w.cz && q < w.cbox) {
         if constexpr (ELECTRIC) box_e<I, T, S, V>(p, w, when, q, (int)chunk);
         else box_h<I, T, S, MUVAR, V>(p, w, when, q, (int)chunk);

@@ -447,6 +447,11 @@ int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool
     w.cz = (unsigned)cz;
     w.cbox = (unsigned)cbox;
     w.cchunk = (unsigned)cchunk;
+    // E takes the chunks from the last to the first: it starts on the planes that
+    // the H launch before left in L2, and the next H on those that E leaves (256^3
+    // 214 -> 211 us per step, two blocks 192x192x96 117 -> 116; a grid many times
+    // L2 gains nothing: 512^3 in FP16 storage 1036 -> 1052)
+    w.flip = electric && !onepass && planes * rows * xs < 64000000 ? (unsigned)((planes + kz - 1) / kz - 1) : 0u;
     w.ctas = (unsigned)ctas;
     w.dnv = fast_div(w.nv);
     w.dxs = fast_div(w.xs);
@@ -461,7 +466,9 @@ int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool
 // nodes of the grid.  us per step, FP32, as V:planes (CTAs of 128 threads; 256 are
 // slower everywhere, fewer warps fit beside the register use):
 //   nodes          1:1    1:2    2:2    2:4    2:8    4:4    4:8    4:16
-//   125 k          8.0   10.1   13
+//   33 k           7.5    6.6    6.6    7.4
+//   125 k          7.8    8.2    7.9    8.7
+//   200 k         10.2    8.5    8.7    9.4
 //   0.29 M (64^3) 12.5   11.4    9.6    9.3   13.2   10.5   15.1   23.6
 //   0.57 M (82^3) 17.9   15.5   13.4   13.4   15.0   14.0   18.5   27.6
 //   1.6 M         35.2   28.9   23.4   21.8   23.5   22.7   27.0   36.1
@@ -469,14 +476,13 @@ int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool
 //   2 x 3.7 M      197    165    126    122    125    117    123    136
 //   5.1 M          133    110   82.7   80.2   81.1   76.2   78.1   84.9
 //   17 M (256^3)   383    332    242    234    231    214    214    223
-// FP16 storage at 512^3: 4:16 1036, 4:8 1064.  FP64 is bound by its pipe: one node
+// FP16 storage at 512^3: 4:16 1036, 4:8 1064 (before E held 80 registers).  FP64 is bound by its pipe: one node
 // per thread, 1 or 2 planes (2 nodes: 1 % slower).
 int choose_sweep(sbp_sim *s)
 {
     const long long nodes = (long long)(s->n[0] + 2) * (s->n[1] + 2) * (s->n[2] + 2);
-    int v = 4, kz = nodes > 64000000 ? 16 : 4;
-    if (nodes < 200000) v = kz = 1;
-    else if (s->prec == SBP_FP64) { v = 1; kz = 2; }
+    int v = 4, kz = nodes < 200000 ? 2 : nodes > 64000000 ? 16 : 4;
+    if (s->prec == SBP_FP64) { v = 1; kz = nodes < 200000 ? 1 : 2; }
     else if (nodes < 2500000 && s->prec == SBP_FP32) v = 2;
     // arrays of 2^32 elements and more (with room for the offsets past the last
     // plane) index with 64 bits; tests ask for it on small grids
@@ -494,7 +500,7 @@ int choose_sweep(sbp_sim *s)
 // pays where the grid is far larger than L2 (per step, FP32, one pass / in place:
 // 61 x 47 x 38 17.6 / 7.8 us, 117 x 96 x 131 39 / 21.8 us, 256^3 236 / 214 us,
 // 512^3 1423 / 1600 us).  With FP16 storage one pass is issue-bound (512^3: 1337 /
-// 1036 us) and never pays.
+// 997 us) and never pays.
 constexpr long long kOnePassNodes = 24000000;
 
 int setup(sbp_sim *s, const sbp_grid_desc *d, const Layout &L, char *ws)
@@ -730,15 +736,13 @@ int launch_half(const sbp_sim *s, bool h)
 {
     using U = unsigned;
     using L = long long;
-    const int v = s->sweep_v;
     if (s->prec == SBP_FP64)
         return s->sweep_big ? launch_half_t<L, double, double, 1>(s, h) : launch_half_t<U, double, double, 1>(s, h);
     if (s->prec == SBP_FP32_FP16STORE)
         return s->sweep_big ? launch_half_t<L, float, __half, 4>(s, h)
-             : v > 1        ? launch_half_t<U, float, __half, 4>(s, h) : launch_half_t<U, float, __half, 1>(s, h);
+                            : launch_half_t<U, float, __half, 4>(s, h);
     return s->sweep_big ? launch_half_t<L, float, float, 4>(s, h)
-         : v == 4       ? launch_half_t<U, float, float, 4>(s, h)
-         : v == 2       ? launch_half_t<U, float, float, 2>(s, h) : launch_half_t<U, float, float, 1>(s, h);
+         : s->sweep_v == 4 ? launch_half_t<U, float, float, 4>(s, h) : launch_half_t<U, float, float, 2>(s, h);
 }
 
 // Parameters of the one-pass interior step reading set `old`, writing set old^1.
@@ -1074,7 +1078,8 @@ int step_group(sbp_sim **sims, int nsims, int64_t nsteps)
             rc = s->fused_step ? launch_fused_phase1(s, !linked_to_other(s)) : launch_half(s, true);
             if (rc) return rc;
         }
-        for (int q = 0; q < nsims; q++) {
+        // (the last block's H is the one still in L2)
+        for (int q = nsims - 1; q >= 0; q--) {
             sbp_sim *s = sims[q];
             if (s->fused_step) {
                 if (!linked_to_other(s)) continue;
@@ -1538,13 +1543,11 @@ int batch_launch_chunk(sbp_batch *b, long long K)
         for (const sbp_batch::Group &G : b->groups)
             for (long long o = 0; o < K; o++) {
                 const bool first = G.first == 0 && o == 0;
-                int rc = G.v == 1   ? launch_half_batched<false, 1>(b, G, (int)o, first)
-                         : G.v == 2 ? launch_half_batched<false, 2>(b, G, (int)o, first)
-                                    : launch_half_batched<false, 4>(b, G, (int)o, first);
+                int rc = G.v == 2 ? launch_half_batched<false, 2>(b, G, (int)o, first)
+                                  : launch_half_batched<false, 4>(b, G, (int)o, first);
                 if (!rc)
-                    rc = G.v == 1   ? launch_half_batched<true, 1>(b, G, (int)o, false)
-                         : G.v == 2 ? launch_half_batched<true, 2>(b, G, (int)o, false)
-                                    : launch_half_batched<true, 4>(b, G, (int)o, false);
+                    rc = G.v == 2 ? launch_half_batched<true, 2>(b, G, (int)o, false)
+                                  : launch_half_batched<true, 4>(b, G, (int)o, false);
                 if (rc) return rc;
             }
     }

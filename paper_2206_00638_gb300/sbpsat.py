@@ -86,6 +86,8 @@ class GridDesc(C.Structure):
 def lib():
     """Load libsbpsat.so (building it first if needed).  Raises if it cannot."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = LIB_PATH if os.path.exists(LIB_PATH) else build()
@@ -231,6 +233,7 @@ class Sim:
         self._keep.clear()
         self._h = h_out.value
         self.nprobes = 0
+        self._shapes = [extents(self.n, c)[::-1] for c in range(6)]
 
     # --- lifetime -------------------------------------------------------
     def close(self):
@@ -251,8 +254,7 @@ class Sim:
 
     # --- problem statement ----------------------------------------------
     def shape(self, comp):
-        e = extents(self.n, comp)
-        return (e[2], e[1], e[0])
+        return self._shapes[comp]
 
     def connect(self, face, other: "Sim", other_face):
         _check(lib().sbp_connect(self._h, int(face), other._h, int(other_face)), "sbp_connect")

@@ -28,12 +28,10 @@ namespace sbp {
 constexpr int kSweepThreads = 128;        // threads of a CTA
 
 // CTAs of a half-step that fit an SM, by registers: 72 a thread in FP32 (76-80 left
-// to the compiler cost 8 % at 117 x 96 x 131), 80 for E in vectors of 4 (96: 512^3
-// in FP16 storage 1048 us per step, 997 now), 112 and more in FP64.
-template <typename T, int V> constexpr int half_ctas(bool electric)
-{
-    return sizeof(T) == 8 ? 4 : V == 4 && electric ? 6 : 7;
-}
+// to the compiler cost 8 % at 117 x 96 x 131; E in vectors of 4, which would take
+// 96: 1048 us per step at 512^3 in FP16 storage, 997 at 80 registers, 964 at 72),
+// 112 and more in FP64.
+template <typename T> constexpr int kHalfCtas = sizeof(T) == 8 ? 4 : 7;
 
 // n / d for n < 2^31, with the multiplier of d found on the host.
 struct FastDiv { unsigned mul, shift; };
@@ -641,7 +639,7 @@ __global__ void __launch_bounds__(kSweepThreads, 7)
 }
 
 template <typename I, typename T, typename S, bool MUVAR, int V>
-__global__ void __launch_bounds__(kSweepThreads, half_ctas<T, V>(false))
+__global__ void __launch_bounds__(kSweepThreads, kHalfCtas<T>)
     half_h(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
 {
     pdl_release();
@@ -649,7 +647,7 @@ __global__ void __launch_bounds__(kSweepThreads, half_ctas<T, V>(false))
 }
 
 template <typename I, typename T, typename S, bool MUVAR, int V>
-__global__ void __launch_bounds__(kSweepThreads, half_ctas<T, V>(true))
+__global__ void __launch_bounds__(kSweepThreads, kHalfCtas<T>)
     half_e(const __grid_constant__ Params<T, S> p, const __grid_constant__ Sweep w)
 {
     pdl_release();
@@ -681,7 +679,7 @@ struct alignas(16) BatchHalf {
 };
 
 template <bool ELECTRIC, int V>
-__global__ void __launch_bounds__(kSweepThreads, half_ctas<float, V>(ELECTRIC))
+__global__ void __launch_bounds__(kSweepThreads, kHalfCtas<float>)
     half_batched(const BatchHalf *grids, const int *pre, int n, int offset)
 {
     __shared__ __align__(16) Params<float> p;
@@ -706,7 +704,7 @@ __global__ void __launch_bounds__(kSweepThreads, half_ctas<float, V>(ELECTRIC))
 // One member of a batch alone: its parameters are the launch's, which cost a CTA
 // no copy (a grid that fills the GPU by itself steps 1.3 times faster so).
 template <bool ELECTRIC, int V>
-__global__ void __launch_bounds__(kSweepThreads, half_ctas<float, V>(ELECTRIC))
+__global__ void __launch_bounds__(kSweepThreads, kHalfCtas<float>)
     half_member(const __grid_constant__ Params<float> p, const __grid_constant__ Sweep w, const long long *counter,
                 long long target, long long probe_base, int offset)
 {

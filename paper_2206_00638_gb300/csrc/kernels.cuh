@@ -674,13 +674,16 @@ __device__ __forceinline__ double energy_h(const Params<T, S> &p, long long o, f
 template <typename T, typename S, bool MUVAR>
 __global__ void __launch_bounds__(kBlockX *kBlockY) energy_sum(const Params<T, S> p)
 {
-    const int i = blockIdx.x * kBlockX + threadIdx.x;
     const int j = blockIdx.y * kBlockY + threadIdx.y;
     const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
+    // x nodes in the order 3 .. nx-2, then the six ends: all but the last warps of a
+    // row then hold two-point rows only (at 160 cells 4 of 6 warps, 3 in the plain order)
+    const int at = blockIdx.x * kBlockX + threadIdx.x, inner = nx - 4, end = at - inner;
+    const int i = at < inner ? at + 3 : end < 3 ? end : nx - 4 + end;
     const int k0 = blockIdx.z * p.kchunk;
     const int k1 = min(k0 + p.kchunk, nz + 2);
     double se = 0.0, sh = 0.0;
-    if (i < nx + 2 && j < ny + 2) {
+    if (at < nx + 2 && j < ny + 2) {
         const S *__restrict__ Hx = p.F[3];
         const S *__restrict__ Hy = p.F[4];
         const S *__restrict__ Hz = p.F[5];
@@ -690,8 +693,7 @@ __global__ void __launch_bounds__(kBlockX *kBlockY) energy_sum(const Params<T, S
         const long long sy = p.sy, sz = p.sz;
         long long o = (long long)k0 * sz + (long long)j * sy + i;
         // the warp's row lies inside the box of two-point rows along x and y
-        const bool inside = (int)blockIdx.x * kBlockX >= 3 && (int)blockIdx.x * kBlockX + kBlockX - 1 <= nx - 2 && j >= 3 &&
-                            j <= ny - 2;
+        const bool inside = (int)blockIdx.x * kBlockX + kBlockX <= inner && j >= 3 && j <= ny - 2;
         const Coef<T> Bx = p.B[0], By = p.B[1], Bz = p.B[2];
         double qa, qb, qc;
         eps_pair_sums(p.eps + o, sy, qa, qb, qc);

@@ -476,7 +476,7 @@ int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool
 //   2 x 3.7 M      197    165    126    122    125    117    123    136
 //   5.1 M          133    110   82.7   80.2   81.1   76.2   78.1   84.9
 //   17 M (256^3)   383    332    242    234    231    214    214    223
-// FP16 storage at 512^3: 4:16 1036, 4:8 1064 (before E held 80 registers).  FP64 is bound by its pipe: one node
+// FP16 storage at 512^3: 4:16 1036, 4:8 1064 (before E held 72 registers).  FP64 is bound by its pipe: one node
 // per thread, 1 or 2 planes (2 nodes: 1 % slower).
 int choose_sweep(sbp_sim *s)
 {
@@ -498,9 +498,9 @@ int choose_sweep(sbp_sim *s)
 // half-steps).  One pass moves 13 words per node instead of 19, but marches
 // planes behind a barrier and leaves the boundary to launches of its own, so it
 // pays where the grid is far larger than L2 (per step, FP32, one pass / in place:
-// 61 x 47 x 38 17.6 / 7.8 us, 117 x 96 x 131 39 / 21.8 us, 256^3 236 / 214 us,
+// 61 x 47 x 38 17.6 / 7.8 us, 117 x 96 x 131 39 / 21.8 us, 256^3 236 / 207 us,
 // 512^3 1423 / 1600 us).  With FP16 storage one pass is issue-bound (512^3: 1337 /
-// 997 us) and never pays.
+// 964 us) and never pays.
 constexpr long long kOnePassNodes = 24000000;
 
 int setup(sbp_sim *s, const sbp_grid_desc *d, const Layout &L, char *ws)

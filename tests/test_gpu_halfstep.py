@@ -46,3 +46,35 @@ def test_bitwise_equal_to_one_pass(n, precision, monkeypatch):
         s.close()
     for a, b, c in zip(*out):
         assert np.array_equal(a, b) and np.array_equal(a, c)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_joined_blocks_bitwise_on_both_paths(axis, monkeypatch):
+    w = wl.coupled_boxes((26, 33, 21), (26, 33, 21), axis, seed=3)
+    out = []
+    for path in ("onepass", "inplace"):
+        monkeypatch.setenv("SBP_STEP_PATH", path)
+        sims = parity.gpu_run(w, 7, sbpsat.FP32)
+        out.append([s.field(c) for s in sims for c in range(6)])
+        for s in sims:
+            s.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+def test_steps_replay_from_a_captured_graph():
+    """Half-steps launched with a programmatic dependency can be captured: replays step on."""
+    stream = torch.cuda.Stream()
+    w = wl.random_box((40, 31, 28), seed=9, sources=False, nprobes=0)
+    with torch.cuda.stream(stream):
+        a = sbpsat.from_workload(w, stream=stream)[0]
+        b = sbpsat.from_workload(w, stream=stream)[0]
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            a.step(3)
+        g.replay()
+        g.replay()
+        b.step(6)
+        for c in range(6):
+            assert np.array_equal(a.field(c), b.field(c))

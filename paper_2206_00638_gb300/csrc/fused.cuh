@@ -19,9 +19,10 @@
 // z-plane, completion on an mbarrier) keeps three planes in flight; H^{n+1/2}
 // of the current and next plane is exchanged through shared memory.
 //
-// band_h / band_e evaluate the remaining nodes (the three boundary layers of
-// each axis, closure rows and SAT penalties) with the general-path code of
-// kernels.cuh, reading the old set and writing the new one.
+// The remaining nodes (the three boundary layers of each axis, closure rows and
+// SAT penalties) are rim_step's (halfstep.cuh), reading the old set and writing
+// the new one; band_h / band_e do the same by slabs for the Yee comparator, and
+// their node code for the persistent batched kernel.
 #pragma once
 #include <cuda.h>
 

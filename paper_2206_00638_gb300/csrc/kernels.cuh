@@ -423,11 +423,6 @@ __device__ __forceinline__ void eps_pair_sums(const float *__restrict__ m, long 
     b = f + fx;
     c = g + gx;
 }
-// number of entries summed by cell_sum<C>
-__host__ __device__ constexpr int cell_count(int c)
-{
-    return (on_plus(c, 0) ? 2 : 1) * (on_plus(c, 1) ? 2 : 1) * (on_plus(c, 2) ? 2 : 1);
-}
 
 // Source waveforms (Sec. VI-B, VI-C): t and t0, tw in seconds.  A call, not
 // inlined: a few lanes of a launch reach it, and its code would sit between the

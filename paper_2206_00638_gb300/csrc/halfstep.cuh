@@ -552,8 +552,11 @@ __device__ __forceinline__ void rim_node(const Params<T, S> &p, S *const (&out)[
         rim_partners<c0 + 2>(p, ax, on, nz2);
     }
     T ex = T(0), ey = T(0), ez = T(0), mx = T(0), my = T(0), mz = T(0);
-    if (ELECTRIC || abs) rim_cells<ELECTRIC>(p.eps, o, sy, sz, ex, ey, ez);
-    if (MUVAR && (!ELECTRIC || abs)) rim_cells<ELECTRIC>(p.mu, o, sy, sz, mx, my, mz);
+    // the last plane repeats its own cells: no component there spans two cells along z,
+    // and the arrays' slack plane does not hold a step along y and z together
+    const I dz = k <= nz ? sz : I(0);
+    if (ELECTRIC || abs) rim_cells<ELECTRIC>(p.eps, o, sy, dz, ex, ey, ez);
+    if (MUVAR && (!ELECTRIC || abs)) rim_cells<ELECTRIC>(p.mu, o, sy, dz, mx, my, mz);
     x = rim_apply<T, c0, MUVAR>(p, ax, idx, x, vx, nx2, ex, mx, marks.J);
     y = rim_apply<T, c0 + 1, MUVAR>(p, ax, idx, y, vy, ny2, ey, my, marks.J);
     z = rim_apply<T, c0 + 2, MUVAR>(p, ax, idx, z, vz, nz2, ez, mz, marks.J);

@@ -696,7 +696,8 @@ __global__ void __launch_bounds__(kBlockX *kBlockY) energy_sum(const Params<T, S
             const T ex = ldg_s(Ex + o), ey = ldg_s(Ey + o), ez = ldg_s(Ez + o);
             const T hx = ldg_s(Hx + o), hy = ldg_s(Hy + o), hz = ldg_s(Hz + o);
             double na, nb, nc;
-            eps_pair_sums(p.eps + o + sz, sy, na, nb, nc);
+            // (the last plane again at the end: no E node there spans two cells along z)
+            eps_pair_sums(p.eps + o + (k <= nz ? sz : 0), sy, na, nb, nc);
             if (inside && k >= 3 && k <= nz - 2) {
                 const T exj = ldg_s(Ex + o - sy), exk = ldg_s(Ex + o - sz), eyi = ldg_s(Ey + o - 1);
                 const T eyk = ldg_s(Ey + o - sz), ezi = ldg_s(Ez + o - 1), ezj = ldg_s(Ez + o - sy);

@@ -32,6 +32,19 @@ void rims(Host &g, int face)
     launch({we.ctas, 1, 1}, block, [&] { sbp::rim_step<true, float>(p, we, out[0], out[1], out[2]); });
 }
 
+template <typename T, bool MU> void energy(Host &g, int face)
+{
+    auto p = g.params<T>(face, MU);
+    const Dim block = {sbp::kBlockX, sbp::kBlockY, 1};
+    for (int kc : {3, 8}) {
+        const Dim grid = {(g.n[0] + 2 + block.x - 1) / block.x, (g.n[1] + 2 + block.y - 1) / block.y,
+                          (unsigned)(g.n[2] + 2 + kc - 1) / kc};
+        p.kchunk = kc;
+        p.partials = guarded<double>(grid.x * grid.y * grid.z);
+        launch(grid, block, [&] { sbp::energy_sum<T, T, MU>(p); });
+    }
+}
+
 int main(int argc, char **argv)
 {
     const int n[3] = {std::atoi(argv[2]), std::atoi(argv[3]), std::atoi(argv[4])}, face = std::atoi(argv[5]);
@@ -39,6 +52,7 @@ int main(int argc, char **argv)
     const char what = argv[1][0];
     if (what == 'h') { halves<float, false>(g, face); halves<double, true>(g, face); halves<float, true>(g, face); }
     if (what == 'r') rims(g, face);
+    if (what == 'e') { energy<float, false>(g, face); energy<double, true>(g, face); }
     return 0;
 }
 """
@@ -62,3 +76,9 @@ def test_half_steps_stay_inside(replay, n, face):
 @pytest.mark.parametrize("n", [m for m in GRIDS if min(m) >= 8])
 def test_rim_of_one_pass_steps_stays_inside(replay, n, face):
     assert replay("rim", n, face) == 0
+
+
+@pytest.mark.parametrize("face", FACES)
+@pytest.mark.parametrize("n", GRIDS)
+def test_energy_stays_inside(replay, n, face):
+    assert replay("energy", n, face) == 0

@@ -676,9 +676,10 @@ __device__ __forceinline__ void band_e_at(const Params<T, S> &p, const int idx[3
     e_gather<T, 1, CG, G>(p, idx, o, vy);
     e_gather<T, 2, CG, G>(p, idx, o, vz);
     const T ex = ldf<CG>(p.F[0] + o), ey = ldf<CG>(p.F[1] + o), ez = ldf<CG>(p.F[2] + o);
-    const T sx = cell_sum<0, T>(p.eps, o, p.sy, p.sz);
-    const T sy = cell_sum<1, T>(p.eps, o, p.sy, p.sz);
-    const T sz = cell_sum<2, T>(p.eps, o, p.sy, p.sz);
+    // (the arrays' slack plane does not hold a step along z together with one along y or a last x)
+    const T sx = have[0] ? cell_sum<0, T>(p.eps, o, p.sy, p.sz) : T(1);
+    const T sy = have[1] ? cell_sum<1, T>(p.eps, o, p.sy, p.sz) : T(1);
+    const T sz = have[2] ? cell_sum<2, T>(p.eps, o, p.sy, p.sz) : T(1);
     if (have[0]) st_s(outs[0] + o, en[0] = quant<S>(e_apply<T, 0, MUVAR, false, G>(p, idx, o, ex, sx, vx, sm, J)));
     if (have[1]) st_s(outs[1] + o, en[1] = quant<S>(e_apply<T, 1, MUVAR, false, G>(p, idx, o, ey, sy, vy, sm, J)));
     if (have[2]) st_s(outs[2] + o, en[2] = quant<S>(e_apply<T, 2, MUVAR, false, G>(p, idx, o, ez, sz, vz, sm, J)));

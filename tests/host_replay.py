@@ -178,7 +178,24 @@ template <typename T> T *guarded(size_t n)
 """
 
 HELPERS = r"""
-// A grid's arrays and parameters as the library lays them out.
+// A grid's band, arrays and parameters as the library lays them out.
+sbp::Band make_band(const int n[3], bool electric)
+{
+    sbp::Band b;
+    b.lo = electric ? 3 : 4;
+    for (int a = 0; a < 3; a++) b.hi[a] = n[a] - 3;
+    b.segs = b.hi[0] / 32 + 1;
+    b.zplanes = b.lo + (n[2] + 1 - b.hi[2]);
+    b.yrows = b.lo + (n[1] + 1 - b.hi[1]);
+    b.jin = b.hi[1] - b.lo + 1;
+    b.xgroups = (n[1] + 2 + 7) / 8;
+    b.wz = b.zplanes * b.jin * b.segs;
+    b.wy = (n[2] + 2) * b.yrows * b.segs;
+    b.wx = (n[2] + 2) * b.xgroups * 2;
+    b.ctas = (b.wz + b.wy + b.wx + 7) / 8;
+    return b;
+}
+
 struct Host {
     int n[3];
     long long sy, sz;

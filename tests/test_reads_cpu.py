@@ -45,6 +45,20 @@ template <typename T, bool MU> void energy(Host &g, int face)
     }
 }
 
+// The slab kernels' nodes (the persistent batch's boundary, one-pass steps with 64-bit indices).
+void bands(Host &g, int face)
+{
+    auto p = g.params<float>(face, false);
+    float *out[3] = {guarded<float>(g.elems), guarded<float>(g.elems), guarded<float>(g.elems)};
+    for (bool electric : {false, true}) {
+        const sbp::Band b = make_band(g.n, electric);
+        launch({b.ctas, 1, 1}, {256, 1, 1}, [&] {
+            if (electric) sbp::band_e<float, false>(p, b, out[0], out[1], out[2]);
+            else sbp::band_h<float, false>(p, b, out[0], out[1], out[2]);
+        });
+    }
+}
+
 int main(int argc, char **argv)
 {
     const int n[3] = {std::atoi(argv[2]), std::atoi(argv[3]), std::atoi(argv[4])}, face = std::atoi(argv[5]);
@@ -52,6 +66,7 @@ int main(int argc, char **argv)
     const char what = argv[1][0];
     if (what == 'h') { halves<float, false>(g, face); halves<double, true>(g, face); halves<float, true>(g, face); }
     if (what == 'r') rims(g, face);
+    if (what == 'b') bands(g, face);
     if (what == 'e') { energy<float, false>(g, face); energy<double, true>(g, face); }
     return 0;
 }
@@ -82,3 +97,9 @@ def test_rim_of_one_pass_steps_stays_inside(replay, n, face):
 @pytest.mark.parametrize("n", GRIDS)
 def test_energy_stays_inside(replay, n, face):
     assert replay("energy", n, face) == 0
+
+
+@pytest.mark.parametrize("face", FACES)
+@pytest.mark.parametrize("n", [m for m in GRIDS if min(m) >= 8])
+def test_band_kernels_stay_inside(replay, n, face):
+    assert replay("band", n, face) == 0

@@ -664,7 +664,8 @@ __global__ void __launch_bounds__(kSweepThreads, kHalfCtas<T>)
 // before it); the step index comes from a device counter, so a captured chunk
 // of K steps can be replayed (its launches carry offsets 0..K-1, batch_advance
 // adds the steps taken).  Grids that reached their target step skip their work,
-// so a chunk may end a grid early.
+// so a chunk may end a grid early; their CTAs wait all the same, since what comes
+// after the launch is ordered behind the launch before it by that wait alone.
 //
 // The grids of a batch are independent, so a chunk need not take every grid
 // through a step before the next: it takes a group of grids, as many as stay in
@@ -699,7 +700,7 @@ __global__ void __launch_bounds__(kSweepThreads, kHalfCtas<float>)
     copy(&p, &B.p, ((int)offsetof(Params<float>, link) + 15) / 16 * 16);   // members have no links
     copy(&w, &B.w[ELECTRIC], sizeof(w));
     const long long step = *B.counter + offset;
-    if (step >= B.target) return;
+    if (step >= B.target) { pdl_wait(); return; }
     __syncthreads();
     half_cta<ELECTRIC, false, V, unsigned>(p, w, {step, step - B.probe_base}, (unsigned)((int)blockIdx.x + first - pre[g]));
 }
@@ -713,7 +714,7 @@ __global__ void __launch_bounds__(kSweepThreads, kHalfCtas<float>)
 {
     pdl_release();
     const long long step = *counter + offset;
-    if (step >= target) return;
+    if (step >= target) { pdl_wait(); return; }
     half_cta<ELECTRIC, false, V, unsigned>(p, w, {step, step - probe_base}, blockIdx.x);
 }
 

@@ -242,9 +242,10 @@ int sbp_tile(const sbp_sim *s, int *rows, int *depth, int *width);
 /* Batches: continuous batching of many simulations.  A batch advances all
  * its member simulations together.  Small members share launches, one per
  * half-step for as many grids as stay in L2 together (a table of work lists over
- * the grids); a member that fills the GPU by itself has its own.  A group runs a
- * whole chunk of steps before the next group, so its fields stay in L2, and small
- * grids fill the GPU as one large launch.  Each member keeps its own fields,
+ * the grids); a member that fills the GPU by itself has its own, and one that
+ * sbp_step takes in one pass takes the same steps here.  A group runs a whole
+ * chunk of steps before the next group, so its fields stay in L2, and small grids
+ * fill the GPU as one large launch.  Each member keeps its own fields,
  * sources, probes and step count and gives bit-identical results to
  * stepping it alone with sbp_step.  Members must be single-block FP32
  * simulations with uniform mu, at least 8 cells per axis and no interface
@@ -258,9 +259,10 @@ int sbp_tile(const sbp_sim *s, int *rows, int *depth, int *width);
  * sample at the final step); samples not taken read 0 in sbp_energy_series. */
 typedef struct sbp_batch sbp_batch;
 /* flags: SBP_BATCH_GRAPHS records each chunk (sbp_batch_step call) as a CUDA
- * graph and replays it, updated in place when the membership changes.  By
- * default a chunk advances each group of members with two launches per step
- * (the H and the E half-step, in place).  SBP_BATCH_PERSISTENT runs the whole chunk as one
+ * graph and replays it, updated in place when the membership changes (members
+ * that step in one pass stay outside it).  By default a chunk advances each group
+ * of members with two launches per step (the H and the E half-step, in place).
+ * SBP_BATCH_PERSISTENT runs the whole chunk as one
  * persistent launch instead: CTAs that stay resident take (step, work item)
  * tickets in order; an item waits only for its own grid's previous step (and
  * band E for its grid's band H), so grids at different steps overlap.  It is

@@ -682,7 +682,10 @@ struct alignas(16) BatchHalf {
     long long probe_base;
 };
 
-template <bool ELECTRIC, int V>
+// Vectors of 2: a member of the 2.5 M nodes from which vectors of 4 pay steps alone.
+constexpr int kBatchV = 2;
+
+template <bool ELECTRIC>
 __global__ void __launch_bounds__(kSweepThreads, kHalfCtas<float>)
     half_batched(const BatchHalf *grids, const int *pre, int n, int offset)
 {
@@ -702,7 +705,7 @@ __global__ void __launch_bounds__(kSweepThreads, kHalfCtas<float>)
     const long long step = *B.counter + offset;
     if (step >= B.target) { pdl_wait(); return; }
     __syncthreads();
-    half_cta<ELECTRIC, false, V, unsigned>(p, w, {step, step - B.probe_base}, (unsigned)((int)blockIdx.x + first - pre[g]));
+    half_cta<ELECTRIC, false, kBatchV, unsigned>(p, w, {step, step - B.probe_base}, (unsigned)((int)blockIdx.x + first - pre[g]));
 }
 
 // One member of a batch alone: its parameters are the launch's, which cost a CTA

@@ -1278,14 +1278,15 @@ struct sbp_batch {
         double *mirror;          // pinned host copy of the latest energy sample (serving), or null
     };
     struct Group {                      // members that run a chunk together
-        int first, n, v;
+        int first, n, v;                // v: vector width of a member that runs by itself
         unsigned ctas[2];
-        const sbp::BatchHalf *alone;    // the member (staging) when it runs by itself
+        const sbp::BatchHalf *alone;    // that member (staging), or null
     };
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;  // private stream the graph is captured on (capture runs nothing)
     int device = 0;
     std::vector<Member> m;
+    int tabled = 0;                     // members in the tables below (not those that step in one pass)
     std::vector<Group> groups;
     sbp::BatchHalf *d_half = nullptr;   // members in group order
     sbp::BatchGrid *d_grids = nullptr;  // members of a persistent batch
@@ -1368,27 +1369,30 @@ constexpr size_t kGroupBytes = 80u << 20;
 // 8 MB and 471 with no batched launches; 32 of up to 64 cells 176, 176 and 245.
 constexpr size_t kAloneBytes = 24u << 20;
 
-// Members in group order: by vector width (a launch has one), then by size, as
-// many to a group as fit kGroupBytes.
+// Members in group order: by size, as many to a group as fit kGroupBytes.  A
+// member that steps in one pass (among them every one whose elements need 64-bit
+// indices) comes last and joins no group: its steps are its own launches (512^3
+// mixed faces 1422 us per step; 1590 in place).
 int batch_groups(sbp_batch *b)
 {
     auto bytes = [](const sbp_sim *s) { return 7 * s->field_elems * sizeof(float); };
     std::stable_sort(b->m.begin(), b->m.end(), [&](const sbp_batch::Member &x, const sbp_batch::Member &y) {
-        return x.s->sweep_v != y.s->sweep_v ? x.s->sweep_v < y.s->sweep_v : bytes(x.s) < bytes(y.s);
+        return x.s->one_pass != y.s->one_pass ? y.s->one_pass : bytes(x.s) < bytes(y.s);
     });
     b->groups.clear();
     size_t held = 0;
-    for (int g = 0; g < (int)b->m.size(); g++) {
+    b->tabled = 0;
+    for (int g = 0; g < (int)b->m.size() && !b->m[g].s->one_pass; g++) {
         const sbp_sim *s = b->m[g].s;
-        const bool alone = bytes(s) > kAloneBytes;
-        if (b->groups.empty() || b->groups.back().v != s->sweep_v || alone || b->groups.back().alone ||
-            held + bytes(s) > kGroupBytes) {
+        const bool alone = bytes(s) > kAloneBytes || s->sweep_v != sbp::kBatchV;
+        if (b->groups.empty() || alone || b->groups.back().alone || held + bytes(s) > kGroupBytes) {
             b->groups.push_back({g, 0, s->sweep_v, {0u, 0u}, alone ? b->h_half + g : nullptr});
             held = 0;
         }
         sbp_batch::Group &G = b->groups.back();
         held += bytes(s);
         G.n++;
+        b->tabled++;
         for (int h = 0; h < 2; h++) {
             if ((long long)G.ctas[h] + s->sweep[h].ctas > INT32_MAX) return SBP_ECAPACITY;
             G.ctas[h] += s->sweep[h].ctas;
@@ -1397,13 +1401,28 @@ int batch_groups(sbp_batch *b)
     return SBP_OK;
 }
 
+// `steps` one-pass steps of a batch member (its parameters and field sets are the host's).
+int batch_step_one_pass(sbp_sim *s, long long steps)
+{
+    for (long long t = 0; t < steps; t++) {
+        s->fused_step = true;
+        int rc = launch_fused_phase1(s, true);
+        s->fused_step = false;
+        if (rc) return rc;
+        s->cur ^= 1;
+        s->step++;
+    }
+    return SBP_OK;
+}
+
 // Upload every member's parameters, prefix tables and step counters.
 int batch_rebuild(sbp_batch *b)
 {
-    const int n = (int)b->m.size();
-    int rc = batch_reserve(b, std::max(n, 1));
+    int rc = batch_reserve(b, std::max((int)b->m.size(), 1));
     if (rc) return rc;
     if (!b->persistent && (rc = batch_groups(b))) return rc;
+    const int n = b->persistent ? (int)b->m.size() : b->tabled;
+    b->tabled = n;
     // the previous upload must have left the pinned staging buffers
     SBP_CUDA(cudaEventSynchronize(b->staged));
     int *pre = b->h_pre;
@@ -1487,7 +1506,7 @@ int batch_rebuild(sbp_batch *b)
 // One half-step of a group at offset `offset` of a chunk.  first: the chunk's
 // first launch, which waits for everything before it (tables and counters); the
 // others may start while the launch before still runs.
-template <bool ELECTRIC, int V>
+template <bool ELECTRIC>
 int launch_half_batched(const sbp_batch *b, const sbp_batch::Group &G, int offset, bool first)
 {
     cudaLaunchAttribute at;
@@ -1501,21 +1520,21 @@ int launch_half_batched(const sbp_batch *b, const sbp_batch::Group &G, int offse
     cfg.numAttrs = first ? 0 : 1;
     if (G.alone) {
         const sbp::BatchHalf &H = G.alone[0];
-        SBP_CUDA(cudaLaunchKernelEx(&cfg, sbp::half_member<ELECTRIC, V>, H.p,
+        SBP_CUDA(cudaLaunchKernelEx(&cfg, G.v == 4 ? sbp::half_member<ELECTRIC, 4> : sbp::half_member<ELECTRIC, 2>, H.p,
                                     static_cast<const sbp::Sweep &>(H.w[ELECTRIC]), H.counter, H.target, H.probe_base,
                                     offset));
         return SBP_OK;
     }
     const sbp::BatchHalf *grids = b->d_half + G.first;
     const int *pre = b->d_pre + (ELECTRIC ? b->cap + 1 : 0) + G.first;
-    SBP_CUDA(cudaLaunchKernelEx(&cfg, sbp::half_batched<ELECTRIC, V>, grids, pre, G.n, offset));
+    SBP_CUDA(cudaLaunchKernelEx(&cfg, sbp::half_batched<ELECTRIC>, grids, pre, G.n, offset));
     return SBP_OK;
 }
 
-// K steps of every member: offsets 0..K-1, then the counters advance by K.
+// K steps of every member in the tables: offsets 0..K-1, then the counters advance by K.
 int batch_launch_chunk(sbp_batch *b, long long K)
 {
-    const int n = (int)b->m.size();
+    const int n = b->tabled;
     if (b->persistent) {
         // one launch for the whole chunk: CTAs take (step, item) tickets in
         // order, items wait only for their own grid's previous step (see
@@ -1543,11 +1562,8 @@ int batch_launch_chunk(sbp_batch *b, long long K)
         for (const sbp_batch::Group &G : b->groups)
             for (long long o = 0; o < K; o++) {
                 const bool first = G.first == 0 && o == 0;
-                int rc = G.v == 2 ? launch_half_batched<false, 2>(b, G, (int)o, first)
-                                  : launch_half_batched<false, 4>(b, G, (int)o, first);
-                if (!rc)
-                    rc = G.v == 2 ? launch_half_batched<true, 2>(b, G, (int)o, false)
-                                  : launch_half_batched<true, 4>(b, G, (int)o, false);
+                int rc = launch_half_batched<false>(b, G, (int)o, first);
+                if (!rc) rc = launch_half_batched<true>(b, G, (int)o, false);
                 if (rc) return rc;
             }
     }
@@ -2180,7 +2196,9 @@ int sbp_batch_step(sbp_batch *b, int64_t nsteps)
     if (b->m.empty() || nsteps == 0) return SBP_OK;
     int rc = SBP_OK;
     if (b->dirty && (rc = batch_rebuild(b))) return rc;
-    if (b->use_graph) {
+    if (b->tabled == 0) {
+        // every member steps in one pass (below)
+    } else if (b->use_graph) {
         if (!b->gexec || b->gK != nsteps || b->gstale) {
             // record the chunk on the private stream (nothing executes during
             // capture), then launch the graph on the batch's stream, which may
@@ -2227,12 +2245,17 @@ int sbp_batch_step(sbp_batch *b, int64_t nsteps)
     if (b->persistent)
         SBP_CUDA(cudaMemcpyAsync(b->h_err, b->d_sched + 2 * b->cap + 1, sizeof(int), cudaMemcpyDeviceToHost,
                                  b->stream));
-    // host bookkeeping: every member took min(nsteps, remaining) steps; then
-    // the energy monitor of the members that reached a sampling step
+    // host bookkeeping: every member took min(nsteps, remaining) steps (those that
+    // step in one pass take them here); then the energy monitor of the members that
+    // reached a sampling step
     for (auto &m : b->m) {
         const long long done = std::min<long long>(nsteps, std::max<long long>(0, m.target - m.s->step));
-        m.s->step += done;
-        if (b->persistent) m.s->cur ^= (int)(done & 1);
+        if (!b->persistent && m.s->one_pass) {
+            if ((rc = batch_step_one_pass(m.s, done))) return rc;
+        } else {
+            m.s->step += done;
+            if (b->persistent) m.s->cur ^= (int)(done & 1);
+        }
         if (done > 0 && (rc = batch_sample_energy(b, m))) return rc;
     }
     return SBP_OK;

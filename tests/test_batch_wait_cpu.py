@@ -26,7 +26,7 @@ int main(int argc, char **argv)
     const Dim block = {sbp::kSweepThreads, 1, 1};
     const sbp::Sweep &w = grids[0].w[1];
     if (argv[1][0] == 's')
-        launch({(unsigned)pre[2], 1, 1}, block, [&] { sbp::half_batched<true, 2>(grids, pre, 2, 2); });
+        launch({(unsigned)pre[2], 1, 1}, block, [&] { sbp::half_batched<true>(grids, pre, 2, 2); });
     else
         launch({w.ctas, 1, 1}, block, [&] { sbp::half_member<true, 2>(grids[0].p, w, counter, grids[0].target, 0, 2); });
     const long long idle = argv[1][0] == 's' ? done * w.ctas : w.ctas;

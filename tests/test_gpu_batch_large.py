@@ -1,0 +1,97 @@
+"""Batch members past the sizes of the small shared launches."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2206_00638_gb300 import sbpsat  # noqa: E402
+from paper_2206_00638_gb300 import workloads as wl  # noqa: E402
+from tests import parity  # noqa: E402
+
+P, M, A = sbpsat.PEC, sbpsat.PMC, sbpsat.ABSORBING
+H = (1e-3,) * 3
+
+
+def _driven(n, at, probes):
+    """A vacuum block driven by a point source, stepped six times as a batch's only member; its
+    probes.  In six steps the field reaches six cells, so any two such blocks agree around the source."""
+    s = sbpsat.Sim(n, H, (P,) * 6)
+    s.add_source(sbpsat.EZ, *at, sbpsat.GAUSS, 100.0, 4e-12, 4e-12)
+    for c, i, j, k in probes:
+        s.add_probe(c, i, j, k)
+    s.reserve_probes(6)
+    batch = sbpsat.Batch()
+    batch.add(s, 6)
+    batch.step(6)
+    out = s.probes()
+    batch.close()
+    s.close()
+    return out
+
+
+def test_member_of_more_than_2_to_32_elements():
+    """Planes past element 2^32 (1024 x 1024 elements a plane, from plane 4096 on) get their own
+    update, and the planes 4096 below them keep their zeros."""
+    torch.cuda.empty_cache()
+    n, high = (1022, 1022, 4128), 4110
+    if torch.cuda.mem_get_info()[0] < 235 << 30:
+        pytest.skip("needs 235 GiB of free device memory")
+    around = [(c, 500 + d, 400 - d, high + e) for c in range(6) for d in (0, 1, 2) for e in (-2, 0, 1)]
+    below = [(c, 500, 400, high - 4096 + e) for c in (0, 2, 3) for e in (-1, 0)]
+    big = _driven(n, (500, 400, high), around + below)
+    small = _driven((40, 40, 40), (20, 20, 20), [(c, i - 480, j - 380, k - high + 20) for c, i, j, k in around])
+    assert np.abs(small).max() > 0
+    assert np.array_equal(big[: len(around)], small)
+    assert not big[len(around):].any()
+
+
+@pytest.mark.parametrize("use_graphs", [True, False])
+def test_one_pass_members_beside_others(use_graphs, monkeypatch):
+    """Members that step in one pass, a batch of them alone first, then with members that step in
+    place: each gives the bits it gives alone, whichever ends first and inside a chunk."""
+    sizes = [((40, 33, 29), 17, "onepass"), ((70, 43, 37), 30, "onepass"), ((33, 20, 17), 21, "inplace"),
+             ((64, 48, 40), 40, "inplace")]
+    works = [wl.random_box(n, faces=(A, P, M, A, P, M), seed=40 + q, steps=st) for q, (n, st, _) in enumerate(sizes)]
+    alone, sims = [], []
+    for w, (_, st, path) in zip(works, sizes):
+        monkeypatch.setenv("SBP_STEP_PATH", path)
+        a = parity.gpu_run(w, st, sbpsat.FP32, energy_every=5)[0]
+        alone.append([a.field(c) for c in range(6)] + [a.probes()])
+        a.close()
+        s = sbpsat.from_workload(w, energy_every=5)[0]
+        s.reserve_probes(st)
+        sims.append(s)
+    batch = sbpsat.Batch(use_graphs=use_graphs)
+    for s, (_, st, _) in zip(sims[:2], sizes):
+        batch.add(s, st)
+    batch.step(7)
+    for s, (_, st, _) in zip(sims[2:], sizes[2:]):
+        batch.add(s, st)
+    for k in (7, 7, 7, 7, 9, 5):
+        batch.step(k)
+    for s, (_, st, _), ref in zip(sims, sizes, alone):
+        assert batch.remaining(s) == 0 and s.step_index == st
+        for c in range(6):
+            assert np.array_equal(s.field(c), ref[c]), (s.n, c)
+        assert np.array_equal(s.probes(), ref[6])
+    batch.close()
+    for s in sims:
+        s.close()
+
+
+def test_members_take_the_path_they_take_alone():
+    """The one-pass kernel's bounded waits, made to run out, are reported from a batch as from
+    sbp_step: a member whose steps go through that kernel goes through it in a batch."""
+    s = sbpsat.Sim((40, 33, 29), H, (P,) * 6, flags=sbpsat.FLAG_TEST_WAIT_TIMEOUT)
+    batch = sbpsat.Batch()
+    batch.add(s, 2)
+    batch.step(2)
+    with pytest.raises(sbpsat.SbpError) as err:
+        s.sync()
+    assert err.value.code == -5
+    batch.close()
+    s.close()

@@ -114,19 +114,16 @@ __device__ __forceinline__ void ldcells(const float *p, T (&v)[V])
     for (int q = 0; q < V; ++q) v[q] = widen<T>(f[q]);
 }
 
-// old + increment of two curl terms, in the rounding order of the general path
-// (FP64 accumulates into the old value: one operation less).
+// old + increment of two curl terms, in the rounding order of the general path.
+// (FP64 too: adding the terms to the old value one by one saves an operation of
+// three and rounds twice at the field's size.)
 template <typename S, typename T>
 __device__ __forceinline__ T advance_plain(T old, const Coef<T> &c0, T d0, const Coef<T> &c1, T d1)
 {
-    if constexpr (std::is_same<T, double>::value) {
-        return fma(-c1.hi, d1, fma(c0.hi, d0, old));
-    } else {
-        typename AccOf<T, S>::type a;
-        a.add(c0, d0);
-        a.add(c1, d1, T(-1));
-        return old + plain_increment(a);
-    }
+    typename AccOf<T, S>::type a;
+    a.add(c0, d0);
+    a.add(c1, d1, T(-1));
+    return old + plain_increment(a);
 }
 
 // Step index and probe sample slot of a launch.

@@ -160,21 +160,43 @@ __device__ __forceinline__ double to_double(float f)
 }
 __device__ __forceinline__ double to_double(double f) { return f; }
 
-// 1/s for a positive s: an FP32 approximation of the reciprocal of s's leading
-// bits (relative error d < 2^-21) corrected in FP64, r (1 + d + d^2), which
-// leaves d^3 < 2^-63 beside the rounding of the last operation.  Three FP64
-// operations; a division takes about ten, at 2 lanes per clock and SM.  Values
-// outside FP32's comfortable range divide.
+// FP32 approximation of 1/s (relative error below 2^-21) from s's leading bits,
+// widened; false outside [2^-100, 2^100), FP32's comfortable range.
+__device__ __forceinline__ bool recip_seed(double s, double &r)
+{
+    const int hi = __double2hiint(s);
+    const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(s), (unsigned)(hi - (896 << 20)), 3));
+    float q;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(f));
+    r = widen<double>(q);
+    return (unsigned)(hi - (923 << 20)) < (unsigned)(200 << 20);
+}
+
+// 1/s for a positive s: the seed r and the geometric series in its residue
+// d = 1 - s r, r (1 + d + d^2), which leaves d^3 < 2^-63 beside the rounding of
+// the last operation.  Three FP64 operations; a division takes about ten, at 2
+// lanes per clock and SM.
 __device__ __noinline__ double recip64_any(double s) { return 1.0 / s; }
 __device__ __forceinline__ double recip64(double s)
 {
-    const int hi = __double2hiint(s);
-    if ((unsigned)(hi - (923 << 20)) >= (unsigned)(200 << 20)) return recip64_any(s);    // not in [2^-100, 2^100)
-    const float f = __uint_as_float(__funnelshift_l((unsigned)__double2loint(s), (unsigned)(hi - (896 << 20)), 3));
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
-    const double rd = widen<double>(r), d = fma(-s, rd, 1.0);
-    return fma(rd, fma(d, d, d), rd);
+    double r;
+    if (!recip_seed(s, r)) return recip64_any(s);
+    const double d = fma(-s, r, 1.0);
+    return fma(r, fma(d, d, d), r);
+}
+
+// a/s for a positive s: a times a reciprocal good to 2^-42, corrected by the
+// remainder of that quotient (Markstein, IBM J. Res. Dev. 34, 1990), which leaves
+// one rounding as a division does.  Five FP64 operations.
+__device__ __noinline__ double quot64_any(double a, double s) { return a / s; }
+__device__ __forceinline__ double quot64(double a, double s)
+{
+    double r;
+    if (!recip_seed(s, r)) return quot64_any(a, s);
+    r = fma(r, fma(-s, r, 1.0), r);
+    const double q = a * r;
+    if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return q;    // infinite or NaN: no remainder
+    return fma(fma(-s, q, a), r, q);
 }
 
 // increment = r * acc with r = 1/s (E nodes, or H nodes with varying mu)
@@ -186,7 +208,7 @@ __device__ __forceinline__ float scaled_increment(const Acc<float> &a, float s)
 }
 __device__ __forceinline__ double scaled_increment(const Acc<double> &a, double s)
 {
-    return a.hi * recip64(s);
+    return quot64(a.hi, s);
 }
 __device__ __forceinline__ float plain_increment(const Acc<float> &a) { return a.hi + a.lo; }
 __device__ __forceinline__ double plain_increment(const Acc<double> &a) { return a.hi; }
@@ -209,7 +231,8 @@ __device__ __forceinline__ float scaled_increment(const AccLite &a, float s)
 }
 __device__ __forceinline__ float plain_increment(const AccLite &a) { return a.hi; }
 
-// old + acc / s (interior nodes).
+// old + acc / s (interior nodes).  FP64 multiplies by the reciprocal inside the
+// sum: its rounding and the sum's, as a quotient and a sum have.
 template <typename A>
 __device__ __forceinline__ float add_scaled(float old, const A &a, float s) { return old + scaled_increment(a, s); }
 __device__ __forceinline__ double add_scaled(double old, const Acc<double> &a, double s)
@@ -367,7 +390,7 @@ template <typename T>
 __device__ __forceinline__ T sat_finish(T old, T inc, T gam)
 {
     if (gam != T(0)) {
-        if constexpr (std::is_same<T, double>::value) return fma_t(T(1) - gam, old, inc) * recip64(T(1) + gam);
+        if constexpr (std::is_same<T, double>::value) return quot64(fma_t(T(1) - gam, old, inc), T(1) + gam);
         return fma_t(T(1) - gam, old, inc) / (T(1) + gam);
     }
     return old + inc;

@@ -37,6 +37,11 @@ template <typename T> constexpr int kHalfCtas = sizeof(T) == 8 ? 4 : 7;
 struct FastDiv { unsigned mul, shift; };
 __device__ __forceinline__ unsigned operator/(unsigned n, const FastDiv &d) { return (__umulhi(n, d.mul) + n) >> d.shift; }
 
+// n / d, for counts of rim nodes: 32-bit ones through the multiplier, 64-bit ones
+// (steps with 64-bit indices, whose layer planes may hold 2^31 nodes) by division.
+__device__ __forceinline__ unsigned quotient(unsigned n, unsigned, const FastDiv &f) { return n / f; }
+__device__ __forceinline__ unsigned long long quotient(unsigned long long n, unsigned d, const FastDiv &) { return n / d; }
+
 // Work list of one in-place half-step launch.
 struct Sweep {
     int lo[3], hi[3];         // the box, inclusive per axis; empty along an axis when hi < lo
@@ -574,30 +579,31 @@ template <typename I, typename T, typename S, bool ELECTRIC, bool MUVAR>
 __device__ __forceinline__ void sweep_rim(const Params<T, S> &p, const Sweep &w, S *const (&out)[3], When when, unsigned cta,
                                           unsigned q, int chunk)
 {
-    unsigned t, count;
+    using N = typename std::conditional<std::is_same<I, unsigned>::value, unsigned, unsigned long long>::type;
+    N t, count;
     int i, j, k;
     if (cta < w.cz) {
-        t = cta * (unsigned)kSweepThreads + threadIdx.x;
-        count = w.zplanes * w.rows * w.xs;
-        if ((t & ~31u) >= count) return;
-        const unsigned tc = min(t, count - 1u), row = tc / w.dxs, pl = row / w.drows;
+        t = (N)cta * (N)kSweepThreads + threadIdx.x;
+        count = (N)w.zplanes * w.rows * w.xs;
+        if ((t & ~(N)31) >= count) return;
+        const N tc = min(t, count - 1), row = quotient(tc, w.xs, w.dxs), pl = quotient(row, w.rows, w.drows);
         i = (int)(tc - row * w.xs);
         j = (int)(row - pl * w.rows);
         k = (int)pl < w.lo[2] ? (int)pl : w.hi[2] + 1 + ((int)pl - w.lo[2]);
     } else {
         const int kb = max(chunk * w.kz, w.lo[2]), ke = min(chunk * w.kz + w.kz - 1, w.hi[2]);
         if (kb > ke) return;
-        t = (q - w.cbox) * (unsigned)kSweepThreads + threadIdx.x;
-        count = (unsigned)(ke - kb + 1) * w.rim;
-        if ((t & ~31u) >= count) return;
-        const unsigned tc = min(t, count - 1u), pl = tc / w.drim, u = tc - pl * w.rim;
+        t = (N)(q - w.cbox) * (N)kSweepThreads + threadIdx.x;
+        count = (N)(ke - kb + 1) * w.rim;
+        if ((t & ~(N)31) >= count) return;
+        const N tc = min(t, count - 1), pl = quotient(tc, w.rim, w.drim), u = tc - pl * w.rim;
         k = kb + (int)pl;
         if (u < w.ynodes) {
-            const unsigned row = u / w.dxs;
+            const N row = quotient(u, w.xs, w.dxs);
             i = (int)(u - row * w.xs);
             j = (int)row < w.lo[1] ? (int)row : w.hi[1] + 1 + ((int)row - w.lo[1]);
         } else {
-            const unsigned row = (u - w.ynodes) / w.dends, e = u - w.ynodes - row * w.ends;
+            const N row = quotient(u - w.ynodes, w.ends, w.dends), e = u - w.ynodes - row * w.ends;
             i = (int)e < w.lo[0] ? (int)e : w.hi[0] + 1 + ((int)e - w.lo[0]);
             j = w.lo[1] + (int)row;
         }

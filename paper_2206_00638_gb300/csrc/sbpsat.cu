@@ -108,6 +108,8 @@ struct sbp_sim {
     sbp::Band band_hb, band_eb;
     sbp::Sweep sweep[2];                  // in-place half-steps: work lists (H, E) and vector width
     sbp::Sweep rim[2];                    // one-pass step: the nodes outside its kernel (H, E)
+    bool rim_ok = false;                  // rim_step takes them (the slab kernels keep the Yee comparator and
+                                          // grids that need 64-bit indices or counts)
     int sweep_v = 1;
     bool sweep_big = false;               // element indices need 64 bits
     float *eps = nullptr;
@@ -414,8 +416,9 @@ sbp::FastDiv fast_div(unsigned d)
 // Work list of an in-place half-step (electric: of E, else of H) of an n-cell
 // grid: vectors of v nodes, z-chunks of kz planes.  onepass: the part of a
 // one-pass step outside its kernel instead (H outside [4, n-3]^3, E outside
-// [3, n-3]^3), no box CTAs.
-int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool onepass = false)
+// [3, n-3]^3), no box CTAs.  *wide: it counts past what 32 bits decode (planes of
+// 3e8 nodes and more), so only the kernels with 64-bit indices take it.
+int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool onepass = false, bool *wide = nullptr)
 {
     std::memset(&w, 0, sizeof(w));
     long long box[3];
@@ -433,8 +436,9 @@ int make_sweep(const int n[3], bool electric, int v, int kz, sbp::Sweep &w, bool
     auto ctas_of = [&](long long items) { return (items + sbp::kSweepThreads - 1) / sbp::kSweepThreads; };
     const long long cz = ctas_of(zplanes * rows * xs), cbox = onepass ? 0 : ctas_of(vecs), cchunk = cbox + ctas_of(kz * rim);
     const long long ctas = cz + cchunk * ((planes + kz - 1) / kz);
-    if (std::max(std::max(zplanes * rows * xs, vecs), kz * rim) >= (1ll << 31) - 1024 || ctas >= (1ll << 31))
-        return SBP_EINVAL;
+    const long long most = (1ll << 31) - 1024;
+    if (vecs >= most || ctas >= (1ll << 31) || rows * xs >= (1ll << 32)) return SBP_EINVAL;
+    if (wide) *wide = *wide || std::max(zplanes * rows * xs, kz * rim) >= most;
     w.kz = kz;
     w.nv = (unsigned)std::max(nv, 1ll);
     w.vecs = (unsigned)vecs;
@@ -489,9 +493,12 @@ int choose_sweep(sbp_sim *s)
     s->sweep_big = s->field_elems + 2 * (size_t)s->sz >= (1ull << 32);
     if (const char *env = std::getenv("SBP_STEP_PATH")) s->sweep_big = s->sweep_big || std::strcmp(env, "inplace64") == 0;
     if (s->sweep_big && s->prec != SBP_FP64) v = 4;
+    bool wide = false;
+    int rc = make_sweep(s->n, false, v, kz, s->sweep[0], false, &wide);
+    if (!rc) rc = make_sweep(s->n, true, v, kz, s->sweep[1], false, &wide);
+    s->sweep_big = s->sweep_big || wide;      // (such grids have their vectors of 4 already)
     s->sweep_v = v;
-    int rc = make_sweep(s->n, false, v, kz, s->sweep[0]);
-    return rc ? rc : make_sweep(s->n, true, v, kz, s->sweep[1]);
+    return rc;
 }
 
 // Whether a step of this simulation runs the one-pass kernel (else the in-place
@@ -537,8 +544,10 @@ int setup(sbp_sim *s, const sbp_grid_desc *d, const Layout &L, char *ws)
     s->fused_width = L.fused_width;
     s->fused_grid = L.fused_grid;
     if (int rc = choose_sweep(s)) return rc;
+    bool wide = false;
     for (int e = 0; e < 2 && s->one_pass; e++)
-        if (int rc = make_sweep(s->n, e == 1, 1, 4, s->rim[e], true)) return rc;
+        if (int rc = make_sweep(s->n, e == 1, 1, 4, s->rim[e], true, &wide)) return rc;
+    s->rim_ok = s->one_pass && !s->fdtd && !s->sweep_big && !wide;
     char *p = ws;
     for (int set = 0; set < (L.fused ? 2 : 1); set++)
         for (int c = 0; c < 6; c++) { s->set[set][c] = p; p += L.field_bytes; }
@@ -833,9 +842,6 @@ int launch_fused_interior_t(sbp_sim *s)
     return SBP_OK;
 }
 
-// The slab kernels keep the Yee comparator and arrays that need 64-bit indices.
-bool rim_runs(const sbp_sim *s) { return s->one_pass && !s->fdtd && !s->sweep_big; }
-
 // Band H (old -> new) on stream st.
 template <typename S>
 int launch_band_h_t(sbp_sim *s, cudaStream_t st)
@@ -846,7 +852,7 @@ int launch_band_h_t(sbp_sim *s, cudaStream_t st)
     if (rc) return rc;
     const sbp::Band &bh = s->band_hb;
     S **ns = reinterpret_cast<S **>(s->set[nw]);
-    if (rim_runs(s))
+    if (s->rim_ok)
         sbp::rim_step<false, S><<<s->rim[0].ctas, sbp::kSweepThreads, 0, st>>>(p, s->rim[0], ns[3], ns[4], ns[5]);
     else
         sbp::band_h<float, false><<<bh.ctas, 256, 0, st>>>(p, bh, ns[3], ns[4], ns[5]);
@@ -864,7 +870,7 @@ int launch_band_e_t(sbp_sim *s, cudaStream_t st)
     if (rc) return rc;
     const sbp::Band &be = s->band_eb;
     S **ns = reinterpret_cast<S **>(s->set[nw]);
-    if (rim_runs(s))
+    if (s->rim_ok)
         sbp::rim_step<true, S><<<s->rim[1].ctas, sbp::kSweepThreads, 0, st>>>(p, s->rim[1], ns[0], ns[1], ns[2]);
     else
         sbp::band_e<float, false><<<be.ctas, 256, 0, st>>>(p, be, ns[0], ns[1], ns[2]);

@@ -235,7 +235,7 @@ def run_ours(args):
     nk = min(max(args.steps, 100), 400)          # steps of the per-kernel timing leg
     sim.reserve_probes(args.warmup + args.steps + nk + 8)
     if not args.no_autotune:
-        sim.autotune(20)                # tile of the one-pass step: rows and depth (state unchanged)
+        sim.autotune(20)                # tile of the one-pass step, if this grid takes it (state unchanged)
     rows, depth, width = sim.tile()
 
     with ClockSampler(local) as clk:
@@ -281,6 +281,8 @@ def run_ours(args):
     moved = {"fused_interior": BYTES_FUSED, "band_h": BYTES_H, "band_e": BYTES_E, "h_update": BYTES_H,
              "e_update": BYTES_E}
     dom = max(times, key=lambda k: times[k][0] * times[k][1])
+    if "fused_interior" not in times:
+        rows = depth = width = None     # steps in place: no tile
     tdom = times[dom][0]
     ucount, bpc = units[dom]
     mpc = BYTES16[dom] if fp16 else moved[dom]

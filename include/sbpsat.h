@@ -227,10 +227,10 @@ int sbp_step_timed(sbp_sim *s, int64_t nsteps, double *avg_ms, int64_t *launches
  * the depth and its time; sbp_tile reports the whole tile.  Synchronises the
  * stream.  A block joined to others by interface faces may be tuned: its
  * trial steps read the partners' current fields and write nothing of theirs.
- * Errors: SBP_EINVAL, SBP_ESTATE (the grid does not run the one-pass step),
+ * Errors: SBP_EINVAL, SBP_ESTATE (a grid that could never run the one-pass step),
  * SBP_ECUDA, SBP_ETIMEOUT.  Which grids step through the one-pass kernel is the
- * library's choice (large FP32 grids); for the others, which step in place, the
- * tile is kept but not used.  A persistent batch runs its members on tiles of 64
+ * library's choice (large FP32 grids); the others step in place, so their tile
+ * stays as it is and *ms_per_step is the time of such a step.  A persistent batch runs its members on tiles of 64
  * columns by 8 rows; a member's own tile is changed to it when the batch is
  * built. */
 int sbp_autotune(sbp_sim *s, int trial_steps, int *chosen_depth, double *ms_per_step);

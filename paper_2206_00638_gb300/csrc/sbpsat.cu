@@ -1192,20 +1192,32 @@ int set_tile(sbp_sim *s, int width, int rows, int depth)
     return SBP_OK;
 }
 
-// Average device time of `trials` fused steps that are not committed: each
-// writes the whole new field set and this step's probe slot, both of which
-// the next real step overwrites, and the current set is left as it was.
+// One step that is not committed, on the path that the simulation's steps take: a
+// one-pass step into the spare set, or half-steps of the spare set in place.  It
+// writes that set and this step's probe slot, both of which the next real step
+// overwrites, and the current set is left as it was.
+int trial_step(sbp_sim *s)
+{
+    if (!s->one_pass) {
+        s->cur ^= 1;
+        int rc = launch_half(s, true);
+        if (!rc) rc = launch_half(s, false);
+        s->cur ^= 1;
+        return rc;
+    }
+    const bool chain = !linked_to_other(s);
+    const int rc = launch_fused_phase1(s, chain);
+    return rc || chain ? rc : launch_fused_phase2(s);
+}
+
+// Average device time of `trials` trial steps.
 int time_trials(sbp_sim *s, int trials, cudaEvent_t e0, cudaEvent_t e1, float *ms)
 {
-    const bool chain = !linked_to_other(s);
-    int rc = launch_fused_phase1(s, chain);           // warm-up of this depth
-    if (!rc && !chain) rc = launch_fused_phase2(s);
+    int rc = trial_step(s);                           // warm-up
     if (rc) return rc;
     SBP_CUDA(cudaEventRecord(e0, s->stream));
-    for (int t = 0; t < trials; t++) {
-        if ((rc = launch_fused_phase1(s, chain))) return rc;
-        if (!chain && (rc = launch_fused_phase2(s))) return rc;
-    }
+    for (int t = 0; t < trials; t++)
+        if ((rc = trial_step(s))) return rc;
     SBP_CUDA(cudaEventRecord(e1, s->stream));
     SBP_CUDA(cudaEventSynchronize(e1));
     SBP_CUDA(cudaEventElapsedTime(ms, e0, e1));
@@ -1223,6 +1235,7 @@ int autotune(sbp_sim *s, int trials, int *chosen, double *best_ms)
     std::vector<TileChoice> cand;
     const int shapes[4][2] = {{64, 8}, {64, 16}, {128, 8}, {128, 12}};   // (width, rows)
     for (const auto &sh : shapes) {
+        if (!s->one_pass) break;                                 // steps in place: no tile to choose
         if (sh[1] > 8 && s->n[1] - 5 < sh[1] - 1) continue;      // no full tile of that height
         if (sh[0] > 64 && s->n[0] - 5 < sh[0] - 1) continue;     // nor of that width
         for (int c : {8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256})

@@ -310,7 +310,8 @@ class Sim:
     def autotune(self, trial_steps=5):
         """Choose the tile of the one-pass step (64 x 8 / 64 x 16 / 128 x 8 / 128 x 12 H
         nodes, z-block depth) by timing candidates (state unchanged); returns (depth, ms per
-        step); ``tile`` gives the whole tile."""
+        step); ``tile`` gives the whole tile.  A grid that steps in place keeps its tile, and the
+        time is of such a step."""
         depth, ms = C.c_int(), C.c_double()
         _check(lib().sbp_autotune(self._h, int(trial_steps), C.byref(depth), C.byref(ms)), "sbp_autotune")
         return depth.value, ms.value

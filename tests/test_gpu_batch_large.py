@@ -95,3 +95,67 @@ def test_members_take_the_path_they_take_alone():
     assert err.value.code == -5
     batch.close()
     s.close()
+
+
+def _members():
+    """Small members of more than one L2 group, two that step by themselves in vectors of 2, one in
+    vectors of 4 (2.5 M nodes), and targets that end inside chunks."""
+    sizes = [(33, 20, 17), (88, 88, 86), (86, 90, 88), (91, 85, 87), (87, 89, 90), (84, 92, 88), (101, 100, 99),
+             (117, 96, 131), (142, 135, 140), (8, 9, 8)]
+    steps = [13, 21, 16, 9, 24, 17, 23, 11, 15, 5]
+    rng = np.random.default_rng(7)
+    out = []
+    for q, (n, st) in enumerate(zip(sizes, steps)):
+        faces = tuple(int(v) for v in rng.choice([P, M, A], size=6))
+        out.append(wl.random_box(n, faces=faces, seed=60 + q, steps=st))
+    return out
+
+
+@pytest.mark.parametrize("use_graphs", [True, False])
+def test_groups_and_lone_members_equal_alone(use_graphs):
+    """Shared launches of several groups, members alone in a launch, and members that leave and join
+    between chunks: every one with the bits it has alone."""
+    works = _members()
+    sims = []
+    for w in works:
+        sims.append(sbpsat.from_workload(w)[0])
+        sims[-1].reserve_probes(w.steps)
+    batch = sbpsat.Batch(use_graphs=use_graphs)
+    late = (2, 8)
+    for q, (s, w) in enumerate(zip(sims, works)):
+        if q not in late:
+            batch.add(s, w.steps)
+    batch.step(6)
+    for q in late:
+        batch.add(sims[q], works[q].steps)
+    batch.remove(sims[9])                                  # done: its target was 5
+    for k in (8, 8, 8):
+        batch.step(k)
+    for q, (s, w) in enumerate(zip(sims, works)):
+        assert s.step_index == w.steps and (q == 9 or batch.remaining(s) == 0)
+        alone = parity.gpu_run(w, w.steps, sbpsat.FP32)[0]
+        for c in range(6):
+            assert np.array_equal(s.field(c), alone.field(c)), (w.blocks[0].n, c)
+        assert np.array_equal(s.probes(), alone.probes())
+        alone.close()
+    batch.close()
+
+
+@pytest.mark.parametrize("n", [(48, 40, 33), (117, 96, 131), (142, 135, 140)])
+@pytest.mark.parametrize("use_graphs", [True, False])
+def test_last_member_ends_one_step_before_the_chunk(n, use_graphs):
+    """The chunk's last launches are those of a finished member: fields read right after are whole."""
+    w = wl.random_box(n, faces=(A, P, M, A, P, M), seed=71, steps=7)
+    alone = parity.gpu_run(w, 7, sbpsat.FP32)[0]
+    ref = [alone.field(c) for c in range(6)]
+    for _ in range(3):
+        s = sbpsat.from_workload(w)[0]
+        s.reserve_probes(7)
+        batch = sbpsat.Batch(use_graphs=use_graphs)
+        batch.add(s, 7)
+        batch.step(8)
+        for c in range(6):
+            assert np.array_equal(s.field(c), ref[c]), c
+        batch.close()
+        s.close()
+    alone.close()

@@ -152,7 +152,8 @@ int sbp_connect_phase(sbp_sim *re, sbp_sim *im, int axis, double alpha);
 
 /* Copy one component (natural extents, x fastest) into the simulation.
  * src: host pointer (is_device = 0, copied before return) or device pointer
- * (is_device = 1, read asynchronously on the simulation's stream). */
+ * (is_device = 1, read asynchronously on the simulation's stream).  SBP_ECUDA
+ * also when the device array does not fit its allocation. */
 int sbp_set_field(sbp_sim *s, int comp, const void *src, int is_device);
 
 /* Copy one component out (natural extents).  to_device = 0: dst is host

@@ -352,17 +352,22 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_
                                    const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// A driver function, or null.
+void *driver_entry(const char *name, unsigned version)
+{
+    void *ptr = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion(name, &ptr, version, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+        return ptr;
+    (void)cudaGetLastError();
+    return nullptr;
+}
+
 EncodeTiledFn encode_fn()
 {
     static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void *ptr = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            return nullptr;
-        fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
+    if (!fn) fn = reinterpret_cast<EncodeTiledFn>(driver_entry("cuTensorMapEncodeTiled", 12000));
     return fn;
 }
 
@@ -1644,19 +1649,27 @@ int get_dense(const sbp_sim *s, int comp, const int e[3], void *dense)
     return launch_move<false, float, float>(s, e, f, dense, 1.0);
 }
 
-// True when a kernel on the simulation's device can address the caller's
-// array: device or managed memory there, aligned to its elements.  Anything
-// else a copy call takes (another device's memory, pinned host memory) keeps
-// going through the copy engine.
-bool kernel_reachable(const sbp_sim *s, const void *ptr)
+// How a field copy reaches the caller's device array: by a kernel (device or
+// managed memory of the simulation's device, aligned to its elements), by a copy
+// call (anything else one takes: another device's memory, pinned host memory), or
+// not at all (its allocation ends before the array does, which a copy call
+// refuses and a kernel would overrun).
+enum class Reach { kernel, copy, none };
+
+Reach reach_of(const sbp_sim *s, const void *ptr, size_t bytes)
 {
-    if (reinterpret_cast<uintptr_t>(ptr) % s->psize) return false;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return false;
-    }
-    return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == s->device;
+    using AttributesFn = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const AttributesFn query = reinterpret_cast<AttributesFn>(driver_entry("cuPointerGetAttributes", 12000));
+    const uintptr_t at = reinterpret_cast<uintptr_t>(ptr);
+    unsigned type = 0;
+    int device = -1;
+    unsigned long long start = 0, size = 0;
+    CUpointer_attribute want[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *got[4] = {&type, &device, &start, &size};
+    if (!query || query(4, want, got, (CUdeviceptr)at) != CUDA_SUCCESS) return Reach::copy;
+    if (size && (at < start || at - start > size || bytes > size - (at - start))) return Reach::none;
+    return type == CU_MEMORYTYPE_DEVICE && device == s->device && at % s->psize == 0 ? Reach::kernel : Reach::copy;
 }
 
 }  // namespace
@@ -1729,9 +1742,11 @@ int sbp_set_field(sbp_sim *s, int comp, const void *src, int is_device)
     int e[3];
     if (!s || !src || extents_of(s, comp, e)) return SBP_EINVAL;
     DeviceGuard dg(s->device);
+    const size_t bytes = (size_t)e[0] * e[1] * e[2] * s->psize;      // of the caller's array
+    const Reach reach = is_device ? reach_of(s, src, bytes) : Reach::copy;
+    if (reach == Reach::none) return SBP_ECUDA;
     if (s->prec == SBP_FP32_FP16STORE) {
         // FP32 values in; stored as value / scale in FP16
-        const size_t bytes = (size_t)e[0] * e[1] * e[2] * sizeof(float);
         const float *d_src = static_cast<const float *>(src);
         float *tmp = nullptr;
         if (!is_device) {
@@ -1749,7 +1764,6 @@ int sbp_set_field(sbp_sim *s, int comp, const void *src, int is_device)
         // host values: one contiguous copy into the spare set's array of this
         // component (dead between steps: the next step overwrites it), then a
         // scatter into the padded layout
-        const size_t bytes = (size_t)e[0] * e[1] * e[2] * s->esize;
         void *stage = s->set[s->cur ^ 1][comp];
         SBP_CUDA(cudaMemcpyAsync(stage, src, bytes, cudaMemcpyHostToDevice, s->stream));
         const int rc = put_dense(s, comp, e, stage);
@@ -1757,7 +1771,7 @@ int sbp_set_field(sbp_sim *s, int comp, const void *src, int is_device)
         SBP_CUDA(cudaStreamSynchronize(s->stream));
         return SBP_OK;
     }
-    if (is_device && kernel_reachable(s, src)) return put_dense(s, comp, e, src);
+    if (reach == Reach::kernel) return put_dense(s, comp, e, src);
     cudaMemcpy3DParms m = {};
     m.srcPtr = make_cudaPitchedPtr(const_cast<void *>(src), e[0] * s->esize, e[0] * s->esize, e[1]);
     m.dstPtr = make_cudaPitchedPtr(s->set[s->cur][comp], s->sy * s->esize, e[0] * s->esize, s->n[1] + 2);
@@ -1773,9 +1787,11 @@ int sbp_get_field(sbp_sim *s, int comp, void *dst, int to_device)
     int e[3];
     if (!s || !dst || extents_of(s, comp, e)) return SBP_EINVAL;
     DeviceGuard dg(s->device);
+    const size_t bytes = (size_t)e[0] * e[1] * e[2] * s->psize;      // of the caller's array
+    const Reach reach = to_device ? reach_of(s, dst, bytes) : Reach::copy;
+    if (reach == Reach::none) return SBP_ECUDA;
     if (s->prec == SBP_FP32_FP16STORE) {
         // stored FP16 values times the field's scale, out as FP32
-        const size_t bytes = (size_t)e[0] * e[1] * e[2] * sizeof(float);
         float *d_dst = static_cast<float *>(dst);
         if (!to_device) SBP_CUDA(cudaMallocAsync(reinterpret_cast<void **>(&d_dst), bytes, s->stream));
         const int rc = get_dense(s, comp, e, d_dst);
@@ -1791,7 +1807,6 @@ int sbp_get_field(sbp_sim *s, int comp, void *dst, int to_device)
     if (!to_device && s->fused_ok) {
         // gather into the spare set's array (dead between steps), then one
         // contiguous copy to the host
-        const size_t bytes = (size_t)e[0] * e[1] * e[2] * s->esize;
         void *stage = s->set[s->cur ^ 1][comp];
         const int rc = get_dense(s, comp, e, stage);
         if (rc) return rc;
@@ -1799,7 +1814,7 @@ int sbp_get_field(sbp_sim *s, int comp, void *dst, int to_device)
         SBP_CUDA(cudaStreamSynchronize(s->stream));
         return check_error_flag(s);
     }
-    if (to_device && kernel_reachable(s, dst)) return get_dense(s, comp, e, dst);
+    if (reach == Reach::kernel) return get_dense(s, comp, e, dst);
     cudaMemcpy3DParms m = {};
     m.srcPtr = make_cudaPitchedPtr(s->set[s->cur][comp], s->sy * s->esize, e[0] * s->esize, s->n[1] + 2);
     m.dstPtr = make_cudaPitchedPtr(dst, e[0] * s->esize, e[0] * s->esize, e[1]);

@@ -267,12 +267,12 @@ def run_ours(args):
     nx, ny, nz = spec.n
     # Algorithmic bytes per cell-update: every field read twice (once per half-step) and
     # written once, plus the cell's eps_r: 6*3*4 + 1 = 73 B (FP32), 6*3*2 + 1 = 37 B (FP16
-    # storage).  The one-pass kernel performs whole steps of its cells; the band kernels
-    # the two half-steps of theirs.
+    # storage).  The one-pass kernel performs whole steps of its cells; the launches
+    # of its boundary half a step of theirs.
     alg = 37.0 if fp16 else 73.0
     units = {   # cells each launch updates, and algorithmic bytes per cell
         "fused_interior": ((nx - 5) * (ny - 5) * (nz - 5), alg),
-        # band kernels: nodes of the padded box outside the interior box of the one-pass step
+        # its boundary: nodes of the padded box outside the interior box of the one-pass step
         "band_h": ((nx + 2) * (ny + 2) * (nz + 2) - (nx - 6) * (ny - 6) * (nz - 6), alg / 2),
         "band_e": ((nx + 2) * (ny + 2) * (nz + 2) - (nx - 5) * (ny - 5) * (nz - 5), alg / 2),
         "h_update": (cells, alg / 2),

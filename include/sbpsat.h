@@ -206,8 +206,9 @@ int sbp_half_step_e(sbp_sim **sims, int nsims);
 /* As sbp_step for one simulation, but brackets every kernel launch with CUDA
  * events on the simulation's stream and, after synchronising, writes the
  * average device time per launch (milliseconds) of each kernel kind to
- * avg_ms[0..n_out-1] in the order: h_update, e_update, band_h,
- * fused_interior, band_e (0 for kinds that did not run), and the number of
+ * avg_ms[0..n_out-1] in the order: h_update, e_update (the in-place half-steps),
+ * band_h (the H half of a one-pass step's boundary), fused_interior, band_e (its
+ * E half) (0 for kinds that did not run), and the number of
  * launches per kind to launches[0..n_out-1] if non-NULL.  For measurement:
  * the events add a small gap between launches. */
 int sbp_step_timed(sbp_sim *s, int64_t nsteps, double *avg_ms, int64_t *launches, int n_out);

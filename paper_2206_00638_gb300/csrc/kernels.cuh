@@ -688,7 +688,7 @@ __device__ __forceinline__ double energy_h(const Params<T, S> &p, long long o, f
 // three components); the norm weights multiply as FP32, where their products
 // are exact, and FP32 values and cells widen by integer operations.  That is 15
 // FP64 operations for an interior node and about 24 at the boundary, where 78
-// were: 168 us for 160 x 144 x 128 cells, 475 before.
+// were: 165 us for 160 x 144 x 128 cells with the final sum, 475 before.
 template <typename T, typename S, bool MUVAR>
 __global__ void __launch_bounds__(kBlockX *kBlockY) energy_sum(const Params<T, S> p)
 {

@@ -10,8 +10,8 @@
 // component's natural extents (Table I) stay zero.
 //
 // Two step paths, bit-identical where both run.  Large FP32 blocks with uniform
-// mu keep two field sets and advance with three launches per step (band_h,
-// fused_interior, band_e: old set -> new set, then swap).  Everything else
+// mu keep two field sets and advance with three launches per step (fused_interior
+// and, beside it, the boundary's H and E: old set -> new set, then swap).  Everything else
 // (smaller grids, FP16 storage, FP64, varying mu, the half-step calls) uses the
 // in-place half_h / half_e pair on the current set.
 #include <cuda_runtime.h>
@@ -103,7 +103,7 @@ struct sbp_sim {
     int fused_width = sbp::kFTX;          // tile columns of the one-pass step (64 or 128)
     dim3 fused_grid;
     bool async_setup = false;             // caller keeps host inputs alive: no stream syncs in setup
-    cudaStream_t side = nullptr;          // band_h runs here, concurrently with fused_interior
+    cudaStream_t side = nullptr;          // the boundary runs here, concurrently with fused_interior
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     sbp::Band band_hb, band_eb;
     sbp::Sweep sweep[2];                  // in-place half-steps: work lists (H, E) and vector width
@@ -410,7 +410,8 @@ int encode_maps(sbp_sim *s)
     return SBP_OK;
 }
 
-// Multiplier and shift of FastDiv's n / d for n < 2^31.
+// Multiplier and shift of FastDiv's n / d for n < 2^31: division by an invariant
+// through the rounded-up reciprocal (Granlund and Montgomery, PLDI 1994).
 sbp::FastDiv fast_div(unsigned d)
 {
     unsigned l = 0;
@@ -1112,7 +1113,8 @@ int step_group(sbp_sim **sims, int nsims, int64_t nsteps)
 }
 
 // sbp_step with CUDA events around every launch (kernel kinds: 0 h_update
-// (half_h), 1 e_update (half_e), 2 band_h, 3 fused_interior, 4 band_e).
+// (half_h), 1 e_update (half_e), 2 band_h and 4 band_e (the boundary of a one-pass
+// step: rim_step, or the slab kernels of those names), 3 fused_interior).
 int step_timed(sbp_sim *s, int64_t nsteps, double *avg_ms, int64_t *launches, int n_out)
 {
     constexpr int kKinds = 5;

@@ -298,6 +298,8 @@ class Sim:
     def step(self, nsteps):
         _check(lib().sbp_step(self._h, int(nsteps)), "sbp_step")
 
+    # kinds of step_timed: the in-place half-steps; the H half of a one-pass step's boundary, the
+    # one-pass kernel, the boundary's E half
     KERNELS = ("h_update", "e_update", "band_h", "fused_interior", "band_e")
 
     def step_timed(self, nsteps):

@@ -159,3 +159,30 @@ def test_last_member_ends_one_step_before_the_chunk(n, use_graphs):
         batch.close()
         s.close()
     alone.close()
+
+
+def test_server_requests_in_one_pass(monkeypatch):
+    """Served requests that step in one pass, admitted and retired between chunks beside each other,
+    give the samples they give alone."""
+    monkeypatch.setenv("SBP_STEP_PATH", "onepass")
+    reqs = wl.serving_stream(nreq=5, seed=12, n_range=(20, 56), steps_range=(20, 70))
+    ref = []
+    for spec, steps in reqs:
+        s = sbpsat.Sim(spec.n, spec.h, spec.faces, eps_r=spec.eps_r, cfl=0.95)
+        for src in spec.sources:
+            s.add_source(src.comp, src.i, src.j, src.k, src.kind, src.amp, src.tw, src.t0, src.f)
+        for p in spec.probes:
+            s.add_probe(p.comp, p.i, p.j, p.k)
+        s.reserve_probes(steps)
+        s.step(steps)
+        ref.append(s.probes())
+        s.close()
+    srv = sbpsat.Server(stream=torch.cuda.Stream(), max_slots=3, chunk=16)
+    tickets = [srv.submit(spec, steps) for spec, steps in reqs]
+    srv.drain()
+    for t, r, (spec, steps) in zip(tickets, ref, reqs):
+        res = srv.poll(t)
+        assert res is not None and res.status == 0 and res.steps == steps
+        assert np.array_equal(srv.probes(t), r), spec.n
+        srv.release(t)
+    srv.close()

@@ -257,9 +257,9 @@ __device__ __forceinline__ void box_h(const Params<T, S> &p, const Sweep &w, Whe
                 a.add(Bz, d0); a.add(By, d1, T(-1));
                 b.add(Bx, d2); b.add(Bz, d3, T(-1));
                 c.add(By, d4); c.add(Bx, d5, T(-1));
-                hx[q] = quant<S>(add_scaled(hx[q], a, m0[q] + mi));
-                hy[q] = quant<S>(add_scaled(hy[q], b, m0[q] + mj[q]));
-                hz[q] = quant<S>(add_scaled(hz[q], c, m0[q] + mk[q]));
+                hx[q] = quant<S>(hx[q] + scaled_increment(a, m0[q] + mi));
+                hy[q] = quant<S>(hy[q] + scaled_increment(b, m0[q] + mj[q]));
+                hz[q] = quant<S>(hz[q] + scaled_increment(c, m0[q] + mk[q]));
             } else {
                 hx[q] = quant<S>(advance_plain<S>(hx[q], Bz, d0, By, d1));
                 hy[q] = quant<S>(advance_plain<S>(hy[q], Bx, d2, Bz, d3));
@@ -362,9 +362,9 @@ __device__ __forceinline__ void box_e(const Params<T, S> &p, const Sweep &w, Whe
         if (marks.J) vec_sources<V>(p, marks.J, r.i0, r.j, k, a, b, c);
 #pragma unroll
         for (int q = 0; q < V; ++q) {
-            ex[q] = quant<S>(add_scaled(ex[q], a[q], qa[q] + na[q]));
-            ey[q] = quant<S>(add_scaled(ey[q], b[q], qb[q] + nb[q]));
-            ez[q] = quant<S>(add_scaled(ez[q], c[q], qb[q] + qc[q]));
+            ex[q] = quant<S>(ex[q] + scaled_increment(a[q], qa[q] + na[q]));
+            ey[q] = quant<S>(ey[q] + scaled_increment(b[q], qb[q] + nb[q]));
+            ez[q] = quant<S>(ez[q] + scaled_increment(c[q], qb[q] + qc[q]));
         }
         stv<V>(Ex + o, ex);
         stv<V>(Ey + o, ey);

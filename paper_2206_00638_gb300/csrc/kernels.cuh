@@ -172,22 +172,13 @@ __device__ __forceinline__ bool recip_seed(double s, double &r)
     return (unsigned)(hi - (923 << 20)) < (unsigned)(200 << 20);
 }
 
-// 1/s for a positive s: the seed r and the geometric series in its residue
-// d = 1 - s r, r (1 + d + d^2), which leaves d^3 < 2^-63 beside the rounding of
-// the last operation.  Three FP64 operations; a division takes about ten, at 2
-// lanes per clock and SM.
-__device__ __noinline__ double recip64_any(double s) { return 1.0 / s; }
-__device__ __forceinline__ double recip64(double s)
-{
-    double r;
-    if (!recip_seed(s, r)) return recip64_any(s);
-    const double d = fma(-s, r, 1.0);
-    return fma(r, fma(d, d, d), r);
-}
-
 // a/s for a positive s: a times a reciprocal good to 2^-42, corrected by the
 // remainder of that quotient (Markstein, IBM J. Res. Dev. 34, 1990), which leaves
-// one rounding as a division does.  Five FP64 operations.
+// one rounding as a division does.  Five FP64 operations; a division takes about
+// ten, at 2 lanes per clock and SM.  (A rounded reciprocal, multiplied inside the
+// sum with the old value, takes two fewer: 96 x 75 x 88 at 1474 instead of 1599 us
+// per 16 steps, and an error 10 % above the quotient's, since a node's reciprocal
+// is off the same way at every step.)
 __device__ __noinline__ double quot64_any(double a, double s) { return a / s; }
 __device__ __forceinline__ double quot64(double a, double s)
 {
@@ -230,15 +221,6 @@ __device__ __forceinline__ float scaled_increment(const AccLite &a, float s)
     return fmaf(rh, a.hi, rl * a.hi);
 }
 __device__ __forceinline__ float plain_increment(const AccLite &a) { return a.hi; }
-
-// old + acc / s (interior nodes).  FP64 multiplies by the reciprocal inside the
-// sum: its rounding and the sum's, as a quotient and a sum have.
-template <typename A>
-__device__ __forceinline__ float add_scaled(float old, const A &a, float s) { return old + scaled_increment(a, s); }
-__device__ __forceinline__ double add_scaled(double old, const Acc<double> &a, double s)
-{
-    return fma(a.hi, recip64(s), old);
-}
 
 // The accumulator of arithmetic type T for fields stored as S.
 template <typename T, typename S> struct AccOf { using type = Acc<T>; };

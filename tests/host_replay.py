@@ -246,7 +246,8 @@ def _device(name):
     text = re.sub(r"^#(include|pragma once).*$", "", text, flags=re.M)
     text = text.replace("extern __shared__", "extern")
     text = re.sub(r'asm\s+volatile\("griddepcontrol\.wait;".*?\);', "pdl_wait_hook();", text, flags=re.S)
-    text = re.sub(r'asm\("rcp\.approx\.ftz\.f32 %0, %1;" : "=f"\(r\) : "f"\((\w+)\)\);', r"r = 1.0f / \1;", text)
+    text = re.sub(r'asm\("rcp\.approx\.ftz\.f32 %0, %1;" : "=f"\((\w+)\) : "f"\((\w+)\)\);', r"\1 = 1.0f / \2;", text)
+    assert "rcp.approx" not in text
     text = re.sub(r"asm\s*(volatile)?\s*\((?:[^()\"]|\"(?:[^\"\\]|\\.)*\"|\((?:[^()\"]|\([^()]*\))*\))*\)\s*;", ";", text)
     assert not re.search(r"\basm\b", re.sub(r"//.*", "", text))
     return text

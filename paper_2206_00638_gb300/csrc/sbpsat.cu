@@ -1669,7 +1669,13 @@ Reach reach_of(const sbp_sim *s, const void *ptr, size_t bytes)
     CUpointer_attribute want[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
                                    CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
     void *got[4] = {&type, &device, &start, &size};
-    if (!query || query(4, want, got, (CUdeviceptr)at) != CUDA_SUCCESS) return Reach::copy;
+    if (!query) return Reach::copy;
+    if (query(4, want, got, (CUdeviceptr)at) != CUDA_SUCCESS) {
+        // a thread's first CUDA call: the runtime's query makes the device's context current
+        cudaPointerAttributes unused;
+        if (cudaPointerGetAttributes(&unused, ptr) != cudaSuccess) (void)cudaGetLastError();
+        if (query(4, want, got, (CUdeviceptr)at) != CUDA_SUCCESS) return Reach::copy;
+    }
     if (size && (at < start || at - start > size || bytes > size - (at - start))) return Reach::none;
     return type == CU_MEMORYTYPE_DEVICE && device == s->device && at % s->psize == 0 ? Reach::kernel : Reach::copy;
 }

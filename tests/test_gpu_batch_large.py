@@ -30,6 +30,7 @@ def _driven(n, at, probes):
     out = s.probes()
     batch.close()
     s.close()
+    torch.cuda.empty_cache()            # the workspace leaves the allocator's pool
     return out
 
 

@@ -263,7 +263,8 @@ typedef struct sbp_batch sbp_batch;
 /* flags: SBP_BATCH_GRAPHS records each chunk (sbp_batch_step call) as a CUDA
  * graph and replays it, updated in place when the membership changes (members
  * that step in one pass stay outside it, launched with the host's step index as
- * sbp_step launches them).  By default a chunk advances each group
+ * sbp_step launches them; a chunk of many launches is replayed in equal pieces).
+ * By default a chunk advances each group
  * of members with two launches per step (the H and the E half-step, in place).
  * SBP_BATCH_PERSISTENT runs the whole chunk as one
  * persistent launch instead: CTAs that stay resident take (step, work item)

@@ -162,6 +162,31 @@ def test_last_member_ends_one_step_before_the_chunk(n, use_graphs):
     alone.close()
 
 
+@pytest.mark.parametrize("steps", [6001, 9000])
+def test_long_chunk_in_pieces(steps):
+    """One call for thousands of steps keeps its graph small (a whole one of 9000 steps of three launches'
+    worth of members would hold some 100 MB on the device) and gives the bits of the same steps alone."""
+    works = [wl.random_box(n, faces=(A, P, M, A, P, A), seed=80 + q, steps=steps - 700 * q)
+             for q, n in enumerate([(8, 9, 8), (14, 11, 12), (101, 100, 20)])]
+    sims = [sbpsat.from_workload(w)[0] for w in works]
+    batch = sbpsat.Batch()
+    for s, w in zip(sims, works):
+        batch.add(s, w.steps)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    batch.step(steps)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20
+    for s, w in zip(sims, works):
+        assert s.step_index == w.steps
+        alone = sbpsat.from_workload(w)[0]
+        alone.step(w.steps)
+        for c in range(6):
+            assert np.array_equal(s.field(c), alone.field(c)), c
+        alone.close()
+    batch.close()
+
+
 def test_server_requests_in_one_pass(monkeypatch):
     """Served requests that step in one pass, admitted and retired between chunks beside each other,
     give the samples they give alone."""

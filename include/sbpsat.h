@@ -286,7 +286,8 @@ int sbp_batch_remove(sbp_batch *b, sbp_sim *s);
 /* Steps s still has to take in this batch. */
 int sbp_batch_remaining(const sbp_batch *b, const sbp_sim *s, int64_t *remaining);
 /* Advance every member by min(nsteps, its remaining steps), asynchronously
- * on the batch's stream. */
+ * on the batch's stream.  SBP_ESTATE if a member has been connected to a block
+ * since it was added. */
 int sbp_batch_step(sbp_batch *b, int64_t nsteps);
 int sbp_batch_size(const sbp_batch *b);
 int sbp_batch_destroy(sbp_batch *b);

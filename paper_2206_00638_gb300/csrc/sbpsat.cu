@@ -918,6 +918,12 @@ int launch_fused_phase1(sbp_sim *s, bool chain_e)
 // Fused path, phase 2 (blocks joined to another block): band E on the main stream.
 int launch_fused_phase2(sbp_sim *s) { return launch_band_e(s, s->stream); }
 
+// True when s has an interface face.
+bool joined(const sbp_sim *s)
+{
+    return std::any_of(s->face, s->face + 6, [](int f) { return f == SBP_INTERFACE; });
+}
+
 // True when an interface face of s joins it to a block other than itself.
 bool linked_to_other(const sbp_sim *s)
 {
@@ -2194,8 +2200,7 @@ int sbp_batch_add(sbp_batch *b, sbp_sim *s, int64_t nsteps)
     if (!b || !s || nsteps < 0) return SBP_EINVAL;
     if (!s->fused_ok || s->prec != SBP_FP32 || s->fdtd || s->stream != b->stream || s->device != b->device)
         return SBP_EINVAL;
-    for (int f = 0; f < 6; f++)
-        if (s->face[f] == SBP_INTERFACE) return SBP_EINVAL;
+    if (joined(s)) return SBP_EINVAL;
     for (auto &m : b->m)
         if (m.s == s) return SBP_ESTATE;
     DeviceGuard dg(b->device);
@@ -2241,6 +2246,8 @@ int sbp_batch_step(sbp_batch *b, int64_t nsteps)
     // behind every chunk)
     if (*static_cast<volatile int *>(b->h_err)) return SBP_ETIMEOUT;
     if (b->m.empty() || nsteps == 0) return SBP_OK;
+    for (const auto &m : b->m)
+        if (joined(m.s)) return SBP_ESTATE;            // connected after it was added
     int rc = SBP_OK;
     if (b->dirty && (rc = batch_rebuild(b))) return rc;
     // a long chunk is replayed as equal pieces, and the few steps that they leave launched

@@ -162,6 +162,29 @@ def test_last_member_ends_one_step_before_the_chunk(n, use_graphs):
     alone.close()
 
 
+@pytest.mark.parametrize("persistent", [False, True])
+def test_members_connected_after_joining_are_refused(persistent):
+    """A batch steps single blocks: connecting members to each other, before or after its first chunk,
+    is refused at the next one (on the host), and the members go on as a group."""
+    for early in (True, False):
+        w = wl.random_box((20, 17, 23), seed=6)
+        sims = [sbpsat.from_workload(w)[0] for _ in range(2)]
+        batch = sbpsat.Batch(persistent=persistent)
+        for s in sims:
+            batch.add(s, 20)
+        if not early:
+            batch.step(2)
+        sims[0].connect(5, sims[1], 4)
+        with pytest.raises(sbpsat.SbpError) as err:
+            batch.step(2)
+        assert err.value.code == -7
+        for s in sims:
+            batch.remove(s)
+        sbpsat.step_group(sims, 2)
+        assert [s.step_index for s in sims] == ([2, 2] if early else [4, 4])
+        batch.close()
+
+
 @pytest.mark.parametrize("steps", [6001, 9000])
 def test_long_chunk_in_pieces(steps):
     """One call for thousands of steps keeps its graph small (a whole one of 9000 steps of three launches'

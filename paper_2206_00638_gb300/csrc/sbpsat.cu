@@ -1304,10 +1304,18 @@ int autotune(sbp_sim *s, int trials, int *chosen, double *best_ms)
 // A batch: many single-block FP32 simulations advanced together (half_batched in
 // halfstep.cuh, or one persistent launch per chunk, fused.cuh).
 struct sbp_batch {
+    // What the batch's tables hold of a member that other calls can change: probe
+    // buffer (address, capacity, first step), step, sources, probes, current set.
+    using State = std::tuple<const void *, long long, long long, long long, size_t, size_t, int>;
+    static State state_of(const sbp_sim *s)
+    {
+        return {s->probe_buf, s->probe_cap, s->probe_base, s->step, s->src.size(), s->prb.size(), s->cur};
+    }
     struct Member {
         sbp_sim *s;
         long long target;        // absolute step index at which the member stops
         double *mirror;          // pinned host copy of the latest energy sample (serving), or null
+        State seen;              // after the batch's last chunk
     };
     struct Group {                      // members that run a chunk together
         int first, n, v;                // v: vector width of a member that runs by itself
@@ -2209,7 +2217,7 @@ int sbp_batch_add(sbp_batch *b, sbp_sim *s, int64_t nsteps)
         int rc = ensure_series(s, (s->step + nsteps) / s->energy_every + 1);
         if (rc) return rc;
     }
-    b->m.push_back({s, s->step + nsteps, nullptr});
+    b->m.push_back({s, s->step + nsteps, nullptr, {}});
     b->dirty = true;
     return batch_sample_energy(b, b->m.back());
 }
@@ -2246,8 +2254,10 @@ int sbp_batch_step(sbp_batch *b, int64_t nsteps)
     // behind every chunk)
     if (*static_cast<volatile int *>(b->h_err)) return SBP_ETIMEOUT;
     if (b->m.empty() || nsteps == 0) return SBP_OK;
-    for (const auto &m : b->m)
+    for (const auto &m : b->m) {
         if (joined(m.s)) return SBP_ESTATE;            // connected after it was added
+        if (m.seen != sbp_batch::state_of(m.s)) b->dirty = true;
+    }
     int rc = SBP_OK;
     if (b->dirty && (rc = batch_rebuild(b))) return rc;
     // a long chunk is replayed as equal pieces, and the few steps that they leave launched
@@ -2314,6 +2324,7 @@ int sbp_batch_step(sbp_batch *b, int64_t nsteps)
             m.s->step += done;
             if (b->persistent) m.s->cur ^= (int)(done & 1);
         }
+        m.seen = sbp_batch::state_of(m.s);
         if (done > 0 && (rc = batch_sample_energy(b, m))) return rc;
     }
     return SBP_OK;

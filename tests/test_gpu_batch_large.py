@@ -162,6 +162,43 @@ def test_last_member_ends_one_step_before_the_chunk(n, use_graphs):
     alone.close()
 
 
+@pytest.mark.parametrize("use_graphs, persistent", [(True, False), (False, False), (True, True)])
+def test_members_changed_between_chunks(use_graphs, persistent):
+    """A member stepped by itself, given new sources and a new probe buffer, or restored from a checkpoint
+    between chunks goes on from that state."""
+    def change(s, k):
+        if k == 0:
+            s.step(3)
+        elif k == 1:
+            s.reserve_probes(50)
+            s.add_source(sbpsat.EX, 5, 6, 7, sbpsat.GAUSS, 50.0, 4e-12, s.dt * s.step_index)
+        elif k == 2:
+            s.load(s.saved)
+
+    works = [wl.random_box(n, faces=(A, P, M, A, P, M), seed=90 + q) for q, n in enumerate([(20, 17, 23), (40, 33, 29)])]
+    batch, sims, refs = sbpsat.Batch(use_graphs=use_graphs, persistent=persistent), [], []
+    for w in works:
+        for group in (sims, refs):
+            group.append(sbpsat.from_workload(w)[0])
+            group[-1].reserve_probes(30)
+        batch.add(sims[-1], 1000)
+    for k in range(4):
+        batch.step(5)
+        for s in refs:
+            s.step(5)
+        if k == 1:
+            for s in sims + refs:
+                s.saved = s.save()
+        for s in (sims[1], refs[1]):
+            change(s, k)
+    for s, r in zip(sims, refs):
+        assert s.step_index == r.step_index
+        for c in range(6):
+            assert np.array_equal(s.field(c), r.field(c)), c
+        assert np.array_equal(s.probes(), r.probes())
+    batch.close()
+
+
 @pytest.mark.parametrize("persistent", [False, True])
 def test_members_connected_after_joining_are_refused(persistent):
     """A batch steps single blocks: connecting members to each other, before or after its first chunk,
